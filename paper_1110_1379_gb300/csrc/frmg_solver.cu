@@ -31,6 +31,7 @@
 #include "frmg.h"
 #include "frmg_internal.h"
 #include "frmg_kernels.cuh"
+#include "frmg_tail.cuh"
 #include "frmg_df.cuh"
 
 using namespace frmg;
@@ -734,12 +735,43 @@ static void upload_set(Scope &S, LevelSet<T> &ls, cudaStream_t st, int tiling = 
   CK(cudaStreamSynchronize(st));
 }
 
+// Tails (k_tail) of the problems whose one-cluster part of the V-cycle begins
+// at one depth: their levels from that depth to the coarsest.
+template <typename T>
+struct TailSet {
+  std::vector<TailDesc<T>> h[2];    // shared-memory layout of the [0] plain, [1] correction form
+  TailDesc<T> *d[2] = {nullptr, nullptr};
+  std::vector<long long> ncell;     // cells of each problem's top level
+  int cs = 1;                       // blocks per cluster
+  size_t smem[2] = {0, 0};          // per block
+  double *norms = nullptr;          // per problem (sum of squares, max): depth 0
+  int size() const { return (int)h[0].size(); }
+  bool empty() const { return h[0].empty(); }
+};
+
+// Lays out the tail of levels lev[l ..] on clusters of cs blocks; returns the
+// shared memory per block.
+template <typename T>
+static size_t tail_desc(const std::vector<Grid<T>> &lev, int l, int cs, bool bg, TailDesc<T> &d) {
+  memset(&d, 0, sizeof(d));
+  d.nl = (int)lev.size() - l;
+  d.field = lev[l].field;
+  d.beta = lev[l].beta;
+  d.cap = lev[l].cap;
+  d.relax = lev[l].relax;
+  unsigned end = 0;
+  for (int q = 0; q < d.nl; q++) end = tail_layout(d.lev[q], lev[l + q], cs, bg, q == 0, end);
+  return (size_t)end * sizeof(T);
+}
+
 // Level hierarchy of a batch of problems in precision T.  BG: background mode
 // (the FP32 inner solve of the mixed loop).
 template <typename T>
 struct Hier {
   int depth = 0;
   std::vector<std::vector<Grid<T>>> lev;  // lev[p][l]
+  std::vector<int> tail_at;               // per problem: depth its tail begins at (nl: none)
+  std::vector<TailSet<T>> tail;           // by depth
   std::vector<LevelSet<T>> cont, next, coarsest, all;
   std::vector<float *> bg_u, bg_E;        // fine-level background arrays per problem
   std::vector<int> par;                   // current u buffer (0/1) per depth
@@ -747,10 +779,103 @@ struct Hier {
   T *cur_x(int pi, int l) const { return par[l] ? lev[pi][l].x2 : lev[pi][l].x; }
 };
 
+// Most blocks per cluster that a tail may use with `smem` bytes each.
+template <typename T, bool BG, bool DIR>
+static int tail_cluster(size_t smem) {
+  static int best = 0;
+  if (!best) {
+    auto *k = k_tail<T, BG, DIR>;
+    CK(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    for (int cs = kTailCluster; cs > 0 && !best; cs /= 2) {
+      cudaLaunchConfig_t c = {};
+      c.gridDim = dim3(cs);
+      c.blockDim = dim3(tail_threads<T>());
+      c.dynamicSmemBytes = smem;
+      cudaLaunchAttribute a[1];
+      a[0].id = cudaLaunchAttributeClusterDimension;
+      a[0].val.clusterDim.x = cs;
+      a[0].val.clusterDim.y = a[0].val.clusterDim.z = 1;
+      c.attrs = a;
+      c.numAttrs = 1;
+      int n = 0;
+      if (cudaOccupancyMaxActiveClusters(&n, k, &c) == cudaSuccess && n > 0) best = cs;
+      else cudaGetLastError();
+    }
+    if (!best) best = 1;
+  }
+  return best;
+}
+
+// Shared memory a tail's block may use (227 KB per block less the static part).
+constexpr size_t kTailSmem = 222 * 1024;
+
+// Chooses the depth at which each problem's tail begins (none above depth
+// tail_min; tail_min < 0: no tails) and uploads the tails' levels.
+template <typename T>
+static void plan_tails(Scope &S, Hier<T> &H, int tail_min, cudaStream_t st) {
+  const int np = (int)H.lev.size();
+  H.tail_at.resize(np);
+  H.tail.assign(H.depth, {});
+  for (int pi = 0; pi < np; pi++) H.tail_at[pi] = (int)H.lev[pi].size();
+  if (tail_min < 0) return;
+  // (a set holds periodic grids or patches, never both)
+  const bool dir = H.lev[0][0].bnd != nullptr;
+  int most = dir ? tail_cluster<T, false, true>(kTailSmem) : tail_cluster<T, false, false>(kTailSmem);
+  if constexpr (sizeof(T) == 4)
+    most = std::min(most, dir ? tail_cluster<T, true, true>(kTailSmem)
+                              : tail_cluster<T, true, false>(kTailSmem));
+  // Blocks per cluster and the largest top level.  Measured (us per V-cycle
+  // tail; time of the solve): one 64^3 field, FP32: top level 32^3 on 16 blocks
+  // 53 us, 1.86 ms; on 8 blocks 64 us, 1.98 ms; top level 16^3 2.28 ms.  48 fields
+  // of 32 to 128 cells: top levels up to 32^3 on 8 blocks 39.0 ms, on 16 blocks
+  // 39.9, up to 16^3 40.9.  FP64, one 32^3 field: top level 16^3 3.16 ms, 8^3
+  // 4.2 ms, 32^3 4.3 ms (the FP64 pipes of 16 SMs are then the bound).  What
+  // shared memory holds bounds FP32 tops at about 40^3 on 16 blocks.
+  const int csz = std::min(most, np <= 8 ? 16 : 8);
+  const long long cap = sizeof(T) == 8 ? 4096 : (np <= 8 ? 110592 : 32768);
+  TailDesc<T> td;
+  for (int pi = 0; pi < np; pi++) {
+    const auto &lev = H.lev[pi];
+    const int nl = (int)lev.size();
+    int at = nl;
+    for (int l = nl - 1; l >= tail_min; l--) {
+      if (nl - l > kTailLev || lev[l].ncell > cap ||
+          tail_desc(lev, l, csz, sizeof(T) == 4, td) > kTailSmem)
+        break;
+      at = l;
+    }
+    H.tail_at[pi] = at;
+    if (at < nl && lev[at].ncell > tail_local<T>()) H.tail[at].cs = csz;
+  }
+  for (int pi = 0; pi < np; pi++) {
+    const auto &lev = H.lev[pi];
+    const int at = H.tail_at[pi];
+    if (at == (int)lev.size()) continue;
+    TailSet<T> &t = H.tail[at];
+    for (int bg = 0; bg < (sizeof(T) == 4 ? 2 : 1); bg++) {
+      t.smem[bg] = std::max(t.smem[bg], tail_desc(lev, at, t.cs, bg != 0, td));
+      t.h[bg].push_back(td);
+    }
+    t.ncell.push_back(lev[at].ncell);
+  }
+  for (auto &t : H.tail) {
+    if (t.empty()) continue;
+    for (int bg = 0; bg < 2; bg++) {
+      if (t.h[bg].empty()) continue;
+      const size_t bytes = t.h[bg].size() * sizeof(TailDesc<T>);
+      t.d[bg] = S.get<TailDesc<T>>(t.h[bg].size());
+      CK(cudaMemcpyAsync(t.d[bg], t.h[bg].data(), bytes, cudaMemcpyHostToDevice, st));
+    }
+    t.norms = S.get<double>(2 * (size_t)t.size());
+  }
+  CK(cudaStreamSynchronize(st));  // the host vectors have been read
+}
+
 template <typename T, bool BG>
 static void build_hier(Scope &S, Hier<T> &H, std::vector<Problem> &P, double cap,
                        cudaStream_t st, frmg_ctx *ctx, int tiling = 0, double relax = 1.0,
-                       int stile = 0) {
+                       int stile = 0, int tail_min = -1, bool all_levels = false) {
   int np = (int)P.size();
   H.lev.assign(np, {});
   H.depth = 0;
@@ -833,10 +958,12 @@ static void build_hier(Scope &S, Hier<T> &H, std::vector<Problem> &P, double cap
   H.next.assign(H.depth, {});
   H.coarsest.assign(H.depth, {});
   H.all.assign(H.depth, {});
+  plan_tails(S, H, tail_min, st);
   for (int pi = 0; pi < np; pi++) {
     int nl = P[pi].nl;
     for (int l = 0; l < nl; l++) {
-      H.all[l].h.push_back(H.lev[pi][l]);
+      if (l == 0) H.all[l].h.push_back(H.lev[pi][l]);
+      if (!all_levels && l >= H.tail_at[pi]) continue;  // in the tail
       if (l < nl - 1) {
         H.cont[l].h.push_back(H.lev[pi][l]);
         H.next[l].h.push_back(H.lev[pi][l + 1]);
@@ -1152,9 +1279,90 @@ static void prolong_level(frmg_ctx *ctx, Hier<T> &H, int l, const int *active, c
   CK_LAUNCH(ctx);
 }
 
+// f^H = A^H(R u^h) - R d^h on every grid of a coarse set.
+template <typename T, bool BG>
+static void fas_rhs(frmg_ctx *ctx, LevelSet<T> &C, int par, const int *active, cudaStream_t st) {
+  if (C.empty()) return;
+  PROF(pname("fas_rhs", sizeof(T) == 8, false));
+  bool done = false;
+  if constexpr (sizeof(T) == 4) {
+    if (C.tiled && C.nblk_fr[BG ? 1 : 0] > 0) {
+      if (C.dirichlet)
+        launch_fas_rhs_tiled<BG, true>(ctx, C, active, par, st);
+      else
+        launch_fas_rhs_tiled<BG, false>(ctx, C, active, par, st);
+      done = true;
+    }
+  }
+  if (!done)
+    k_fas_rhs<T, BG><<<C.nblk_full, 256, 0, st>>>(C.d, C.d_off_full, C.size(), active, par);
+  CK_LAUNCH(ctx);
+}
+
+// The tails of a set, from level `skip` of each on, in one launch.
+template <typename T, bool BG, bool DIR>
+static void launch_tail_k(frmg_ctx *ctx, TailSet<T> &t, int skip, int pin, int pout, bool fas,
+                        bool finest, const CycleOpts &o, const int *active, cudaStream_t st) {
+  auto *k = k_tail<T, BG, DIR>;
+  static bool attr_set = false;
+  if (!attr_set) {
+    CK(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem));
+    attr_set = true;
+  }
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3((unsigned)(t.size() * t.cs));
+  c.blockDim = dim3(tail_threads<T>());
+  c.dynamicSmemBytes = t.smem[BG ? 1 : 0];
+  c.stream = st;
+  cudaLaunchAttribute a[1];
+  a[0].id = cudaLaunchAttributeClusterDimension;
+  a[0].val.clusterDim.x = t.cs;
+  a[0].val.clusterDim.y = a[0].val.clusterDim.z = 1;
+  c.attrs = a;
+  c.numAttrs = 1;
+  const TailOpts to{o.pre, o.post, fas ? 1 : 0, finest ? 1 : 0, o.crs_rel, o.crs_abs,
+                    o.crs_maxit, o.crs_stall, o.crs_meanfix};
+  PROF(sizeof(T) == 8 ? "tail_f64" : (BG ? "tail_bg_f32" : "tail_f32"));
+  CK(cudaLaunchKernelEx(&c, k, (const TailDesc<T> *)t.d[BG ? 1 : 0], skip, pin, pout, to, active,
+                        finest && sizeof(T) == 4 ? t.norms : (double *)nullptr));
+  CK_LAUNCH(ctx);
+}
+
+template <typename T, bool BG>
+static void launch_tail(frmg_ctx *ctx, TailSet<T> &t, int skip, int pin, int pout, bool fas,
+                        bool finest, const CycleOpts &o, const int *active, cudaStream_t st) {
+  if (t.h[0][0].lev[0].bnd)
+    launch_tail_k<T, BG, true>(ctx, t, skip, pin, pout, fas, finest, o, active, st);
+  else
+    launch_tail_k<T, BG, false>(ctx, t, skip, pin, pout, fas, finest, o, active, st);
+}
+
+// entry: the cycle begins at level l (its right-hand side is complete);
+// otherwise f of level l holds R d.
+template <typename T, bool BG>
+static void vcycle_launched(frmg_ctx *ctx, Hier<T> &H, int l, const CycleOpts &o,
+                            const int *active, cudaStream_t st);
 template <typename T, bool BG>
 static void vcycle(frmg_ctx *ctx, Hier<T> &H, int l, const CycleOpts &o, const int *active,
-                   cudaStream_t st) {
+                   cudaStream_t st, bool entry = true) {
+  if (H.lev.size() == 1 && l >= H.tail_at[0]) {
+    const int at = H.tail_at[0];
+    launch_tail<T, BG>(ctx, H.tail[at], l - at, H.par[l], H.par[l], !entry, l == 0, o, active, st);
+    return;
+  }
+  const int p0 = H.par[l];
+  vcycle_launched<T, BG>(ctx, H, l, o, active, st);
+  // after the launched levels: the depth's buffer parity may have changed, and
+  // the tails' data moves with it
+  if (!H.tail[l].empty())
+    launch_tail<T, BG>(ctx, H.tail[l], 0, p0, H.par[l], !entry, l == 0, o, active, st);
+}
+
+// The V-cycle of the problems whose level l is not in a tail.
+template <typename T, bool BG>
+static void vcycle_launched(frmg_ctx *ctx, Hier<T> &H, int l, const CycleOpts &o,
+                            const int *active, cudaStream_t st) {
   if (!H.coarsest[l].empty()) {
     auto &c = H.coarsest[l];
     PROF(sizeof(T) == 8 ? "coarsest_f64" : "coarsest_f32");
@@ -1188,24 +1396,14 @@ static void vcycle(frmg_ctx *ctx, Hier<T> &H, int l, const CycleOpts &o, const i
     }
     CK_LAUNCH(ctx);
   }
-  {
-    PROF(pname("fas_rhs", sizeof(T) == 8, false));
-    bool done = false;
-    if constexpr (sizeof(T) == 4) {
-      if (C.tiled && C.nblk_fr[BG ? 1 : 0] > 0) {
-        if (C.dirichlet)
-          launch_fas_rhs_tiled<BG, true>(ctx, C, active, H.par[l + 1], st);
-        else
-          launch_fas_rhs_tiled<BG, false>(ctx, C, active, H.par[l + 1], st);
-        done = true;
-      }
-    }
-    if (!done)
-      k_fas_rhs<T, BG><<<C.nblk_full, 256, 0, st>>>(C.d, C.d_off_full, C.size(), active,
-                                                    H.par[l + 1]);
-    CK_LAUNCH(ctx);
+  // FAS right-hand sides of the coarser level (a tail forms its own)
+  if (H.tail[l + 1].empty()) {
+    fas_rhs<T, BG>(ctx, C, H.par[l + 1], active, st);
+  } else if (H.lev.size() > 1) {
+    fas_rhs<T, BG>(ctx, H.cont[l + 1], H.par[l + 1], active, st);
+    fas_rhs<T, BG>(ctx, H.coarsest[l + 1], H.par[l + 1], active, st);
   }
-  vcycle<T, BG>(ctx, H, l + 1, o, active, st);
+  vcycle<T, BG>(ctx, H, l + 1, o, active, st, false);
   if constexpr (sizeof(T) == 4 && !BG) {
     if (can_fuse_prolong<BG>(F, tiled_ok ? &plan_post : nullptr)) {
       // prolongation fused into the first post-smoothing sweep (reported as
@@ -1391,18 +1589,28 @@ static void fused_fine_norms(frmg_ctx *ctx, Hier<T> &H, int np, cudaStream_t st,
                              std::vector<double> &out) {
   out.assign(np, std::nan(""));
   LevelSet<T> &C = H.next[0];
-  if (C.empty()) return;
-  int ng = C.size();
-  const int *offs = H.cont[0].rr_tiled ? H.cont[0].d_off_rr : C.d_off_full;
-  k_reduce_partials<<<ng, 256, 0, st>>>(C.partial, offs, ng, C.red);
-  CK_LAUNCH(ctx);
-  double *hp = pinned_buf(ctx, 2 * (size_t)ng);
-  CK(cudaMemcpyAsync(hp, C.red, 2 * ng * sizeof(double), cudaMemcpyDeviceToHost, st));
+  TailSet<T> &Q = H.tail[0];
+  const int ng = C.empty() ? 0 : C.size(), nt = Q.size();
+  if (ng + nt == 0) return;
+  double *hp = pinned_buf(ctx, 2 * (size_t)(ng + nt));
+  if (ng) {
+    const int *offs = H.cont[0].rr_tiled ? H.cont[0].d_off_rr : C.d_off_full;
+    k_reduce_partials<<<ng, 256, 0, st>>>(C.partial, offs, ng, C.red);
+    CK_LAUNCH(ctx);
+    CK(cudaMemcpyAsync(hp, C.red, 2 * ng * sizeof(double), cudaMemcpyDeviceToHost, st));
+  }
+  if (nt)
+    CK(cudaMemcpyAsync(hp + 2 * ng, Q.norms, 2 * nt * sizeof(double), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   prof_harvest(ctx);
   for (int g = 0; g < ng; g++) {
     const Grid<T> &F = H.cont[0].h[g];
     out[F.field] = std::sqrt(hp[2 * g] / (double)F.ncell);
+  }
+  for (int t = 0; t < nt; t++) {
+    const TailDesc<T> &D = Q.h[0][t];
+    if (D.nl > 1)  // one level: no residual is formed
+      out[D.field] = std::sqrt(hp[2 * (ng + t)] / (double)Q.ncell[t]);
   }
 }
 
@@ -1464,7 +1672,8 @@ static void solve_fp64(frmg_ctx *ctx, std::vector<Problem> &P, const SolveCfg &c
   Scope S(ctx);
   int np = (int)P.size();
   Hier<double> H;
-  build_hier<double, false>(S, H, P, cfg.cap, st, ctx, 0, cfg.relax);
+  build_hier<double, false>(S, H, P, cfg.cap, st, ctx, 0, cfg.relax, 0,
+                            cfg.tau_alpha > 0 ? 1 : 0);
   for (int pi = 0; pi < np; pi++) {
     Grid<double> &G = H.lev[pi][0];
     k_expm1<double><<<nblocks(G.ncell), 256, 0, st>>>(G.u, G.x, G.ncell);
@@ -1533,7 +1742,8 @@ static void solve_mixed(frmg_ctx *ctx, std::vector<Problem> &P, const SolveCfg &
   for (auto &p : P1) p.nl = 1;
   build_hier<double, false>(S, H64, P1, cfg.cap, st, ctx);
   Hier<float> H;
-  build_hier<float, true>(S, H, P, cfg.cap, st, ctx, cfg.tiling, cfg.relax, cfg.stile);
+  build_hier<float, true>(S, H, P, cfg.cap, st, ctx, cfg.tiling, cfg.relax, cfg.stile,
+                          cfg.tau_alpha > 0 ? 1 : 0, cfg.fmg && np == 1);
   std::vector<double *> d64(np);
   int *flag = S.get<int>(1);
   CK(cudaMemsetAsync(flag, 0, sizeof(int), st));
@@ -1717,7 +1927,7 @@ static void solve_mixed(frmg_ctx *ctx, std::vector<Problem> &P, const SolveCfg &
                                                        H.cur_x(pi, 0), G.ncell);
         CK_LAUNCH(ctx);
       }
-      for (size_t l = 1; l < H.lev[pi].size(); l++) {
+      for (int l = 1; l < (int)H.lev[pi].size() && l <= H.tail_at[pi]; l++) {
         Grid<float> &F = H.lev[pi][l - 1];
         Grid<float> &C = H.lev[pi][l];
         k_restrict_avg<float><<<nblocks(C.ncell), 256, 0, st>>>(F.ubg, F.n0, F.n1, F.n2,
@@ -1824,7 +2034,8 @@ static void solve_mixed_df(frmg_ctx *ctx, std::vector<Problem> &P, const SolveCf
   Scope S(ctx);
   const int np = (int)P.size();
   Hier<float> H;
-  build_hier<float, true>(S, H, P, cfg.cap, st, ctx, cfg.tiling, cfg.relax, cfg.stile);
+  build_hier<float, true>(S, H, P, cfg.cap, st, ctx, cfg.tiling, cfg.relax, cfg.stile,
+                          cfg.tau_alpha > 0 ? 1 : 0, cfg.fmg && np == 1);
   const double ln2 = std::log(2.0);
   float ln2h, ln2l;
   split_host(ln2, ln2h, ln2l);
@@ -2096,7 +2307,7 @@ static void solve_mixed_df(frmg_ctx *ctx, std::vector<Problem> &P, const SolveCf
       for (int pi = 0; pi < np; pi++) {
         if (!act[pi]) continue;
         r0[pi] = nr[2 * pi];
-        for (size_t l = 1; l < H.lev[pi].size(); l++) {
+        for (int l = 1; l < (int)H.lev[pi].size() && l <= H.tail_at[pi]; l++) {
           Grid<float> &F = H.lev[pi][l - 1];
           Grid<float> &C = H.lev[pi][l];
           k_restrict_avg<float><<<nblocks(C.ncell), 256, 0, st>>>(F.ubg, F.n0, F.n1, F.n2,

@@ -1,0 +1,95 @@
+"""The one-cluster tail of the V-cycle (frmg_tail.cuh) at the edges of its
+layout: grids that are all tail, levels kept in one block, planes that do not
+divide evenly over the cluster, coarsest grids of more than one warp's cells,
+and sets of more grids than run at once."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from gpu_common import ctx, dev, host  # noqa: E402
+from oracle import oracle as O  # noqa: E402
+from paper_1110_1379_gb300 import synth  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+# n2 x n1 x n0: one level (8x6x10), coarsest grids of 48 to 2744 cells, 12, 20
+# and 28 planes over 16 blocks, 16^3 and 32^3 tops, one level above the tail
+SHAPES = [(8, 6, 10), (8, 8, 8), (16, 8, 12), (12, 24, 16), (20, 20, 24), (28, 28, 28),
+          (32, 16, 48), (40, 32, 24), (56, 64, 48)]
+
+
+@pytest.fixture(scope="module")
+def C():
+    c = ctx()
+    yield c
+    c.close()
+
+
+def _case(shape, seed, fr0=1e-5):
+    return synth.lognormal_density(shape, seed, sigma=1.0), dict(
+        box=2.0 * shape[2], a=1.0, omega_m=0.24, fr0=fr0)
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_fp64_tail_vcycles_match_oracle(C, shape):
+    """The same V-cycles as the oracle's: iterates agree to FP64 rounding (the
+    bound of the other V-cycle parity tests)."""
+    rho, P = _case(shape, 8100)
+    ref = O.solve(rho, ncycles=2, **P)
+    u = torch.zeros(shape, dtype=torch.float64, device="cuda")
+    C.vcycles(dev(rho), u, 2, **P)
+    assert np.abs(host(u) - ref.u).max() < 1e-10
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("opts", [{}, dict(pre=1, post=2, relax=1.15), dict(fmg=1),
+                                  dict(tau_alpha=1e-13)])
+def test_mixed_tail_solve_matches_oracle(C, shape, opts):
+    """rms(L) <= 1e-11 fixes u to about 1e-10 (smallest mass term beta/2 ~ 1.6);
+    the oracle is solved to 1e-12."""
+    rho, P = _case(shape, 8200)
+    ref = O.solve(rho, tol=1e-12, **P)
+    u = torch.zeros(shape, dtype=torch.float64, device="cuda")
+    st, s = C.solve(dev(rho), u, tol=1e-11, prec="mixed", **opts, **P)
+    assert st == 0 and s.res_rms <= 1e-11
+    assert np.abs(host(u) - ref.u).max() < 1e-8
+
+
+@pytest.mark.parametrize("post", [1, 2])
+def test_mixed_batch_of_tails_and_launched_grids(C, post):
+    """Fields whose tails begin at different depths, more of them than clusters
+    fit the GPU, with odd and even numbers of sweeps: each as if solved alone."""
+    shapes = [(64, 64, 64), (32, 32, 32), (48, 32, 16), (16, 16, 16)] * 6
+    cases = [_case(s, 8300 + i, fr0=(1e-5, 1e-6)[i % 2]) for i, s in enumerate(shapes)]
+    us = [torch.zeros(s, dtype=torch.float64, device="cuda") for s in shapes]
+    st, stats = C.solve_batch([dev(r) for r, _ in cases], us,
+                              boxes=[p["box"] for _, p in cases], avals=[1.0] * len(cases),
+                              fr0s=[p["fr0"] for _, p in cases], omega_m=0.24, tol=1e-11,
+                              prec="mixed", pre=1, post=post, tiling=1)
+    assert st == 0
+    for i in range(8):
+        ref = O.solve(cases[i][0], tol=1e-12, **cases[i][1])
+        assert np.abs(host(us[i]) - ref.u).max() < 1e-8, shapes[i]
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("sizes", [[(8, 8, 8)], [(24, 20, 28), (16, 16, 16), (32, 32, 32)],
+                                   [(16, 12, 8)] * 10])
+def test_patch_tails_match_oracle(C, prec, sizes):
+    n = 40
+    rho, P = _case((n,) * 3, 8400)
+    patches, gp = [], []
+    for i, s in enumerate(sizes):
+        org = (2 + 3 * (i % 4), 1 + i, 3)
+        b = rho[org[2]:org[2] + s[0] // 2, org[1]:org[1] + s[1] // 2, org[0]:org[0] + s[2] // 2]
+        r = synth.refine_density(b, 8500 + i)
+        patches.append(dict(parent=-1, origin=org, rho=r))
+        gp.append(dict(parent=-1, origin=org, density=dev(r),
+                       u=torch.zeros(s, dtype=torch.float64, device="cuda")))
+    _, ref = O.solve_levels(rho, patches, tol=1e-12, **P)
+    u = torch.zeros((n,) * 3, dtype=torch.float64, device="cuda")
+    st, _ = C.solve_levels(dev(rho), u, gp, tol=1e-11, prec=prec, **P)
+    assert st == 0
+    for p, r in zip(gp, ref):
+        assert np.abs(host(p["u"]) - r.u).max() < 1e-8
