@@ -74,8 +74,10 @@ typedef struct {
     int use_graph;          /* capture repeated V-cycles in CUDA graphs; 1 */
     int temporal_depth;     /* FP32 sweeps per pass of the tiled smoother: 1 or 2;
                                0 = library default */
-    int tiling;             /* FP32 shared-memory kernels: 0 = where the grids fill the
-                               GPU, 1 = wherever possible (grids >= 16 a side), -1 = never */
+    int tiling;             /* FP32 shared-memory kernels: 0 = on levels large enough for
+                               them to pay (about 2e5 cells), 1 = wherever possible (grids
+                               >= 16 a side), -1 = never.  Small levels run in one kernel of
+                               their own whatever the choice. */
     int defect_precision;   /* mixed: arithmetic of the fine-grid defect, the update of u
                                and the convergence test: 0 = double-float (pairs of FP32
                                values, ~48-bit significands, on the FP32 pipes),

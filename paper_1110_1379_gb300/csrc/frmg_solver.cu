@@ -603,13 +603,24 @@ static void upload_set(Scope &S, LevelSet<T> &ls, cudaStream_t st, int tiling = 
     txy += (long long)((G.n0 + kTX - 1) / kTX) * ((G.n1 + kTY - 1) / kTY);
   }
   if (ls.tiled) {
-    // chunks of z so that the set yields about 1216 blocks (several waves of
-    // resident blocks), never thinner than 32 planes; sets too small to fill
-    // the GPU with such blocks use the one-thread-per-cell kernel instead
+    // (two sweeps per pass) chunks of z so that the set yields about 1216 blocks
+    // (several waves of resident blocks), never thinner than 32 planes
     long long nz = std::max<long long>(1, (1216 + txy - 1) / txy);
     ls.zc = (int)std::max<long long>(std::min(32, maxn2), (maxn2 + nz - 1) / nz);
     ls.tiled_ok = true;
-    if (tiling == 0 && txy * ((maxn2 + ls.zc - 1) / ls.zc) < 304) ls.tiled = false;
+    if (tiling == 0) {
+      // worth it from about 2e5 cells on, unless most of the tiles' cells lie
+      // outside the grids (narrow grids).  Whole solves, one colour per launch
+      // against tiles: 96^3 3.12 and 2.40 ms, 64^3 1.88 and 1.62, 48 x 64 x 80
+      // 2.11 and 1.92; sets of 1.1e5 cells no difference; 24 x 256 x 256 (37 % of
+      // the tiles used) 30.2 and 29.4, 16 x 256 x 256 (25 %) 22.9 and 27.2
+      long long cells = 0, covered = 0;
+      for (const Grid<T> &G : ls.h) {
+        cells += G.ncell;
+        covered += (long long)((G.n0 + kTX - 1) / kTX) * ((G.n1 + kTY - 1) / kTY) * kTX * kTY * G.n2;
+      }
+      if (cells < 196608 || 100 * cells < 35 * covered) ls.tiled = false;
+    }
     if (tiling < 0) ls.tiled = false;
   }
   if (ls.tiled_ok) {

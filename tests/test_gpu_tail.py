@@ -14,9 +14,10 @@ from paper_1110_1379_gb300 import synth  # noqa: E402
 pytestmark = pytest.mark.gpu
 
 # n2 x n1 x n0: one level (8x6x10), coarsest grids of 48 to 2744 cells, 12, 20
-# and 28 planes over 16 blocks, 16^3 and 32^3 tops, one level above the tail
+# and 28 planes over 16 blocks, 16^3 and 32^3 tops, one level above the
+# tail (launched cell by cell, and in tiles of which some are partial)
 SHAPES = [(8, 6, 10), (8, 8, 8), (16, 8, 12), (12, 24, 16), (20, 20, 24), (28, 28, 28),
-          (32, 16, 48), (40, 32, 24), (56, 64, 48)]
+          (32, 16, 48), (40, 32, 24), (56, 64, 48), (64, 56, 72)]
 
 
 @pytest.fixture(scope="module")
