@@ -36,6 +36,7 @@
 #include <utility>
 
 #include "frmg_dfmath.cuh"
+#include "frmg_f64math.cuh"
 
 namespace frmg {
 
@@ -106,7 +107,7 @@ __device__ __forceinline__ float m_expm1(float d) {
   if (fabsf(d) < 0.0625f) return m_expm1_taylor(d);
   return __fsub_rn(expf(d), 1.0f);
 }
-__device__ __forceinline__ double m_expm1(double v) { return expm1(v); }
+__device__ __forceinline__ double m_expm1(double v) { return f64_expm1(v); }
 __device__ __forceinline__ float m_sqrt(float v) { return sqrtf(v); }
 __device__ __forceinline__ double m_sqrt(double v) { return sqrt(v); }
 __device__ __forceinline__ float m_rsqrt(float v) { return rsqrtf(v); }
@@ -254,6 +255,35 @@ struct OpAcc<float, false> {
   }
 };
 
+// The same regrouping in FP64 (24 FP64 operations for the six faces instead of
+// 36); a ghost's terms join the sums directly.
+template <>
+struct OpAcc<double, false> {
+  double di, Ei, xi, Bi, ubi;
+  double S1 = 0.0, S2 = 0.0, S3 = 0.0;
+  int n = 0;
+  __device__ __forceinline__ OpAcc(double d, double E, double x, double B, double ub)
+      : di(d), Ei(E), xi(x), Bi(B), ubi(ub) {}
+  __device__ __forceinline__ void reg(double dj, double xj, double, double) {
+    const double dd = dj - di;
+    S1 += dd;
+    S2 = fma(xj, dd, S2);
+    S3 += xj;
+    n++;
+  }
+  __device__ __forceinline__ void ghost(double ubf) {
+    double ga = 0.0, gd = 0.0;
+    face_ghost<double, false>(ubf, di, Ei, xi, Bi, ubi, ga, gd);
+    S2 += ga;
+    S3 -= gd;
+  }
+  __device__ __forceinline__ void done(double &a, double &da) const {
+    const double b1 = Bi + 1.0;
+    a = fma(b1, S1, S2);
+    da = fma(Bi, S1, (double)-n * b1) - S3;
+  }
+};
+
 // The FP32 correction form regroups its face sum the same way: with
 // P = E x (so B = E + P) and g_j = ub_j - ub_i,
 //   acc  = sum (P_i + P_j) g_j + (B_i + B_j)(d_j - d_i)
@@ -293,18 +323,18 @@ struct OpAcc<float, true> {
 
 // Mass term and final assembly:  N = (alpha/2) acc + beta F (e^{-d/2} - 1),
 // dN = (alpha/2) dacc - (beta/2) F e^{-d/2},  F = e^{-ub/2}.
-// FP64 uses IEEE sqrt and division; FP32 uses the SFU reciprocal square root
+// FP32 uses the SFU reciprocal square root
 // and reciprocal (the same expression in every FP32 kernel, so all of them
 // see one and the same discrete operator).
 __device__ __forceinline__ void finish_op(double xi, double Ei, double acc, double dacc,
                                           double ah, double beta, bool bg, double &N,
                                           double &dN) {
-  double B1 = 1.0 + xi;
-  double s = sqrt(B1);
-  double y = -xi / (B1 + s);
-  double F = bg ? rsqrt(Ei) : 1.0;
-  N = ah * acc + beta * F * y;
-  dN = ah * dacc - 0.5 * beta * F / s;
+  const double B1 = 1.0 + xi;
+  const double rs = f64_rsqrt(B1);
+  const double y = -xi * f64_rcp(fma(B1, rs, B1));  // -x / (B + sqrt B)
+  const double bF = bg ? beta * rsqrt(Ei) : beta;
+  N = fma(ah, acc, bF * y);
+  dN = fma(ah, dacc, -0.5 * bF * rs);
 }
 
 // SFU reciprocal and reciprocal square root (PTX rcp.approx / rsqrt.approx,
@@ -331,16 +361,34 @@ __device__ __forceinline__ void finish_op(float xi, float Ei, float acc, float d
   dN = fmaf(ah, dacc, -__fmul_rn(__fmul_rn(0.5f, bF), rs));
 }
 
-__device__ __forceinline__ double newton_step(double r, double dN) { return -r / dN; }
 __device__ __forceinline__ float newton_step(float r, float dN) {
   return __fmul_rn(-r, sfu_rcp(dN));
 }
 // relaxed Newton step w (N - f) / -dN of a cell
-__device__ __forceinline__ double newton_du(double N, double f, double dN, double w) {
-  return w * newton_step(N - f, dN);
-}
 __device__ __forceinline__ float newton_du(float N, float f, float dN, float w) {
   return __fmul_rn(w, newton_step(__fsub_rn(N, f), dN));
+}
+
+// The clamped, relaxed Newton step of a cell from its face sums.  FP64, plain
+// form: with q = B + sqrt(B) both N - f and dN are multiplied by q, so that one
+// reciprocal serves the mass term and the step.
+template <typename T, bool BG>
+__device__ __forceinline__ T newton_from_sums(T xi, T Ei, T acc, T dacc, T f, T ah, T beta, T cap,
+                                              T relax) {
+  if constexpr (sizeof(T) == 8 && !BG) {
+    const T B1 = T(1) + xi, rs = f64_rsqrt(B1), q = fma(B1, rs, B1);
+    const T num = fma(-beta, xi, fma(ah, acc, -f) * q);
+    const T den = fma(ah, dacc, T(-0.5) * beta * rs) * q;
+    const T du = -relax * num * f64_rcp(den);
+    // the comparison by the high words first (an FP64 comparison takes the FP64 pipe)
+    if ((__double2hiint(du) & 0x7fffffff) < __double2hiint(cap)) return du;
+    return du > cap ? cap : (du < -cap ? -cap : du);
+  } else {
+    T N, dN;
+    finish_op(xi, Ei, acc, dacc, ah, beta, BG, N, dN);
+    const T du = newton_du(N, f, dN, relax);
+    return du > cap ? cap : (du < -cap ? -cap : du);
+  }
 }
 
 // ---- packed FP32 pairs (add2, sub2, fma2, mul2, splat2 of frmg_dfmath.cuh)
@@ -396,13 +444,14 @@ __device__ __forceinline__ float2 newton2_plain(float2 di, float2 xi, float2 fi,
   return add2(di, du);
 }
 
-// A_i (or N_i) and its derivative at cell (i,j,k) from global memory.
+// Face sums of the operator and its derivative at cell (i,j,k) from global
+// memory, with the cell's own u, x and E.
 template <typename T, bool BG>
-__device__ __forceinline__ void cell_eval(const Grid<T> &G, int i, int j, int k, long long c,
-                                          T &N, T &dN) {
-  const T di = G.u[c];
-  const T xi = G.x[c];
-  const T Ei = BG ? (T)G.Ebg[c] : T(1);
+__device__ __forceinline__ void cell_sums(const Grid<T> &G, int i, int j, int k, long long c,
+                                          T &di, T &xi, T &Ei, T &acc, T &dacc) {
+  di = G.u[c];
+  xi = G.x[c];
+  Ei = BG ? (T)G.Ebg[c] : T(1);
   const T ubi = BG ? (T)G.ubg[c] : T(0);
   const T Bi = BG ? Ei + Ei * xi : T(1) + xi;
   OpAcc<T, BG> A(di, Ei, xi, Bi, ubi);
@@ -432,8 +481,15 @@ __device__ __forceinline__ void cell_eval(const Grid<T> &G, int i, int j, int k,
   if (k < G.n2 - 1) nb(c + sz);
   else if (!dir) nb(c - (G.n2 - 1) * sz);
   else A.ghost(face_value(G, 5, i, j, k));
-  T acc, dacc;
   A.done(acc, dacc);
+}
+
+// A_i (or N_i) and its derivative at cell (i,j,k).
+template <typename T, bool BG>
+__device__ __forceinline__ void cell_eval(const Grid<T> &G, int i, int j, int k, long long c,
+                                          T &N, T &dN) {
+  T di, xi, Ei, acc, dacc;
+  cell_sums<T, BG>(G, i, j, k, c, di, xi, Ei, acc, dacc);
   finish_op(xi, Ei, acc, dacc, G.ah, G.beta, BG, N, dN);
 }
 
@@ -445,16 +501,23 @@ __device__ __forceinline__ T rhs_at(const Grid<T> &G, long long c) {
 template <typename T, bool BG>
 __device__ __forceinline__ void ngs_update(const Grid<T> &G, int i, int j, int k) {
   long long c = idx3(G, i, j, k);
-  T N, dN;
-  cell_eval<T, BG>(G, i, j, k, c, N, dN);
-  T du = newton_du(N, rhs_at(G, c), dN, G.relax);
-  du = du > G.cap ? G.cap : (du < -G.cap ? -G.cap : du);
-  T unew = G.u[c] + du;
+  T di, xi, Ei, acc, dacc;
+  cell_sums<T, BG>(G, i, j, k, c, di, xi, Ei, acc, dacc);
+  const T unew = di + newton_from_sums<T, BG>(xi, Ei, acc, dacc, rhs_at(G, c), G.ah, G.beta,
+                                              G.cap, G.relax);
   G.u[c] = unew;
   G.x[c] = m_expm1(unew);
 }
 
 // ---------------------------------------------------------------------------
+// Threads per block of the one-thread-per-cell kernels without a block sum.
+// FP64: the FP64 pipes bound them, and small blocks spread a small level over
+// all SMs (32^3: 512 warps on 152 SMs).
+template <typename T>
+__host__ __device__ constexpr int cell_threads() {
+  return sizeof(T) == 8 ? 64 : 256;
+}
+
 // One colour of a red-black Newton-Gauss-Seidel sweep; one thread per cell of
 // that colour.  off[] maps blocks to grids (n0/2 * n1 * n2 threads per grid).
 template <typename T, bool BG>
@@ -596,46 +659,56 @@ __global__ void k_reduce_chunks(const double *tmp, int nch, int ngrid, double *o
 
 // Fused residual + restriction (Sec. V.B.2): for each coarse cell, the 8 fine
 // children give  u^H = uR = mean(u^h),  x^H = expm1(u^H),  f^H <- mean(d^h)
-// (the coarse operator is added by k_fas_rhs).  One thread per coarse cell;
-// optionally accumulates per-block (sum d^2, max |d|) of the fine residual.
+// (the coarse operator is added by k_fas_rhs).  One thread per fine cell, the
+// children of a coarse cell in eight neighbouring lanes; a block's 32 coarse
+// cells are written by its first warp.  Optionally accumulates per-block
+// (sum d^2, max |d|) of the fine residual.  (One thread per coarse cell left
+// most SMs idle on small FP64 levels: 45 us at 32^3 against 8 us.)
 template <typename T, bool BG>
 __global__ void __launch_bounds__(256)
     k_resid_restrict(const Grid<T> *fine, const Grid<T> *coarse, const int *off, int ngrid,
                      const int *active, int fpar, int cpar, double *partial) {
+  __shared__ T cu[32], cd[32];
   int g = find_grid(off, ngrid, blockIdx.x);
   const Grid<T> F = view(fine, g, fpar);
   const Grid<T> C = view(coarse, g, cpar);
-  float ss = 0.0f, mx = 0.0f;
-  long long t = (long long)(blockIdx.x - off[g]) * blockDim.x + threadIdx.x;
-  if (grid_active(active, F.field) && t < C.ncell) {
+  const bool on = grid_active(active, F.field);
+  const long long c0 = (long long)(blockIdx.x - off[g]) * 32;
+  const long long t = c0 + (threadIdx.x >> 3);
+  T d = T(0), u = T(0);
+  if (on && t < C.ncell) {
+    const int q = threadIdx.x & 7;
     int I, J, K;
     cell_ijk(C, t, I, J, K);
-    T su = T(0), sd = T(0);
-#pragma unroll
-    for (int cz = 0; cz < 2; cz++)
-#pragma unroll
-      for (int cy = 0; cy < 2; cy++)
-#pragma unroll
-        for (int cx = 0; cx < 2; cx++) {
-          int i = 2 * I + cx, j = 2 * J + cy, k = 2 * K + cz;
-          long long c = idx3(F, i, j, k);
-          T N, dN;
-          cell_eval<T, BG>(F, i, j, k, c, N, dN);
-          T d = N - rhs_at(F, c);
-          sd += d;
-          const float df_ = (float)d;
-          ss = fmaf(df_, df_, ss);
-          mx = fmaxf(mx, fabsf(df_));
-          su += F.u[c];
-        }
-    T uh = su * T(0.125);
-    C.uR[t] = uh;
-    C.u[t] = uh;
-    C.x[t] = m_expm1(uh);
-    const_cast<T *>(C.f)[t] = sd * T(0.125);
+    const int i = 2 * I + (q & 1), j = 2 * J + ((q >> 1) & 1), k = 2 * K + (q >> 2);
+    const long long c = idx3(F, i, j, k);
+    T N, dN;
+    cell_eval<T, BG>(F, i, j, k, c, N, dN);
+    d = N - rhs_at(F, c);
+    u = F.u[c];
+  }
+  const float df_ = (float)d;
+  // even lanes add up u, odd lanes d (one addition per step for the two sums)
+  const bool odd = threadIdx.x & 1;
+  const T give = odd ? u : d;
+  T s = (odd ? d : u) + __shfl_xor_sync(0xffffffffu, give, 1);
+  s += __shfl_xor_sync(0xffffffffu, s, 2);
+  s += __shfl_xor_sync(0xffffffffu, s, 4);
+  if ((threadIdx.x & 7) == 0) cu[threadIdx.x >> 3] = s;
+  if ((threadIdx.x & 7) == 1) cd[threadIdx.x >> 3] = s;
+  __syncthreads();
+  if (threadIdx.x < 32 && on && c0 + threadIdx.x < C.ncell) {
+    const long long w = c0 + threadIdx.x;
+    const T uh = cu[threadIdx.x] * T(0.125);
+    C.uR[w] = uh;
+    C.u[w] = uh;
+    C.x[w] = m_expm1(uh);
+    const_cast<T *>(C.f)[w] = cd[threadIdx.x] * T(0.125);
   }
   // fine-grid residual norm partials (the residual after pre-smoothing)
-  if (partial) block_reduce2f<256>(ss, mx, &partial[2 * blockIdx.x], &partial[2 * blockIdx.x + 1]);
+  if (partial)
+    block_reduce2f<256>(df_ * df_, fabsf(df_), &partial[2 * blockIdx.x],
+                        &partial[2 * blockIdx.x + 1]);
 }
 
 // f^H = A^H(R u^h) - R d^h, in place over the R d^h stored in f (fs = 1, fo = 0).

@@ -439,9 +439,12 @@ template <typename T>
 struct LevelSet {
   std::vector<Grid<T>> h;
   Grid<T> *d = nullptr;
-  std::vector<int> off_half, off_full;
-  int *d_off_half = nullptr, *d_off_full = nullptr;
-  int nblk_half = 0, nblk_full = 0;
+  // block offsets of the one-thread-per-cell kernels: cells of one colour and
+  // all cells (cell_threads per block), all cells (256 per block), and the
+  // cells of the next finer level (256 per block, 32 coarse cells)
+  std::vector<int> off_half, off_cell, off_full, off_fine;
+  int *d_off_half = nullptr, *d_off_cell = nullptr, *d_off_full = nullptr, *d_off_fine = nullptr;
+  int nblk_half = 0, nblk_cell = 0, nblk_full = 0, nblk_fine = 0;
   // tiled FP32 smoother: blocks per grid for TX x TY tiles and zc-plane chunks
   bool tiled = false;     // the tiled smoother is used for this set
   bool tiled_ok = false;  // it could be used (every grid >= 16 cells a side)
@@ -567,26 +570,35 @@ static void upload_set(Scope &S, LevelSet<T> &ls, cudaStream_t st, int tiling = 
   if (ls.empty()) return;
   int ng = ls.size();
   ls.off_half.assign(ng + 1, 0);
+  ls.off_cell.assign(ng + 1, 0);
   ls.off_full.assign(ng + 1, 0);
+  ls.off_fine.assign(ng + 1, 0);
   for (int g = 0; g < ng; g++) {
     long long half = (long long)(ls.h[g].n0 / 2) * ls.h[g].n1 * ls.h[g].n2;
-    ls.off_half[g + 1] = ls.off_half[g] + nblocks(half);
+    ls.off_half[g + 1] = ls.off_half[g] + nblocks(half, cell_threads<T>());
+    ls.off_cell[g + 1] = ls.off_cell[g] + nblocks(ls.h[g].ncell, cell_threads<T>());
     ls.off_full[g + 1] = ls.off_full[g] + nblocks(ls.h[g].ncell);
+    ls.off_fine[g + 1] = ls.off_fine[g] + nblocks(ls.h[g].ncell, 32);
   }
   ls.nblk_half = ls.off_half[ng];
+  ls.nblk_cell = ls.off_cell[ng];
   ls.nblk_full = ls.off_full[ng];
+  ls.nblk_fine = ls.off_fine[ng];
   // every grid reaches the device through here: its index dividers too
   for (auto &g : ls.h) {
     g.fd0 = make_fastdiv((unsigned)g.n0);
     g.fd1 = make_fastdiv((unsigned)g.n1);
   }
   ls.d = S.get<Grid<T>>(ng);
-  ls.d_off_half = S.get<int>(ng + 1);
-  ls.d_off_full = S.get<int>(ng + 1);
+  ls.d_off_half = S.get<int>(4 * (size_t)(ng + 1));
+  ls.d_off_cell = ls.d_off_half + (ng + 1);
+  ls.d_off_full = ls.d_off_cell + (ng + 1);
+  ls.d_off_fine = ls.d_off_full + (ng + 1);
   CK(cudaMemcpyAsync(ls.d, ls.h.data(), ng * sizeof(Grid<T>), cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(ls.d_off_half, ls.off_half.data(), (ng + 1) * sizeof(int),
-                     cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(ls.d_off_full, ls.off_full.data(), (ng + 1) * sizeof(int),
+  std::vector<int> offs;
+  for (auto *v : {&ls.off_half, &ls.off_cell, &ls.off_full, &ls.off_fine})
+    offs.insert(offs.end(), v->begin(), v->end());
+  CK(cudaMemcpyAsync(ls.d_off_half, offs.data(), offs.size() * sizeof(int),
                      cudaMemcpyHostToDevice, st));
   ls.dirichlet = ls.h[0].bnd != nullptr;
   for (int g = 1; g < ng; g++)
@@ -737,7 +749,7 @@ static void upload_set(Scope &S, LevelSet<T> &ls, cudaStream_t st, int tiling = 
                        cudaMemcpyHostToDevice, st));
     ls.rr_tiled = true;
   }
-  ls.partial = S.get<double>(2 * (size_t)std::max(ls.nblk_full, ls.nblk_rr));
+  ls.partial = S.get<double>(2 * (size_t)std::max({ls.nblk_full, ls.nblk_fine, ls.nblk_rr}));
   ls.red_nch = red_chunks(ls.off_full);
   if (ls.red_nch) ls.red_tmp = S.get<double>(2 * (size_t)ls.red_nch * ng);
   ls.red = S.get<double>(2 * (size_t)ng);
@@ -1259,7 +1271,7 @@ static void smooth_set(frmg_ctx *ctx, LevelSet<T> &s, int sweeps, const std::vec
   for (int it = 0; it < sweeps; it++)
     for (int colour = 0; colour < 2; colour++) {
       PROF(pname("smooth", sizeof(T) == 8, fine));
-      k_smooth<T, BG><<<s.nblk_half, 256, 0, st>>>(s.d, s.d_off_half, s.size(), colour, active,
+      k_smooth<T, BG><<<s.nblk_half, cell_threads<T>(), 0, st>>>(s.d, s.d_off_half, s.size(), colour, active,
                                                    par);
       CK_LAUNCH(ctx);
     }
@@ -1285,8 +1297,8 @@ static void prolong_level(frmg_ctx *ctx, Hier<T> &H, int l, const int *active, c
     }
   }
   if (!done)
-    k_prolong<T><<<C.nblk_full, 256, 0, st>>>(F.d, C.d, C.d_off_full, F.size(), active,
-                                              H.par[l], H.par[l + 1]);
+    k_prolong<T><<<C.nblk_cell, cell_threads<T>(), 0, st>>>(F.d, C.d, C.d_off_cell, F.size(),
+                                                            active, H.par[l], H.par[l + 1]);
   CK_LAUNCH(ctx);
 }
 
@@ -1306,7 +1318,8 @@ static void fas_rhs(frmg_ctx *ctx, LevelSet<T> &C, int par, const int *active, c
     }
   }
   if (!done)
-    k_fas_rhs<T, BG><<<C.nblk_full, 256, 0, st>>>(C.d, C.d_off_full, C.size(), active, par);
+    k_fas_rhs<T, BG><<<C.nblk_cell, cell_threads<T>(), 0, st>>>(C.d, C.d_off_cell, C.size(),
+                                                                active, par);
   CK_LAUNCH(ctx);
 }
 
@@ -1396,12 +1409,12 @@ static void vcycle_launched(frmg_ctx *ctx, Hier<T> &H, int l, const CycleOpts &o
         launch_rr_tiled<BG>(ctx, F, C, active, H.par[l], H.par[l + 1],
                             l == 0 ? C.partial : nullptr, st);
       } else {
-        k_resid_restrict<T, BG><<<C.nblk_full, 256, 0, st>>>(F.d, C.d, C.d_off_full, C.size(),
+        k_resid_restrict<T, BG><<<C.nblk_fine, 256, 0, st>>>(F.d, C.d, C.d_off_fine, C.size(),
                                                              active, H.par[l], H.par[l + 1],
                                                              l == 0 ? C.partial : nullptr);
       }
     } else {
-      k_resid_restrict<T, BG><<<C.nblk_full, 256, 0, st>>>(F.d, C.d, C.d_off_full, C.size(),
+      k_resid_restrict<T, BG><<<C.nblk_fine, 256, 0, st>>>(F.d, C.d, C.d_off_fine, C.size(),
                                                            active, H.par[l], H.par[l + 1],
                                                            l == 0 ? C.partial : nullptr);
     }
@@ -1605,7 +1618,7 @@ static void fused_fine_norms(frmg_ctx *ctx, Hier<T> &H, int np, cudaStream_t st,
   if (ng + nt == 0) return;
   double *hp = pinned_buf(ctx, 2 * (size_t)(ng + nt));
   if (ng) {
-    const int *offs = H.cont[0].rr_tiled ? H.cont[0].d_off_rr : C.d_off_full;
+    const int *offs = H.cont[0].rr_tiled ? H.cont[0].d_off_rr : C.d_off_fine;
     k_reduce_partials<<<ng, 256, 0, st>>>(C.partial, offs, ng, C.red);
     CK_LAUNCH(ctx);
     CK(cudaMemcpyAsync(hp, C.red, 2 * ng * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -1659,7 +1672,7 @@ static std::vector<double> tau_norms(frmg_ctx *ctx, Hier<T> &H, int np, cudaStre
   if (H.cont.empty() || H.cont[0].empty()) return out;
   auto &F = H.cont[0];
   auto &C = H.next[0];
-  k_resid_restrict<T, false><<<C.nblk_full, 256, 0, st>>>(F.d, C.d, C.d_off_full, C.size(),
+  k_resid_restrict<T, false><<<C.nblk_fine, 256, 0, st>>>(F.d, C.d, C.d_off_fine, C.size(),
                                                           nullptr, H.par[0], H.par[1], nullptr);
   CK_LAUNCH(ctx);
   k_tau<T><<<C.nblk_full, 256, 0, st>>>(F.d, C.d, C.d_off_full, C.size(), H.par[0], H.par[1],

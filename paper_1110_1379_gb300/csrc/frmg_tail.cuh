@@ -213,11 +213,11 @@ struct TailPut {
   }
 };
 
-// A_i (or N_i) and its derivative at cell (i, j) of own plane kl: cell_eval on
-// the level's shared-memory arrays.  All loads come first.
+// Face sums at cell (i, j) of own plane kl: cell_sums on the level's
+// shared-memory arrays.  All loads come first.
 template <typename T, bool BG, bool DIR>
-__device__ __forceinline__ void tail_eval(const TailLevel<T> &L, T beta, int i, int j, int kl,
-                                          T &ui, T &xi, T &N, T &dN) {
+__device__ __forceinline__ void tail_sums(const TailLevel<T> &L, int i, int j, int kl, T &ui,
+                                          T &xi, T &Ei, T &acc, T &dacc) {
   const T *sm = tail_smem<T>();
   const int n0 = L.n0, pl = L.plane, o = (kl + 1) * pl + j * n0 + i;
   const bool b0 = i == 0, b1 = i == n0 - 1, b2 = j == 0, b3 = j == L.n1 - 1;
@@ -234,7 +234,7 @@ __device__ __forceinline__ void tail_eval(const TailLevel<T> &L, T beta, int i, 
   }
   ui = sm[L.u + o];
   xi = sm[L.x + o];
-  const T Ei = BG ? sm[L.E + o] : T(1);
+  Ei = BG ? sm[L.E + o] : T(1);
   const T ubi = BG ? sm[L.ub + o] : T(0);
   const T Bi = BG ? Ei + Ei * xi : T(1) + xi;
   OpAcc<T, BG> A(ui, Ei, xi, Bi, ubi);
@@ -250,8 +250,15 @@ __device__ __forceinline__ void tail_eval(const TailLevel<T> &L, T beta, int i, 
 #pragma unroll
     for (int q = 0; q < 6; q++) A.reg(du[q], dx[q], db[q], dE[q]);
   }
-  T acc, dacc;
   A.done(acc, dacc);
+}
+
+// A_i (or N_i) and its derivative at that cell.
+template <typename T, bool BG, bool DIR>
+__device__ __forceinline__ void tail_eval(const TailLevel<T> &L, T beta, int i, int j, int kl,
+                                          T &ui, T &xi, T &N, T &dN) {
+  T Ei, acc, dacc;
+  tail_sums<T, BG, DIR>(L, i, j, kl, ui, xi, Ei, acc, dacc);
   finish_op(xi, Ei, acc, dacc, L.ah, beta, BG, N, dN);
 }
 
@@ -317,12 +324,10 @@ __device__ __noinline__ void tail_smooth(const TailBlock<T> &B, int l, int sweep
   };
   auto update = [&](int c) {
     const int i = i0 + ((c0 + c) & 1), q = j * L.n0 + i;
-    T ui, xi, N, dN;
+    T ui, xi, Ei, acc, dacc;
     const T f = sm[L.f + kl * L.plane + q];
-    tail_eval<T, BG, DIR>(L, beta, i, j, kl, ui, xi, N, dN);
-    T du = newton_du(N, f, dN, relax);
-    du = du > cap ? cap : (du < -cap ? -cap : du);
-    const T un = ui + du;
+    tail_sums<T, BG, DIR>(L, i, j, kl, ui, xi, Ei, acc, dacc);
+    const T un = ui + newton_from_sums<T, BG>(xi, Ei, acc, dacc, f, L.ah, beta, cap, relax);
     put(L.u, un, L.x, m_expm1(un), kl, q);
   };
   const bool one = n <= nt;
@@ -594,8 +599,8 @@ __device__ __noinline__ void tail_coarsest_warp(TailBlock<T> &B, int l, const Ta
       }
     }
   }
-  // N - f and dN of a cell, its u and x
-  auto eval = [&](int p, int v, T &ui, T &xi, T &r, T &dN, T &N) {
+  // face sums of a cell, its u and x
+  auto sums = [&](int p, int v, T &ui, T &xi, T &a, T &da) {
     T du[6], dx[6], db[6], dE[6];
 #pragma unroll
     for (int q = 0; q < 6; q++) {
@@ -616,10 +621,7 @@ __device__ __noinline__ void tail_coarsest_warp(TailBlock<T> &B, int l, const Ta
       if (DIR && g[q]) acc.ghost(gb[p][v][q]);
       else acc.reg(du[q], dx[q], db[q], dE[q]);
     }
-    T a, da;
     acc.done(a, da);
-    finish_op(xi, Ei, a, da, ah, beta, BG, N, dN);
-    r = N - f[p][v];
   };
   auto sum = [&](A a) {
     for (int q = 16; q > 0; q >>= 1) a += __shfl_xor_sync(0xffffffffu, a, q);
@@ -634,11 +636,10 @@ __device__ __noinline__ void tail_coarsest_warp(TailBlock<T> &B, int l, const Ta
 #pragma unroll
         for (int p = 0; p < P; p++) {
           if (!mine[p]) continue;
-          T ui, xi, r, dN, N;
-          eval(p, v, ui, xi, r, dN, N);
-          T du = newton_du(N, f[p][v], dN, relax);
-          du = du > cap ? cap : (du < -cap ? -cap : du);
-          const T un = ui + du;
+          T ui, xi, a, da;
+          sums(p, v, ui, xi, a, da);
+          const T un = ui + newton_from_sums<T, BG>(xi, E[p][v], a, da, f[p][v], ah, beta, cap,
+                                                    relax);
           U[at[p][v]] = un;
           X[at[p][v]] = m_expm1(un);
         }
@@ -652,9 +653,10 @@ __device__ __noinline__ void tail_coarsest_warp(TailBlock<T> &B, int l, const Ta
 #pragma unroll
         for (int v = 0; v < 2; v++) {
           if (!mine[p]) continue;
-          T ui, xi, r, dN, N;
-          eval(p, v, ui, xi, r, dN, N);
-          const A d = (A)r;
+          T ui, xi, a, da, N, dN;
+          sums(p, v, ui, xi, a, da);
+          finish_op(xi, E[p][v], a, da, ah, beta, BG, N, dN);
+          const A d = (A)(N - f[p][v]);
           if (what) {
             s += d * d;
           } else {
