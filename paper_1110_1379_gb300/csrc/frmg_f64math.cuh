@@ -48,16 +48,12 @@ __device__ const double kExpTab[32] = {
     0x1.68efde3a8a893p-54,  0x1.34d754db0abb6p-55,  0x1.59f48a72a4c6cp-55,
     0x1.690cebb7aafb0p-56,  0x1.063e1e21c5409p-54};
 
-// e^u - 1 by the table-driven method (P. T. P. Tang, "Table-driven
+// e^u = t (1 + p) with t = 2^(k/16) and p = e^r - 1, u = k ln2/16 + r, |r| <=
+// ln2/32: the table-driven method of P. T. P. Tang, "Table-driven
 // implementation of the Expm1 function in IEEE floating-point arithmetic",
-// ACM TOMS 18 (1992) 211): u = k ln2/16 + r, |r| <= ln2/32, e^u = t (1 + p) with
-// t = 2^(k/16) from a 16-entry table and p = e^r - 1 by its Taylor series to
-// degree 7 (remainder below 2^-54 relative to r); e^u - 1 = (t - 1) + t p, the
-// first bracket exact.  For |u| < ln2/32 this is the series itself.  Error at
-// most 2 ulp (near |u| = 0.022; 0.8 ulp beyond 0.4), below 0.07 ulp of e^u where
-// it is largest; 14 FP64 instructions.
-__device__ __forceinline__ double f64_expm1(double u) {
-  if (!(fabs(u) < 700.0)) return expm1(u);  // overflow, -1, NaN
+// ACM TOMS 18 (1992) 211, with a 16-entry table and the Taylor series of p to
+// degree 7 (remainder below 2^-54 relative to r).  |u| < 700.
+__device__ __forceinline__ void f64_exp_parts(double u, double &t, double &p) {
   const double shift = 0x1.8p52;
   const double ks = fma(u, 0x1.71547652b82fep+4, shift);  // 16 / ln2
   const int k = __double2loint(ks);
@@ -67,12 +63,29 @@ __device__ __forceinline__ double f64_expm1(double u) {
   r = fma(-kd, 0x1.a39ef35793c76p-37, r);
   const int m = (k + 8) >> 4, i = (k + 8) & 15;
   const double t0 = __ldg(kExpTab + i), dt = __ldg(kExpTab + 16 + i);
-  const double t = __hiloint2double(__double2hiint(t0) + (m << 20), __double2loint(t0));
+  t = __hiloint2double(__double2hiint(t0) + (m << 20), __double2loint(t0));
   const double r2 = r * r;
   const double a = fma(r, 1.0 / 6.0, 0.5), b = fma(r, 1.0 / 120.0, 1.0 / 24.0),
                c = fma(r, 1.0 / 5040.0, 1.0 / 720.0);
-  const double p = fma(fma(fma(c, r2, b), r2, a), r2, r + dt);
+  p = fma(fma(fma(c, r2, b), r2, a), r2, r + dt);
+}
+
+// e^u - 1 = (t - 1) + t p, the first bracket exact; for |u| < ln2/32 the series
+// itself.  Error at most 2 ulp (near |u| = 0.022; 0.8 ulp beyond 0.4), below
+// 0.07 ulp of e^u where it is largest; 14 FP64 instructions.
+__device__ __forceinline__ double f64_expm1(double u) {
+  if (!(fabs(u) < 700.0)) return expm1(u);  // overflow, -1, NaN
+  double t, p;
+  f64_exp_parts(u, t, p);
   return fma(t, p, t - 1.0);
+}
+
+// e^u, error below 1 ulp.
+__device__ __forceinline__ double f64_exp(double u) {
+  if (!(fabs(u) < 700.0)) return exp(u);
+  double t, p;
+  f64_exp_parts(u, t, p);
+  return fma(t, p, t);
 }
 
 }  // namespace frmg

@@ -47,6 +47,7 @@
 
 #include "frmg.h"
 #include "frmg_dfmath.cuh"
+#include "frmg_f64math.cuh"
 #include "frmg_internal.h"
 
 using namespace frmg;
@@ -75,7 +76,14 @@ struct MError {
 
 constexpr int kNT = 256;
 
-long long nblk(long long n) { return (n + kNT - 1) / kNT; }
+long long nblk(long long n, int nt = kNT) { return (n + nt - 1) / nt; }
+
+// Threads per block of the per-active-cell kernels without a block sum; small
+// in FP64, whose pipes bound them, so that small levels spread over all SMs.
+template <typename T>
+__host__ __device__ constexpr int m_threads() {
+  return sizeof(T) == 8 ? 64 : kNT;
+}
 
 // One level of a masked region, iterate and work arrays in T (FP64, or FP32
 // in a mixed-precision solve); the mask, density and ghost boundary values are
@@ -89,6 +97,7 @@ struct MLevelT {
                     // (BG: 0) elsewhere
   T *b;             // exp(u) (BG: expm1(v)) of every cell, rewritten wherever u changes
   const double *m;  // mask
+  const unsigned char *nb;  // bit f: the neighbour across face f is active (active cells)
   const double *rho;
   T *f;             // FAS right-hand side (0 on the finest level)
   T *uR;            // R u^h of the active cells (coarse levels)
@@ -105,7 +114,7 @@ struct MLevelT {
 };
 using MLevel = MLevelT<double>;
 
-__device__ __forceinline__ double m_exp(double v) { return exp(v); }
+__device__ __forceinline__ double m_exp(double v) { return f64_exp(v); }
 __device__ __forceinline__ float m_exp(float v) { return expf(v); }
 // the per-cell cache of a new value
 template <typename T, bool BG>
@@ -144,22 +153,22 @@ __device__ __forceinline__ void m_cell(const MLevelT<T, BG> &L, long long c, T &
     // correction differences); a ghost face has background value
     // u_b - r u_b + r ubg_i and correction r v_i; the mass term is
     // beta e^{-ubg_i/2} (e^{-v_i/2} - 1); the density term cancels
-    const T vi = L.u[c], xi = L.b[c], mi = (T)L.m[c];
+    const T vi = L.u[c], xi = L.b[c];
     const T gi = L.bgu[c], Ei = L.bgE[c];
     const T Bi = Ei + Ei * xi;
     T acc = T(0), dacc = T(0);
+    const unsigned nb = L.nb[c];
 #pragma unroll
     for (int f = 0; f < 6; f++) {
       const long long cj = c + face_step(L, f);
-      const double mjd = L.m[cj];
-      if (mjd > 0.0) {
+      if (nb >> f & 1) {
         const T vj = L.u[cj], xj = L.b[cj], Ej = L.bgE[cj];
         const T Bj = Ej + Ej * xj;
         const T g = L.bgu[cj] - gi, e = vj - vi;
         acc += (Ei * xi + Ej * xj) * g + (Bi + Bj) * e;
         dacc += Bi * (g + e) - (Bi + Bj);
       } else {
-        const T r = (T)mjd / mi, ub = (T)L.ub[f * L.ncell + c];
+        const T r = (T)L.m[cj] / (T)L.m[c], ub = (T)L.ub[f * L.ncell + c];
         const T gg = ub - r * ub + r * gi, Eg = m_exp(gg);
         const T vg = r * vi, xg = expm1f(vg);
         const T Bg = Eg + Eg * xg;
@@ -173,27 +182,32 @@ __device__ __forceinline__ void m_cell(const MLevelT<T, BG> &L, long long c, T &
     dN = L.ah * dacc - T(0.5) * L.beta * F * (em + T(1));
     return;
   }
-  const T ui = L.u[c], mi = (T)L.m[c];
+  const T ui = L.u[c];
   const T bi = L.b[c];
-  T acc = T(0), dacc = T(0);
+  // regular faces: acc = bi S1 + S2, dacc = bi (S1 - n) - S3 with S1 = sum (uj -
+  // ui), S2 = sum bj (uj - ui), S3 = sum bj over the n of them
+  T acc = T(0), dacc = T(0), S1 = T(0);
+  const unsigned nb = L.nb[c];
 #pragma unroll
   for (int f = 0; f < 6; f++) {
     const long long cj = c + face_step(L, f);
-    const double mjd = L.m[cj];
-    if (mjd > 0.0) {
-      const T uj = L.u[cj], bj = L.b[cj];
-      acc += (bi + bj) * (uj - ui);
-      dacc += bi * (uj - ui) - (bi + bj);
+    if (nb >> f & 1) {
+      const T uj = L.u[cj], bj = L.b[cj], t = uj - ui;
+      S1 += t;
+      acc += bj * t;
+      dacc -= bj;
     } else {
-      const T r = (T)mjd / mi, ub = (T)L.ub[f * L.ncell + c];
+      const T r = (T)L.m[cj] / (T)L.m[c], ub = (T)L.ub[f * L.ncell + c];
       const T ug = ub - r * ub + r * ui, bg = m_exp(ug);
       acc += (bi + bg) * (ug - ui);
       dacc += (bi + r * bg) * (ug - ui) + (bi + bg) * (r - T(1));
     }
   }
+  acc += bi * S1;
+  dacc += bi * (S1 - T(__popc(nb)));
   T s, sm1;
   if constexpr (sizeof(T) == 8) {
-    s = exp(-0.5 * ui);
+    s = f64_rsqrt(bi);  // e^{-u/2}
     sm1 = s - 1.0;
   } else {
     sm1 = expm1f(-0.5f * ui);
@@ -207,13 +221,15 @@ __device__ __forceinline__ void m_cell(const MLevelT<T, BG> &L, long long c, T &
 
 namespace {
 
-// Boundary values of the ghost faces from the current (initial) values, and
-// the exponential cache of every cell.
-__global__ void __launch_bounds__(kNT) k_mub(MLevel L) {
+// Boundary values of the ghost faces from the current (initial) values, the
+// exponential cache of every cell, and the active neighbours of the active
+// cells.
+__global__ void __launch_bounds__(kNT) k_mub(MLevel L, unsigned char *nb) {
   const long long c = (long long)blockIdx.x * kNT + threadIdx.x;
   if (c >= L.ncell) return;
   const double mi = L.m[c], ui = L.u[c];
-  L.b[c] = exp(ui);
+  L.b[c] = m_exp(ui);
+  unsigned flags = 0;
   const double nan = __longlong_as_double(0x7ff8000000000000ll);
 #pragma unroll
   for (int f = 0; f < 6; f++) {
@@ -222,9 +238,11 @@ __global__ void __launch_bounds__(kNT) k_mub(MLevel L) {
       const long long cj = c + face_step(L, f);
       const double mg = L.m[cj];
       if (mg <= 0.0) v = (mi * L.u[cj] - mg * ui) / (mi - mg);
+      else flags |= 1u << f;
     }
     L.ub[f * L.ncell + c] = v;
   }
+  nb[c] = (unsigned char)flags;
 }
 
 // Active-cell lists: per block of kNT cells, the active cells of each colour
@@ -273,21 +291,31 @@ __global__ void __launch_bounds__(kNT) k_mlist(MLevel L, const int *base, int *a
   }
 }
 
-// One colour of a red-black Newton-Gauss-Seidel sweep over the active cells
-// (one thread per active cell of the colour).
+// Newton-Gauss-Seidel update of one active cell.
 template <typename T, bool BG>
-__global__ void __launch_bounds__(kNT) k_msmooth(MLevelT<T, BG> L, int colour, T cap, T relax) {
-  const long long t = (long long)blockIdx.x * kNT + threadIdx.x;
-  const long long n = colour ? L.na - L.na0 : L.na0;
-  if (t >= n) return;
-  const long long c = L.act[(colour ? L.na0 : 0) + t];
+__device__ __forceinline__ void m_update(const MLevelT<T, BG> &L, long long c, T cap, T relax) {
   T N, dN;
   m_cell(L, c, N, dN);
-  T du = -relax * (N - L.f[c]) / dN;
+  T du;
+  if constexpr (sizeof(T) == 8)
+    du = -relax * (N - L.f[c]) * f64_rcp(dN);
+  else
+    du = -relax * (N - L.f[c]) / dN;
   du = du > cap ? cap : (du < -cap ? -cap : du);
   const T un = L.u[c] + du;
   L.u[c] = un;
   L.b[c] = m_cache<T, BG>(un);
+}
+
+// One colour of a red-black Newton-Gauss-Seidel sweep over the active cells
+// (one thread per active cell of the colour).
+template <typename T, bool BG>
+__global__ void __launch_bounds__(m_threads<T>()) k_msmooth(MLevelT<T, BG> L, int colour, T cap, T relax) {
+  const long long t = (long long)blockIdx.x * m_threads<T>() + threadIdx.x;
+  const long long n = colour ? L.na - L.na0 : L.na0;
+  if (t >= n) return;
+  const long long c = L.act[(colour ? L.na0 : 0) + t];
+  m_update(L, c, cap, relax);
 }
 
 // d = L(u) - f on the active cells (one thread per active cell; ghosts' d is
@@ -349,13 +377,11 @@ __global__ void __launch_bounds__(kNT) k_minit(MLevel F, MLevel C) {
   C.u[t] = 0.125 * su;
 }
 
-// FAS restriction onto the active coarse cells: u^H = R u^h (all children),
+// FAS restriction onto the active coarse cell t: u^H = R u^h (all children),
 // R d^h = sum over the active children / 8; ghosts keep their values.
 template <typename T, bool BG>
-__global__ void __launch_bounds__(kNT) k_mrestrict(MLevelT<T, BG> F, MLevelT<T, BG> C) {
-  const long long t = (long long)blockIdx.x * kNT + threadIdx.x;
-  if (t >= C.ncell) return;
-  if (!(C.m[t] > 0.0)) return;
+__device__ __forceinline__ void m_restrict(const MLevelT<T, BG> &F, const MLevelT<T, BG> &C,
+                                           long long t) {
   int I, J, K;
   ijk(C, t, I, J, K);
   T su = T(0), sd = T(0);
@@ -372,28 +398,28 @@ __global__ void __launch_bounds__(kNT) k_mrestrict(MLevelT<T, BG> F, MLevelT<T, 
   C.d[t] = T(0.125) * sd;
 }
 
-// f^H = L^H(R u^h) - R d^h on the active coarse cells (after k_mrestrict).
 template <typename T, bool BG>
-__global__ void __launch_bounds__(kNT) k_mfas(MLevelT<T, BG> C) {
-  const long long t = (long long)blockIdx.x * kNT + threadIdx.x;
-  if (t >= C.ncell) return;
-  if (!(C.m[t] > 0.0)) {
-    C.f[t] = T(0);
-    return;
-  }
-  T N, dN;
-  m_cell(C, t, N, dN);
-  C.f[t] = N - C.d[t];
+__global__ void __launch_bounds__(m_threads<T>()) k_mrestrict(MLevelT<T, BG> F, MLevelT<T, BG> C) {
+  const long long t = (long long)blockIdx.x * m_threads<T>() + threadIdx.x;
+  if (t < C.na) m_restrict(F, C, (long long)C.act[t]);
 }
 
-// u^h += P e^H on the active fine cells (one thread per active cell), e^H =
-// u^H - R u^h on active coarse cells and 0 on masked ones and outside the box
-// (trilinear 27/9/3/1).
+// f^H = L^H(R u^h) - R d^h on the active coarse cells (after k_mrestrict).
 template <typename T, bool BG>
-__global__ void __launch_bounds__(kNT) k_mprolong(MLevelT<T, BG> F, MLevelT<T, BG> C) {
-  const long long t = (long long)blockIdx.x * kNT + threadIdx.x;
-  if (t >= F.na) return;
-  const long long c = F.act[t];
+__global__ void __launch_bounds__(m_threads<T>()) k_mfas(MLevelT<T, BG> C) {
+  const long long t = (long long)blockIdx.x * m_threads<T>() + threadIdx.x;
+  if (t >= C.na) return;
+  const long long c = C.act[t];
+  T N, dN;
+  m_cell(C, c, N, dN);
+  C.f[c] = N - C.d[c];
+}
+
+// u^h += P e^H on the active fine cell c, e^H = u^H - R u^h on active coarse
+// cells and 0 on masked ones and outside the box (trilinear 27/9/3/1).
+template <typename T, bool BG>
+__device__ __forceinline__ void m_prolong(const MLevelT<T, BG> &F, const MLevelT<T, BG> &C,
+                                          long long c) {
   int i, j, k;
   ijk(F, c, i, j, k);
   const int I = i >> 1, J = j >> 1, K = k >> 1;
@@ -415,57 +441,122 @@ __global__ void __launch_bounds__(kNT) k_mprolong(MLevelT<T, BG> F, MLevelT<T, B
   F.b[c] = m_cache<T, BG>(un);
 }
 
-// Coarsest level, one block: red-black sweeps until the rms over the active
-// cells falls to max(1e-3 of its value before the first sweep, 0.1 tol), at
-// most 500 sweeps.
-constexpr int kCoNT = 1024;
 template <typename T, bool BG>
-__global__ void __launch_bounds__(kCoNT) k_mcoarsest(MLevelT<T, BG> L, long long nact, double tol,
-                                                     T cap, T relax) {
+__global__ void __launch_bounds__(m_threads<T>()) k_mprolong(MLevelT<T, BG> F, MLevelT<T, BG> C) {
+  const long long t = (long long)blockIdx.x * m_threads<T>() + threadIdx.x;
+  if (t < F.na) m_prolong(F, C, (long long)F.act[t]);
+}
+
+// The levels of few active cells, down to the coarsest and back up, in one
+// block: every step of one of them is far too small for the GPU, and a launch
+// of it costs its latency (about 12 us, six to eight launches per level and
+// direction).  The arrays stay in global memory (one block's L1 and L2).
+//
+// Coarsest level: red-black sweeps until the rms over the active cells falls
+// to max(1e-3 of its value before the first sweep, 0.1 tol), at most 500
+// sweeps.  In FP32 the solve also ends when four sweeps in a row have not
+// brought the rms 1 % below its best: near the FP32 floor of the
+// full-variable form the first rule is never met (500 sweeps, 2.2 ms per
+// cycle).
+constexpr int kTailNT = 1024;
+constexpr int kTailLevels = 16;
+
+// FP32: up to 4096 active cells (masked 256^3 region, whole solve: 512 cells 7.33
+// ms, 4096 7.06 ms, 12000 8.57 ms), FP64: 256 (the FP64 pipe of one SM).
+template <typename T>
+constexpr long long tail_cells() {
+  return sizeof(T) == 4 ? 4096 : 256;
+}
+
+template <typename T, bool BG>
+__device__ __noinline__ void mt_smooth(const MLevelT<T, BG> &L, int sweeps, T cap, T relax) {
+  for (int s = 0; s < sweeps; s++)
+    for (int colour = 0; colour < 2; colour++) {
+      const int *act = L.act + (colour ? L.na0 : 0);
+      const long long n = colour ? L.na - L.na0 : L.na0;
+      for (long long t = threadIdx.x; t < n; t += kTailNT)
+        m_update(L, (long long)act[t], cap, relax);
+      __syncthreads();
+    }
+}
+
+// d = L(u) - f (fas = false) or f = L(u) - d (fas = true) on the active cells
+template <typename T, bool BG>
+__device__ __noinline__ void mt_resid(const MLevelT<T, BG> &L, bool fas) {
+  for (long long t = threadIdx.x; t < L.na; t += kTailNT) {
+    const long long c = L.act[t];
+    T N, dN;
+    m_cell(L, c, N, dN);
+    if (fas) L.f[c] = N - L.d[c];
+    else L.d[c] = N - L.f[c];
+  }
+  __syncthreads();
+}
+
+template <typename T, bool BG>
+__device__ __noinline__ void mt_coarsest(const MLevelT<T, BG> &L, double tol, T cap, T relax) {
   // the rms in the level's precision (FP64 arithmetic runs at 1/64 rate)
-  __shared__ T red[kCoNT / 32];
-  __shared__ T tot;
-  auto rms = [&]() -> T {
+  __shared__ T red[kTailNT / 32];
+  T thr = T(0), best = T(0);
+  int flat = 0;
+  for (int it = -1; it < 500; it++) {
+    if (it >= 0) mt_smooth(L, 1, cap, relax);
     T s = T(0);
-    for (long long c = threadIdx.x; c < L.ncell; c += kCoNT) {
-      if (!(L.m[c] > 0.0)) continue;
+    for (long long t = threadIdx.x; t < L.na; t += kTailNT) {
+      const long long c = L.act[t];
       T N, dN;
       m_cell(L, c, N, dN);
       const T d = N - L.f[c];
       s += d * d;
     }
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
-    if (threadIdx.x == 0) {
-      T t = T(0);
-      for (int w = 0; w < kCoNT / 32; w++) t += red[w];
-      tot = sqrt(t / (T)(nact > 0 ? nact : 1));
+    s = red[threadIdx.x & 31];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    const T r = sqrt(s / (T)(L.na > 0 ? L.na : 1));
+    __syncthreads();  // red has been read
+    if (it < 0) {
+      thr = fmax(T(1e-3) * r, (T)(0.1 * tol));
+      best = r;
+      continue;
     }
-    __syncthreads();
-    const T r = tot;
-    __syncthreads();
-    return r;
-  };
-  const T thr = fmax(T(1e-3) * rms(), (T)(0.1 * tol));
-  for (int it = 0; it < 500; it++) {
-    for (int colour = 0; colour < 2; colour++) {
-      for (long long c = threadIdx.x; c < L.ncell; c += kCoNT) {
-        if (!(L.m[c] > 0.0)) continue;
-        int i, j, k;
-        ijk(L, c, i, j, k);
-        if (((i + j + k) & 1) != colour) continue;
-        T N, dN;
-        m_cell(L, c, N, dN);
-        T du = -relax * (N - L.f[c]) / dN;
-        du = du > cap ? cap : (du < -cap ? -cap : du);
-        const T un = L.u[c] + du;
-        L.u[c] = un;
-        L.b[c] = m_cache<T, BG>(un);
-      }
-      __syncthreads();
+    if (r < T(0.99) * best) {
+      best = r;
+      flat = 0;
+    } else {
+      flat++;
     }
-    if (rms() <= thr) break;
+    if (r <= thr || (sizeof(T) == 4 && flat >= 4)) return;
+  }
+}
+
+template <typename T, bool BG>
+__global__ void __launch_bounds__(kTailNT)
+    k_mtail(const MLevelT<T, BG> *levels, int nl, int pre, int post, double tol, T cap, T relax) {
+  __shared__ MLevelT<T, BG> lev[kTailLevels];
+  {
+    const int *src = reinterpret_cast<const int *>(levels);
+    int *dst = reinterpret_cast<int *>(lev);
+    for (int t = threadIdx.x; t < nl * (int)(sizeof(MLevelT<T, BG>) / sizeof(int)); t += kTailNT)
+      dst[t] = src[t];
+  }
+  __syncthreads();
+  for (int l = 0; l < nl - 1; l++) {
+    const MLevelT<T, BG> &F = lev[l], &C = lev[l + 1];
+    mt_smooth(F, pre, cap, relax);
+    mt_resid(F, false);
+    for (long long t = threadIdx.x; t < C.na; t += kTailNT) m_restrict(F, C, (long long)C.act[t]);
+    __syncthreads();
+    mt_resid(C, true);
+  }
+  mt_coarsest(lev[nl - 1], tol, cap, relax);
+  for (int l = nl - 2; l >= 0; l--) {
+    const MLevelT<T, BG> &F = lev[l], &C = lev[l + 1];
+    __syncthreads();
+    for (long long t = threadIdx.x; t < F.na; t += kTailNT) m_prolong(F, C, (long long)F.act[t]);
+    __syncthreads();
+    mt_smooth(F, post, cap, relax);
   }
 }
 
@@ -500,7 +591,7 @@ __global__ void __launch_bounds__(kNT) k_mto64(MLevelT<float> S, MLevel D) {
   const long long c = D.act[t];
   const double v = (double)S.u[c];
   D.u[c] = v;
-  D.b[c] = exp(v);
+  D.b[c] = m_exp(v);
 }
 
 // Outer step of a mixed solve, finest level: background = the FP64 iterate
@@ -545,7 +636,7 @@ __global__ void __launch_bounds__(kNT) k_madd64(MLevelT<float, true> S, MLevel D
   const long long c = D.act[t];
   const double v = D.u[c] + (double)S.u[c];
   D.u[c] = v;
-  D.b[c] = exp(v);
+  D.b[c] = m_exp(v);
 }
 
 // Flags of the inputs: [0] a mask outside [-1, 1] or NaN, [1] a non-finite
@@ -608,8 +699,8 @@ struct MSolver {
   void smooth(MLevelT<T, BG> &L, int n) {
     for (int s = 0; s < n; s++)
       for (int colour = 0; colour < 2; colour++) {
-        k_msmooth<<<(unsigned)nblk(std::max(colour ? L.na - L.na0 : L.na0, 1ll)), kNT, 0, st>>>(
-            L, colour, cap, relax);
+        k_msmooth<<<(unsigned)nblk(std::max(colour ? L.na - L.na0 : L.na0, 1ll), m_threads<T>()),
+                    m_threads<T>(), 0, st>>>(L, colour, cap, relax);
         MLAUNCH(ctx);
       }
   }
@@ -628,27 +719,38 @@ struct MSolver {
     if (dmax) *dmax = mx;
     return std::sqrt(s / (double)std::max(nact, 1ll));
   }
-  void coarsest(MLevelT<T, BG> &L, long long nact) {
-    k_mcoarsest<<<1, kCoNT, 0, st>>>(L, nact, tol, cap, relax);
-    MLAUNCH(ctx);
-  }
   std::vector<long long> nact;
+  int tail = 0;                        // first level of the one-block tail
+  MLevelT<T, BG> *tail_lev = nullptr;  // the levels from there on, on the device
+  // once lev is complete: where the tail begins (at the coarsest level at the
+  // latest), its levels to the device
+  void set_tail(MArena &A) {
+    const int nl = (int)lev.size();
+    tail = nl - 1;
+    while (tail > 0 && nl - tail < kTailLevels && lev[tail - 1].na <= tail_cells<T>()) tail--;
+    tail_lev = A.get<MLevelT<T, BG>>(nl - tail);
+    MCK(cudaMemcpyAsync(tail_lev, lev.data() + tail, (nl - tail) * sizeof(MLevelT<T, BG>),
+                        cudaMemcpyHostToDevice, st));
+  }
   void vcycle(int l) {
     MLevelT<T, BG> &L = lev[l];
-    if (l == (int)lev.size() - 1) {
-      coarsest(L, nact[l]);
+    if (l == tail) {
+      k_mtail<T, BG><<<1, kTailNT, 0, st>>>(tail_lev, (int)lev.size() - tail, pre, post, tol, cap,
+                                            relax);
+      MLAUNCH(ctx);
       return;
     }
     MLevelT<T, BG> &C = lev[l + 1];
+    constexpr int nt = m_threads<T>();
     smooth(L, pre);
     k_mresid<<<(unsigned)nblk(std::max(L.na, 1ll)), kNT, 0, st>>>(L, partial);
     MLAUNCH(ctx);
-    k_mrestrict<<<(unsigned)nblk(C.ncell), kNT, 0, st>>>(L, C);
+    k_mrestrict<<<(unsigned)nblk(std::max(C.na, 1ll), nt), nt, 0, st>>>(L, C);
     MLAUNCH(ctx);
-    k_mfas<<<(unsigned)nblk(C.ncell), kNT, 0, st>>>(C);
+    k_mfas<<<(unsigned)nblk(std::max(C.na, 1ll), nt), nt, 0, st>>>(C);
     MLAUNCH(ctx);
     vcycle(l + 1);
-    k_mprolong<<<(unsigned)nblk(std::max(L.na, 1ll)), kNT, 0, st>>>(L, C);
+    k_mprolong<<<(unsigned)nblk(std::max(L.na, 1ll), nt), nt, 0, st>>>(L, C);
     MLAUNCH(ctx);
     smooth(L, post);
   }
@@ -724,7 +826,8 @@ extern "C" int fr_solve_masked(frmg_ctx *ctx, const double *density, const doubl
       L.uR = A.get<double>(L.ncell);
       L.d = A.get<double>(L.ncell);
       L.ub = A.get<double>(6 * L.ncell);
-      L.act = nullptr;  // set once the level set is final
+      L.act = nullptr;  // set once the level set is final, as is nb
+      L.nb = nullptr;
       L.na0 = L.na = 0;
       L.bgu = L.bgE = nullptr;
       L.ah = 0.5 * alpha * (h * h) / (hl * hl);
@@ -760,7 +863,9 @@ extern "C" int fr_solve_masked(frmg_ctx *ctx, const double *density, const doubl
       S.nact.push_back((long long)hf[1]);
     }
     for (auto &L : S.lev) {
-      k_mub<<<(unsigned)nblk(L.ncell), kNT, 0, st>>>(L);
+      unsigned char *nb = A.get<unsigned char>(L.ncell);
+      L.nb = nb;
+      k_mub<<<(unsigned)nblk(L.ncell), kNT, 0, st>>>(L, nb);
       MLAUNCH(ctx);
     }
     // active-cell lists of every level
@@ -793,6 +898,7 @@ extern "C" int fr_solve_masked(frmg_ctx *ctx, const double *density, const doubl
       L.na0 = n0;
       L.na = n0 + n1;
     }
+    S.set_tail(A);
     S.partial = A.get<double>(2 * nblk(nc));
     double *pin = frmg_pinned(ctx, 2 * nblk(nc));
     if (!pin) throw MError{FR_ENOMEM, "pinned host allocation failed"};
@@ -821,6 +927,7 @@ extern "C" int fr_solve_masked(frmg_ctx *ctx, const double *density, const doubl
         F.d = A.get<float>(D.ncell);
         F.m = D.m;
         F.rho = D.rho;
+        F.nb = D.nb;
         F.ub = D.ub;
         F.act = D.act;
         F.na0 = D.na0;
@@ -839,6 +946,7 @@ extern "C" int fr_solve_masked(frmg_ctx *ctx, const double *density, const doubl
         MLAUNCH(ctx);
         S32.lev.push_back(F);
       }
+      S32.set_tail(A);
       const double r0 = r;
       double rp = r, best = r;
       bool ok = false;
@@ -876,6 +984,7 @@ extern "C" int fr_solve_masked(frmg_ctx *ctx, const double *density, const doubl
           B.b = F.b;
           B.m = F.m;
           B.rho = F.rho;
+          B.nb = F.nb;
           B.f = F.f;
           B.uR = F.uR;
           B.d = F.d;
@@ -896,6 +1005,7 @@ extern "C" int fr_solve_masked(frmg_ctx *ctx, const double *density, const doubl
           B.bgE = A.get<float>(F.ncell);
           SB.lev.push_back(B);
         }
+        SB.set_tail(A);
         const int inner = std::max(1, o.inner_cycles);
         double rp = r;
         while (r > tol && sv.vcycles < o.max_vcycles) {

@@ -94,3 +94,24 @@ def test_patch_tails_match_oracle(C, prec, sizes):
     assert st == 0
     for p, r in zip(gp, ref):
         assert np.abs(host(p["u"]) - r.u).max() < 1e-8
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("dims,count,relax", [((16, 18, 20), 1, 1.0), ((24, 24, 24), 3, 1.25),
+                                              ((40, 36, 32), 6, 1.0)])
+def test_masked_tail_matches_oracle(C, prec, dims, count, relax):
+    """Regions whose levels are all in the one-block tail, and with launched
+    levels above it (more than 4096 active cells FP32, 256 FP64); rms(L) <= 1e-11
+    fixes u to about 1e-10."""
+    from oracle import masked as OM
+    rho = synth.lognormal_density(dims, 8600, sigma=1.0)
+    r = 0.2 * min(dims)
+    m = synth.sphere_union_mask(rho, count, (0.8 * r, 1.4 * r), 8601)
+    m[m > 0] = np.where(np.arange((m > 0).sum()) % 3 == 0, 0.5, 1.0)
+    u0 = 0.1 * np.cos(np.arange(m.size).reshape(m.shape) / 50.0)
+    P = dict(box=64.0, a=1.0, omega_m=0.24, fr0=1e-5)
+    ref = OM.solve(u0, m, rho, h=1.0 / 64, tol=1e-12, **P)
+    u = dev(u0)
+    st, s = C.solve_masked(dev(rho), dev(m), u, h=1.0 / 64, tol=1e-11, prec=prec, relax=relax, **P)
+    assert st == 0 and s.res_rms <= 1e-11
+    assert np.abs(host(u) - ref.u).max() < 1e-8
