@@ -24,10 +24,25 @@ struct DFGrid {
   float gah, gal;        // gamma
 };
 
+// One grid of a batch: its state and its FP32 arrays (Grid, finest level).
+struct DFJob {
+  DFGrid g;
+  double *u64;
+  const double *rho;
+  float *f, *bgu, *bgE;
+  float *u[2], *x[2];
+  int field, check_rho;
+};
+
+// Every step below exists for one grid (its description in the kernel's
+// parameters) and, as k_..._many, for all grids of a batch in one launch: block
+// b works on the grid whose range of off holds it, 256 cells per block.  (One
+// launch per grid cost 12 to 20 us each on grids of 32 to 64 cells a side.)
+
 // State set-up: u (FP64, or zero), e^u and gamma (rho - 1) as double-float.
-__global__ void k_df_init(DFGrid G, const double *u64, const double *rho, int zero_u,
-                          float ln2h, float ln2l) {
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void df_init(const DFGrid &G, const double *u64, const double *rho,
+                                        int zero_u, float ln2h, float ln2l, long long blk) {
+  long long t = blk * 256 + threadIdx.x;
   if (t >= G.ncell) return;
   df u = zero_u ? df{0.f, 0.f} : split_bits(u64[t]);
   G.u[t] = make_float2(u.h, u.l);
@@ -36,6 +51,17 @@ __global__ void k_df_init(DFGrid G, const double *u64, const double *rho, int ze
   const df r = df_mul(df_add_f(split_bits(rho[t]), -1.0f), df{G.gah, G.gal});
   G.r[t] = make_float2(r.h, r.l);
 }
+__global__ void __launch_bounds__(256) k_df_init(DFGrid G, const double *u64, const double *rho,
+                                                 int zero_u, float ln2h, float ln2l) {
+  df_init(G, u64, rho, zero_u, ln2h, ln2l, blockIdx.x);
+}
+__global__ void __launch_bounds__(256)
+    k_df_init_many(const DFJob *jobs, const int *off, int nj, int zero_u, float ln2h,
+                   float ln2l) {
+  const int j = find_grid(off, nj, blockIdx.x);
+  const DFGrid G = jobs[j].g;
+  df_init(G, jobs[j].u64, jobs[j].rho, zero_u, ln2h, ln2l, blockIdx.x - off[j]);
+}
 
 // u += delta and e^u, two cells (an x-pair) per thread.  For |delta| < 2^-5
 // (the correction steps) e^u is the old e^u times e^delta, e^delta by its
@@ -43,9 +69,9 @@ __global__ void k_df_init(DFGrid G, const double *u64, const double *rho, int ze
 // 8!, far under the pair's rounding), on packed FP32 pairs, when every cell
 // of the warp takes it; otherwise (the first update after the full-variable
 // phase) e^u is recomputed from u.
-__global__ void __launch_bounds__(128) k_df_update(DFGrid G, const float *delta, float ln2h,
-                                                   float ln2l) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void df_update(const DFGrid &G, const float *delta, float ln2h,
+                                          float ln2l, long long blk) {
+  const long long t = blk * 128 + threadIdx.x;
   const bool in = t < (G.ncell >> 1);
   float4 *U4 = reinterpret_cast<float4 *>(G.u);
   float4 *B4 = reinterpret_cast<float4 *>(G.B);
@@ -85,12 +111,34 @@ __global__ void __launch_bounds__(128) k_df_update(DFGrid G, const float *delta,
   }
   B4[t] = Bn;
 }
+__global__ void __launch_bounds__(128) k_df_update(DFGrid G, const float *delta, float ln2h,
+                                                   float ln2l) {
+  df_update(G, delta, ln2h, ln2l, blockIdx.x);
+}
+// the active fields; their corrections lie in the buffers par[field]
+__global__ void __launch_bounds__(128)
+    k_df_update_many(const DFJob *jobs, const int *off, int nj, const int *active,
+                     const int *par, float ln2h, float ln2l) {
+  const int j = find_grid(off, nj, blockIdx.x);
+  const int field = jobs[j].field;
+  if (!active[field]) return;
+  const DFGrid G = jobs[j].g;
+  df_update(G, jobs[j].u[par[field]], ln2h, ln2l, blockIdx.x - off[j]);
+}
 
-__global__ void k_df_final(DFGrid G, double *u64) {
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void df_final(const DFGrid &G, double *u64, long long blk) {
+  long long t = blk * 256 + threadIdx.x;
   if (t >= G.ncell) return;
   const float2 v = G.u[t];
   u64[t] = join_bits(v.x, v.y);
+}
+__global__ void __launch_bounds__(256) k_df_final(DFGrid G, double *u64) {
+  df_final(G, u64, blockIdx.x);
+}
+__global__ void __launch_bounds__(256) k_df_final_many(const DFJob *jobs, const int *off, int nj) {
+  const int j = find_grid(off, nj, blockIdx.x);
+  const DFGrid G = jobs[j].g;
+  df_final(G, jobs[j].u64, blockIdx.x - off[j]);
 }
 
 // FP64-accurate defect d = A(u) - gamma (rho - 1) of the fine grid in
@@ -104,10 +152,10 @@ __global__ void k_df_final(DFGrid G, double *u64) {
 // first face initialises the sums (adding a normalised pair to zero returns
 // it).  256 cells per block of 128 threads.
 template <bool BIG>
-__global__ void __launch_bounds__(128)
-    k_df_defect(DFGrid G, float *r32, float *ub32, float *E32, float *delta, float *x32,
-                 double *partial, int base, float ln2h, float ln2l, double *dout = nullptr) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void df_defect(const DFGrid &G, float *r32, float *ub32, float *E32,
+                                          float *delta, float *x32, double *partial, float ln2h,
+                                          float ln2l, double *dout, long long blk) {
+  const long long t = blk * 128 + threadIdx.x;
   const long long np = G.ncell >> 1;
   float s2 = 0.0f, mx = 0.0f;
   if (t < np) {
@@ -223,8 +271,26 @@ __global__ void __launch_bounds__(128)
     s2 = fmaf(dv.y, dv.y, dv.x * dv.x);
     mx = fmaxf(fabsf(dv.x), fabsf(dv.y));
   }
-  block_reduce2f<128>(s2, mx, &partial[2 * (base + blockIdx.x)],
-                      &partial[2 * (base + blockIdx.x) + 1]);
+  block_reduce2f<128>(s2, mx, &partial[0], &partial[1]);
+}
+template <bool BIG>
+__global__ void __launch_bounds__(128)
+    k_df_defect(DFGrid G, float *r32, float *ub32, float *E32, float *delta, float *x32,
+                 double *partial, int base, float ln2h, float ln2l, double *dout = nullptr) {
+  df_defect<BIG>(G, r32, ub32, E32, delta, x32, partial + 2 * ((long long)base + blockIdx.x),
+                 ln2h, ln2l, dout, blockIdx.x);
+}
+// the active fields; par: the current buffer of the FP32 finest levels
+template <bool BIG>
+__global__ void __launch_bounds__(128)
+    k_df_defect_many(const DFJob *jobs, const int *off, int nj, const int *active, int par,
+                     double *partial, float ln2h, float ln2l) {
+  const int j = find_grid(off, nj, blockIdx.x);
+  const DFJob &J = jobs[j];
+  if (!active[J.field]) return;
+  const DFGrid G = J.g;
+  df_defect<BIG>(G, J.f, J.bgu, J.bgE, J.u[par], J.x[par], partial + 2 * (long long)blockIdx.x,
+                 ln2h, ln2l, nullptr, blockIdx.x - off[j]);
 }
 
 }  // namespace frmg

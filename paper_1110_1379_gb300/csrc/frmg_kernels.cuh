@@ -1133,6 +1133,28 @@ __global__ void k_restrict_avg(const T *fine, int nf0, int nf1, int nf2, T *coar
   coarse[t] = s * T(0.125);
 }
 
+// Background of the correction form on a level from the next finer one: mean
+// of the 8 children and its exponential, for every active grid of the set.
+__global__ void __launch_bounds__(256)
+    k_bg_restrict(const Grid<float> *fine, const Grid<float> *coarse, const int *off, int ngrid,
+                  const int *active) {
+  const int g = find_grid(off, ngrid, blockIdx.x);
+  const Grid<float> &F = fine[g];
+  const Grid<float> &C = coarse[g];
+  if (!grid_active(active, F.field)) return;
+  const long long t = (long long)(blockIdx.x - off[g]) * 256 + threadIdx.x;
+  if (t >= C.ncell) return;
+  int I, J, K;
+  cell_ijk(C, t, I, J, K);
+  float s = 0.0f;
+#pragma unroll
+  for (int q = 0; q < 8; q++)
+    s += F.ubg[idx3(F, 2 * I + (q & 1), 2 * J + ((q >> 1) & 1), 2 * K + (q >> 2))];
+  const float ub = s * 0.125f;
+  const_cast<float *>(C.ubg)[t] = ub;
+  const_cast<float *>(C.Ebg)[t] = expf(ub);
+}
+
 // ---------------------------------------------------------------------------
 // Tiled FP32 smoother with temporal blocking: S full red-black sweeps per pass.
 //

@@ -362,6 +362,15 @@ __global__ void k_any_nonzero(const double *u, long long n, int *flag) {
   if (__any_sync(0xffffffffu, nz) && (threadIdx.x & 31) == 0) *flag = 1;
 }
 
+// The same over all grids of a batch (block ranges off, 256 cells per block).
+__global__ void k_any_nonzero_many(const DFJob *jobs, const int *off, int nj, int *flag) {
+  const int j = find_grid(off, nj, blockIdx.x);
+  const long long t = (long long)(blockIdx.x - off[j]) * 256 + threadIdx.x;
+  const bool nz = t < jobs[j].g.ncell &&
+                  ((unsigned long long)__double_as_longlong(jobs[j].u64[t]) << 1) != 0;
+  if (__any_sync(0xffffffffu, nz) && (threadIdx.x & 31) == 0) *flag = 1;
+}
+
 // n doubles from device memory to page-locked host memory written by the
 // kernel itself (a zero-copy read-back that does not wait behind copies
 // queued on the copy engines).
@@ -1968,10 +1977,9 @@ static void solve_mixed(frmg_ctx *ctx, std::vector<Problem> &P, const SolveCfg &
 
 // Zero-start set-up of the double-float loop: the FP32 right-hand side is the
 // high part of gamma (rho - 1); block partials of its norm as k_prep_zero.
-__global__ void __launch_bounds__(256) k_prep_zero_df(const float2 *rv, float *r32, float *u32,
-                                                      float *x32, long long n, double *partial,
-                                                      int base) {
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void prep_zero_df(const float2 *rv, float *r32, float *u32, float *x32,
+                                             long long n, double *partial, long long blk) {
+  long long t = blk * 256 + threadIdx.x;
   float s = 0.0f, m = 0.0f;
   if (t < n) {
     float r = rv[t].x;
@@ -1981,7 +1989,11 @@ __global__ void __launch_bounds__(256) k_prep_zero_df(const float2 *rv, float *r
     s = r * r;
     m = fabsf(r);
   }
-  block_reduce2f<256>(s, m, &partial[2 * (base + blockIdx.x)], &partial[2 * (base + blockIdx.x) + 1]);
+  block_reduce2f<256>(s, m, &partial[0], &partial[1]);
+}
+__global__ void __launch_bounds__(256) k_prep_zero_df(const float2 *rv, float *r32, float *u32,
+                                                      float *x32, long long n, double *partial) {
+  prep_zero_df(rv, r32, u32, x32, n, partial + 2 * (long long)blockIdx.x, blockIdx.x);
 }
 
 // Zero start of the double-float state and of the FP32 full-variable phase in
@@ -1990,10 +2002,10 @@ __global__ void __launch_bounds__(256) k_prep_zero_df(const float2 *rv, float *r
 // residual of u = 0).  Equals k_df_init with zero_u followed by k_prep_zero_df.
 // check_rho > 0: also the density validation of k_check_density (negative
 // values allowed if 2), flagged in *bad.
-__global__ void __launch_bounds__(256) k_df_init_zero(DFGrid G, const double *rho, float *r32,
-                                                      float *u32, float *x32, double *partial,
-                                                      int base, int check_rho, int *bad) {
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void df_init_zero(const DFGrid &G, const double *rho, float *r32,
+                                             float *u32, float *x32, double *partial,
+                                             int check_rho, int *bad, long long blk) {
+  long long t = blk * 256 + threadIdx.x;
   float s = 0.0f, m = 0.0f;
   if (t < G.ncell) {
     if (check_rho > 0) {
@@ -2012,8 +2024,32 @@ __global__ void __launch_bounds__(256) k_df_init_zero(DFGrid G, const double *rh
     s = r.h * r.h;
     m = fabsf(r.h);
   }
-  block_reduce2f<256>(s, m, &partial[2 * (base + blockIdx.x)], &partial[2 * (base + blockIdx.x) + 1]);
+  block_reduce2f<256>(s, m, &partial[0], &partial[1]);
 }
+__global__ void __launch_bounds__(256) k_df_init_zero(DFGrid G, const double *rho, float *r32,
+                                                      float *u32, float *x32, double *partial,
+                                                      int check_rho, int *bad) {
+  df_init_zero(G, rho, r32, u32, x32, partial + 2 * (long long)blockIdx.x, check_rho, bad,
+               blockIdx.x);
+}
+__global__ void __launch_bounds__(256)
+    k_df_init_zero_many(const DFJob *jobs, const int *off, int nj, int par, double *partial,
+                        int *bad) {
+  const int j = find_grid(off, nj, blockIdx.x);
+  const DFJob &J = jobs[j];
+  const DFGrid G = J.g;
+  df_init_zero(G, J.rho, J.f, J.u[par], J.x[par], partial + 2 * (long long)blockIdx.x,
+               J.check_rho, bad, blockIdx.x - off[j]);
+}
+// k_prep_zero_df of every grid of a batch
+__global__ void __launch_bounds__(256)
+    k_prep_zero_df_many(const DFJob *jobs, const int *off, int nj, int par, double *partial) {
+  const int j = find_grid(off, nj, blockIdx.x);
+  const DFJob &J = jobs[j];
+  prep_zero_df(J.g.r, J.f, J.u[par], J.x[par], J.g.ncell, partial + 2 * (long long)blockIdx.x,
+               blockIdx.x - off[j]);
+}
+
 
 static void split_host(double v, float &h, float &l) {
   h = (float)v;
@@ -2077,6 +2113,35 @@ static void solve_mixed_df(frmg_ctx *ctx, std::vector<Problem> &P, const SolveCf
   double *red = S.get<double>(2 * (size_t)np);
   int *d_boff = S.get<int>(np + 1);
   CK(cudaMemcpyAsync(d_boff, boff.data(), (np + 1) * sizeof(int), cudaMemcpyHostToDevice, st));
+  // the fine-grid steps of a batch take all its grids in one launch
+  const bool many = np > 1;
+  bool wide = false;  // a grid of 2^31 cells or more
+  DFJob *jobs = nullptr;
+  int *d_fpar = nullptr;
+  if (many) {
+    std::vector<DFJob> hj(np);
+    for (int pi = 0; pi < np; pi++) {
+      const Grid<float> &G = H.lev[pi][0];
+      DFJob &j = hj[pi];
+      j.g = D[pi];
+      j.u64 = P[pi].u;
+      j.rho = P[pi].rho;
+      j.f = const_cast<float *>(G.f);
+      j.bgu = H.bg_u[pi];
+      j.bgE = H.bg_E[pi];
+      j.u[0] = G.u;
+      j.u[1] = G.u2;
+      j.x[0] = G.x;
+      j.x[1] = G.x2;
+      j.field = pi;
+      j.check_rho = P[pi].check_rho;
+      wide = wide || D[pi].ncell >= (1ll << 31);
+    }
+    jobs = S.get<DFJob>(np);
+    d_fpar = S.get<int>(np);
+    CK(cudaMemcpyAsync(jobs, hj.data(), np * sizeof(DFJob), cudaMemcpyHostToDevice, st));
+    CK(cudaStreamSynchronize(st));  // hj has been read
+  }
   // a zero start that the caller declared (initial_guess = 0) reads no u and
   // sets the state up in one fused pass below; otherwise u is scanned for a
   // non-zero value
@@ -2088,18 +2153,20 @@ static void solve_mixed_df(frmg_ctx *ctx, std::vector<Problem> &P, const SolveCf
   if (!zero_start) {
     int *flag = S.get<int>(1);
     CK(cudaMemsetAsync(flag, 0, sizeof(int), st));
-    for (int pi = 0; pi < np; pi++) {
-      k_any_nonzero<<<nblocks(D[pi].ncell), 256, 0, st>>>(P[pi].u, D[pi].ncell, flag);
-      CK_LAUNCH(ctx);
-    }
+    if (many)
+      k_any_nonzero_many<<<boff[np], 256, 0, st>>>(jobs, d_boff, np, flag);
+    else
+      k_any_nonzero<<<nblocks(D[0].ncell), 256, 0, st>>>(P[0].u, D[0].ncell, flag);
+    CK_LAUNCH(ctx);
     CK(cudaMemcpyAsync(&nonzero, flag, sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    for (int pi = 0; pi < np; pi++) {
-      PROF("df_init");
-      k_df_init<<<nblocks(D[pi].ncell), 256, 0, st>>>(D[pi], P[pi].u, P[pi].rho, !nonzero, ln2h,
-                                                      ln2l);
-      CK_LAUNCH(ctx);
-    }
+    PROF("df_init");
+    if (many)
+      k_df_init_many<<<boff[np], 256, 0, st>>>(jobs, d_boff, np, !nonzero, ln2h, ln2l);
+    else
+      k_df_init<<<nblocks(D[0].ncell), 256, 0, st>>>(D[0], P[0].u, P[0].rho, !nonzero, ln2h,
+                                                     ln2l);
+    CK_LAUNCH(ctx);
   }
   const int bnch = red_chunks(boff);
   double *btmp = bnch ? S.get<double>(2 * (size_t)bnch * np) : nullptr;
@@ -2126,10 +2193,11 @@ static void solve_mixed_df(frmg_ctx *ctx, std::vector<Problem> &P, const SolveCf
     }
   };
   auto finalize = [&]() {
-    for (int pi = 0; pi < np; pi++) {
-      k_df_final<<<nblocks(D[pi].ncell), 256, 0, st>>>(D[pi], P[pi].u);
-      CK_LAUNCH(ctx);
-    }
+    if (many)
+      k_df_final_many<<<boff[np], 256, 0, st>>>(jobs, d_boff, np);
+    else
+      k_df_final<<<nblocks(D[0].ncell), 256, 0, st>>>(D[0], P[0].u);
+    CK_LAUNCH(ctx);
   };
   int *active = S.get<int>(np);
   std::vector<int> act(np, 1);
@@ -2156,12 +2224,15 @@ static void solve_mixed_df(frmg_ctx *ctx, std::vector<Problem> &P, const SolveCf
                                                   : cfg.tol;
   };
   auto update = [&]() {
-    for (int pi = 0; pi < np; pi++) {
-      if (!act[pi]) continue;
-      PROF("df_update");
-      k_df_update<<<nblocks(D[pi].ncell), 128, 0, st>>>(D[pi], fine_u(pi), ln2h, ln2l);
-      CK_LAUNCH(ctx);
+    PROF("df_update");
+    if (many) {
+      // the fields of this outer step (active holds act again after inner())
+      CK(cudaMemcpyAsync(d_fpar, fpar.data(), np * sizeof(int), cudaMemcpyHostToDevice, st));
+      k_df_update_many<<<boff[np], 128, 0, st>>>(jobs, d_boff, np, active, d_fpar, ln2h, ln2l);
+    } else {
+      k_df_update<<<nblocks(D[0].ncell), 128, 0, st>>>(D[0], fine_u(0), ln2h, ln2l);
     }
+    CK_LAUNCH(ctx);
   };
   CycleGraph gr_bg, gr_plain;
   // Stopping signal: the fine residual after pre-smoothing of each cycle (fused
@@ -2258,19 +2329,22 @@ static void solve_mixed_df(frmg_ctx *ctx, std::vector<Problem> &P, const SolveCf
   try {
     CK(cudaMemcpyAsync(active, act.data(), np * sizeof(int), cudaMemcpyHostToDevice, st));
     if (!nonzero) {
-      for (int pi = 0; pi < np; pi++) {
-        Grid<float> &G = H.lev[pi][0];
+      {
         PROF("prep_inner");
-        if (zero_start)
-          k_df_init_zero<<<nblocks(G.ncell), 256, 0, st>>>(D[pi], P[pi].rho,
-                                                           const_cast<float *>(G.f),
-                                                           H.cur_u(pi, 0), H.cur_x(pi, 0),
-                                                           partial, boff[pi], P[pi].check_rho,
-                                                           rho_bad);
+        Grid<float> &G = H.lev[0][0];
+        if (many && zero_start)
+          k_df_init_zero_many<<<boff[np], 256, 0, st>>>(jobs, d_boff, np, H.par[0], partial,
+                                                        rho_bad);
+        else if (many)
+          k_prep_zero_df_many<<<boff[np], 256, 0, st>>>(jobs, d_boff, np, H.par[0], partial);
+        else if (zero_start)
+          k_df_init_zero<<<nblocks(G.ncell), 256, 0, st>>>(
+              D[0], P[0].rho, const_cast<float *>(G.f), H.cur_u(0, 0), H.cur_x(0, 0), partial,
+              P[0].check_rho, rho_bad);
         else
-          k_prep_zero_df<<<nblocks(G.ncell), 256, 0, st>>>(D[pi].r, const_cast<float *>(G.f),
-                                                           H.cur_u(pi, 0), H.cur_x(pi, 0),
-                                                           G.ncell, partial, boff[pi]);
+          k_prep_zero_df<<<nblocks(G.ncell), 256, 0, st>>>(D[0].r, const_cast<float *>(G.f),
+                                                           H.cur_u(0, 0), H.cur_x(0, 0), G.ncell,
+                                                           partial);
         CK_LAUNCH(ctx);
       }
       read_norms(nr);
@@ -2297,13 +2371,21 @@ static void solve_mixed_df(frmg_ctx *ctx, std::vector<Problem> &P, const SolveCf
     }
     for (int outer = 0; outer < cfg.max_outer; outer++) {
       CK(cudaMemcpyAsync(active, act.data(), np * sizeof(int), cudaMemcpyHostToDevice, st));
-      for (int pi = 0; pi < np; pi++) {
-        if (!act[pi]) continue;
-        Grid<float> &G = H.lev[pi][0];
+      {
         PROF("df_defect");
-        launch_df_defect(ctx, D[pi], const_cast<float *>(G.f), H.bg_u[pi], H.bg_E[pi],
-                         H.cur_u(pi, 0), H.cur_x(pi, 0), partial, boff[pi], ln2h, ln2l, nullptr,
-                         st);
+        if (many) {
+          if (wide)
+            k_df_defect_many<true><<<boff[np], 128, 0, st>>>(jobs, d_boff, np, active, H.par[0],
+                                                             partial, ln2h, ln2l);
+          else
+            k_df_defect_many<false><<<boff[np], 128, 0, st>>>(jobs, d_boff, np, active, H.par[0],
+                                                              partial, ln2h, ln2l);
+          CK_LAUNCH(ctx);
+        } else {
+          Grid<float> &G = H.lev[0][0];
+          launch_df_defect(ctx, D[0], const_cast<float *>(G.f), H.bg_u[0], H.bg_E[0],
+                           H.cur_u(0, 0), H.cur_x(0, 0), partial, 0, ln2h, ln2l, nullptr, st);
+        }
       }
       read_norms(nr);
       int nact = 0;
@@ -2328,18 +2410,15 @@ static void solve_mixed_df(frmg_ctx *ctx, std::vector<Problem> &P, const SolveCf
       if (nact == 0) break;
       CK(cudaMemcpyAsync(active, act.data(), np * sizeof(int), cudaMemcpyHostToDevice, st));
       std::vector<double> r0(np, 0.0);
-      for (int pi = 0; pi < np; pi++) {
-        if (!act[pi]) continue;
-        r0[pi] = nr[2 * pi];
-        for (int l = 1; l < (int)H.lev[pi].size() && l <= H.tail_at[pi]; l++) {
-          Grid<float> &F = H.lev[pi][l - 1];
-          Grid<float> &C = H.lev[pi][l];
-          k_restrict_avg<float><<<nblocks(C.ncell), 256, 0, st>>>(F.ubg, F.n0, F.n1, F.n2,
-                                                                  const_cast<float *>(C.ubg));
-          CK_LAUNCH(ctx);
-          k_expf<<<nblocks(C.ncell), 256, 0, st>>>(C.ubg, const_cast<float *>(C.Ebg), C.ncell);
-          CK_LAUNCH(ctx);
-        }
+      for (int pi = 0; pi < np; pi++)
+        if (act[pi]) r0[pi] = nr[2 * pi];
+      // the background on the coarser launched levels and the tails' top levels
+      for (int l = 1; l < H.depth && !H.next[l - 1].empty(); l++) {
+        LevelSet<float> &C = H.next[l - 1];
+        k_bg_restrict<<<C.nblk_full, 256, 0, st>>>(H.cont[l - 1].d, C.d, C.d_off_full, C.size(),
+                                                   active);
+        CK_LAUNCH(ctx);
+        if (np == 1 && l >= H.tail_at[0]) break;
       }
       const bool likely_last = inner(true, r0, 1e-6, std::max(cfg.inner_cycles, 12));
       update();
