@@ -458,6 +458,8 @@ struct LevelSet {
   bool tiled = false;     // the tiled smoother is used for this set
   bool tiled_ok = false;  // it could be used (every grid >= 16 cells a side)
   bool dirichlet = false; // patches (all grids of a set are patches or all periodic)
+  // correction-form sweeps one colour per launch although the set is tiled
+  bool bg_cells = false;
   int zc = 0;
   std::vector<int> off_tile;
   int *d_off_tile = nullptr;
@@ -643,6 +645,11 @@ static void upload_set(Scope &S, LevelSet<T> &ls, cudaStream_t st, int tiling = 
       if (cells < 196608 || 100 * cells < 35 * covered) ls.tiled = false;
     }
     if (tiling < 0) ls.tiled = false;
+    // The register-column sweep of the correction form spills on patches (its
+    // ghost faces diverge in every row).  Patch solves, tiled sweeps against one
+    // colour per launch: 8 of 64^3 5.98 and 5.94 ms, 24 of 48^3 8.70 and 8.40,
+    // 12 of 96^3 24.4 and 21.5, 8 of 128^3 33.5 and 30.2.
+    ls.bg_cells = ls.dirichlet && tiling == 0;
   }
   if (ls.tiled_ok) {
     ls.off_tile.assign(ng + 1, 0);
@@ -1263,7 +1270,7 @@ static void smooth_set(frmg_ctx *ctx, LevelSet<T> &s, int sweeps, const std::vec
                        const int *active, int &par, cudaStream_t st, bool fine = true) {
   if (s.empty() || sweeps <= 0) return;
   if constexpr (sizeof(T) == 4) {
-    if (s.tiled && plan) {
+    if (s.tiled && plan && !(BG && s.bg_cells)) {
       for (int S : *plan) {
         // the correction form is reported apart from the plain one (different kernel)
         PROF(BG ? (fine ? "smooth_bg_f32@fine" : "smooth_bg_f32@coarse") : pname("smooth", false, fine));
