@@ -617,9 +617,14 @@ __global__ void __launch_bounds__(NT) k_residual(const Grid<T> *grids, const int
 }
 
 // Per-grid sums of the block partials: out[2g] = sum of squares, out[2g+1] = max.
-__global__ void k_reduce_partials(const double *partial, const int *off, int ngrid, double *out) {
+// Blocks past ngrid append pairs that are summed already.
+__global__ void k_reduce_partials(const double *partial, const int *off, int ngrid, double *out,
+                                  const double *done = nullptr) {
   int g = blockIdx.x;
-  if (g >= ngrid) return;
+  if (g >= ngrid) {
+    if (done && threadIdx.x < 2) out[2 * g + threadIdx.x] = done[2 * (g - ngrid) + threadIdx.x];
+    return;
+  }
   double s = 0.0, m = 0.0;
   for (int b = off[g] + threadIdx.x; b < off[g + 1]; b += blockDim.x) {
     s += partial[2 * b];

@@ -63,6 +63,9 @@ struct FrError {
   } while (0)
 
 static void einval(const std::string &m) { throw FrError{FR_EINVAL, m}; }
+static const char *kBadDensity = "density has NaN/Inf or negative values";
+static const char *kBadStencil =
+    "patch interpolation stencil leaves its parent (needs a 1-parent-cell margin)";
 
 // ---------------------------------------------------------------------------
 // context: device, caching allocator, pinned readback buffer
@@ -232,6 +235,45 @@ struct Scope {
   }
   ~Scope() {
     for (void *p : ptrs) frmg_release(c, p);
+  }
+};
+
+// Small host arrays of one set-up, gathered into few device blocks and sent in
+// one copy per block (one copy and one synchronisation per array and level set
+// came to 0.4 ms for a 64^3 field).  put() returns where the array will be;
+// it is there once flush() has run and the stream has reached it.
+struct Upload {
+  struct Block {
+    char *dev;
+    std::vector<char> host;
+    size_t used;
+  };
+  Scope &S;
+  cudaStream_t st;
+  std::vector<Block> blocks;
+  Upload(Scope &S_, cudaStream_t st_) : S(S_), st(st_) {}
+  template <typename T>
+  T *put(const T *src, size_t n) {
+    const size_t bytes = (n * sizeof(T) + 255) & ~(size_t)255;
+    if (blocks.empty() || blocks.back().used + bytes > blocks.back().host.size()) {
+      const size_t cap = std::max<size_t>(bytes, 64 * 1024);
+      blocks.push_back({S.get<char>(cap), std::vector<char>(cap), 0});
+    }
+    Block &b = blocks.back();
+    memcpy(b.host.data() + b.used, src, n * sizeof(T));
+    T *d = reinterpret_cast<T *>(b.dev + b.used);
+    b.used += bytes;
+    return d;
+  }
+  template <typename T>
+  T *put(const std::vector<T> &v) {
+    return put(v.data(), v.size());
+  }
+  void flush() {
+    for (Block &b : blocks)
+      CK(cudaMemcpyAsync(b.dev, b.host.data(), b.used, cudaMemcpyHostToDevice, st));
+    CK(cudaStreamSynchronize(st));  // the host blocks have been read
+    blocks.clear();
   }
 };
 
@@ -576,8 +618,7 @@ template <bool DIR>
 static long long rr_slots();
 
 template <typename T>
-static void upload_set(Scope &S, LevelSet<T> &ls, cudaStream_t st, int tiling = 0,
-                       int stile = 0) {
+static void upload_set(Scope &S, LevelSet<T> &ls, Upload &up, int tiling = 0, int stile = 0) {
   if (ls.empty()) return;
   int ng = ls.size();
   ls.off_half.assign(ng + 1, 0);
@@ -600,17 +641,11 @@ static void upload_set(Scope &S, LevelSet<T> &ls, cudaStream_t st, int tiling = 
     g.fd0 = make_fastdiv((unsigned)g.n0);
     g.fd1 = make_fastdiv((unsigned)g.n1);
   }
-  ls.d = S.get<Grid<T>>(ng);
-  ls.d_off_half = S.get<int>(4 * (size_t)(ng + 1));
-  ls.d_off_cell = ls.d_off_half + (ng + 1);
-  ls.d_off_full = ls.d_off_cell + (ng + 1);
-  ls.d_off_fine = ls.d_off_full + (ng + 1);
-  CK(cudaMemcpyAsync(ls.d, ls.h.data(), ng * sizeof(Grid<T>), cudaMemcpyHostToDevice, st));
-  std::vector<int> offs;
-  for (auto *v : {&ls.off_half, &ls.off_cell, &ls.off_full, &ls.off_fine})
-    offs.insert(offs.end(), v->begin(), v->end());
-  CK(cudaMemcpyAsync(ls.d_off_half, offs.data(), offs.size() * sizeof(int),
-                     cudaMemcpyHostToDevice, st));
+  ls.d = up.put(ls.h);
+  ls.d_off_half = up.put(ls.off_half);
+  ls.d_off_cell = up.put(ls.off_cell);
+  ls.d_off_full = up.put(ls.off_full);
+  ls.d_off_fine = up.put(ls.off_fine);
   ls.dirichlet = ls.h[0].bnd != nullptr;
   for (int g = 1; g < ng; g++)
     if ((ls.h[g].bnd != nullptr) != ls.dirichlet)
@@ -659,9 +694,7 @@ static void upload_set(Scope &S, LevelSet<T> &ls, cudaStream_t st, int tiling = 
       ls.off_tile[g + 1] = ls.off_tile[g] + nt;
     }
     ls.nblk_tile = ls.off_tile[ng];
-    ls.d_off_tile = S.get<int>(ng + 1);
-    CK(cudaMemcpyAsync(ls.d_off_tile, ls.off_tile.data(), (ng + 1) * sizeof(int),
-                       cudaMemcpyHostToDevice, st));
+    ls.d_off_tile = up.put(ls.off_tile);
     if constexpr (sizeof(T) == 4) {
       std::vector<long long> tl(ng);
       std::vector<int> n2s(ng);
@@ -678,9 +711,7 @@ static void upload_set(Scope &S, LevelSet<T> &ls, cudaStream_t st, int tiling = 
           ls.off_rb[v][g + 1] =
               ls.off_rb[v][g] + (int)(tl[g] * ((n2s[g] + ls.zc_rb[v] - 1) / ls.zc_rb[v]));
         ls.nblk_rb[v] = ls.off_rb[v][ng];
-        ls.d_off_rb[v] = S.get<int>(ng + 1);
-        CK(cudaMemcpyAsync(ls.d_off_rb[v], ls.off_rb[v].data(), (ng + 1) * sizeof(int),
-                           cudaMemcpyHostToDevice, st));
+        ls.d_off_rb[v] = up.put(ls.off_rb[v]);
       }
       if (stile == 8 || stile == 16) {
         // plain form on 64 x stile tiles, correction form on 64 x 8 tiles
@@ -702,9 +733,7 @@ static void upload_set(Scope &S, LevelSet<T> &ls, cudaStream_t st, int tiling = 
             ls.off_rc[v][g + 1] =
                 ls.off_rc[v][g] + (int)(tl[g] * ((n2s[g] + ls.zc_rc[v] - 1) / ls.zc_rc[v]));
           ls.nblk_rc[v] = ls.off_rc[v][ng];
-          ls.d_off_rc[v] = S.get<int>(ng + 1);
-          CK(cudaMemcpyAsync(ls.d_off_rc[v], ls.off_rc[v].data(), (ng + 1) * sizeof(int),
-                             cudaMemcpyHostToDevice, st));
+          ls.d_off_rc[v] = up.put(ls.off_rc[v]);
         }
       }
       for (int g = 0; g < ng; g++)
@@ -718,9 +747,7 @@ static void upload_set(Scope &S, LevelSet<T> &ls, cudaStream_t st, int tiling = 
           ls.off_fr[v][g + 1] =
               ls.off_fr[v][g] + (int)(tl[g] * ((n2s[g] + ls.zc_fr[v] - 1) / ls.zc_fr[v]));
         ls.nblk_fr[v] = ls.off_fr[v][ng];
-        ls.d_off_fr[v] = S.get<int>(ng + 1);
-        CK(cudaMemcpyAsync(ls.d_off_fr[v], ls.off_fr[v].data(), (ng + 1) * sizeof(int),
-                           cudaMemcpyHostToDevice, st));
+        ls.d_off_fr[v] = up.put(ls.off_fr[v]);
       }
     }
   }
@@ -747,9 +774,7 @@ static void upload_set(Scope &S, LevelSet<T> &ls, cudaStream_t st, int tiling = 
         for (int g = 0; g < ng; g++)
           ls.off_pl[g + 1] = ls.off_pl[g] + (int)(tl[g] * ((n2s[g] + ls.kc_pl - 1) / ls.kc_pl));
         ls.nblk_pl = ls.off_pl[ng];
-        ls.d_off_pl = S.get<int>(ng + 1);
-        CK(cudaMemcpyAsync(ls.d_off_pl, ls.off_pl.data(), (ng + 1) * sizeof(int),
-                           cudaMemcpyHostToDevice, st));
+        ls.d_off_pl = up.put(ls.off_pl);
       }
     }
     ls.off_rr.assign(ng + 1, 0);
@@ -760,9 +785,7 @@ static void upload_set(Scope &S, LevelSet<T> &ls, cudaStream_t st, int tiling = 
       ls.off_rr[g + 1] = ls.off_rr[g] + nt;
     }
     ls.nblk_rr = ls.off_rr[ng];
-    ls.d_off_rr = S.get<int>(ng + 1);
-    CK(cudaMemcpyAsync(ls.d_off_rr, ls.off_rr.data(), (ng + 1) * sizeof(int),
-                       cudaMemcpyHostToDevice, st));
+    ls.d_off_rr = up.put(ls.off_rr);
     ls.rr_tiled = true;
   }
   ls.partial = S.get<double>(2 * (size_t)std::max({ls.nblk_full, ls.nblk_fine, ls.nblk_rr}));
@@ -770,8 +793,15 @@ static void upload_set(Scope &S, LevelSet<T> &ls, cudaStream_t st, int tiling = 
   if (ls.red_nch) ls.red_tmp = S.get<double>(2 * (size_t)ls.red_nch * ng);
   ls.red = S.get<double>(2 * (size_t)ng);
   ls.d_dout = S.get<T *>(ng);
-  // host vectors must stay alive until the copies finished
-  CK(cudaStreamSynchronize(st));
+}
+
+// One level set on its own.
+template <typename T>
+static void upload_set(Scope &S, LevelSet<T> &ls, cudaStream_t st, int tiling = 0,
+                       int stile = 0) {
+  Upload up(S, st);
+  upload_set(S, ls, up, tiling, stile);
+  up.flush();
 }
 
 // Tails (k_tail) of the problems whose one-cluster part of the V-cycle begins
@@ -852,7 +882,7 @@ constexpr size_t kTailSmem = 222 * 1024;
 // Chooses the depth at which each problem's tail begins (none above depth
 // tail_min; tail_min < 0: no tails) and uploads the tails' levels.
 template <typename T>
-static void plan_tails(Scope &S, Hier<T> &H, int tail_min, cudaStream_t st) {
+static void plan_tails(Scope &S, Hier<T> &H, int tail_min, Upload &up) {
   const int np = (int)H.lev.size();
   H.tail_at.resize(np);
   H.tail.assign(H.depth, {});
@@ -901,14 +931,10 @@ static void plan_tails(Scope &S, Hier<T> &H, int tail_min, cudaStream_t st) {
   for (auto &t : H.tail) {
     if (t.empty()) continue;
     for (int bg = 0; bg < 2; bg++) {
-      if (t.h[bg].empty()) continue;
-      const size_t bytes = t.h[bg].size() * sizeof(TailDesc<T>);
-      t.d[bg] = S.get<TailDesc<T>>(t.h[bg].size());
-      CK(cudaMemcpyAsync(t.d[bg], t.h[bg].data(), bytes, cudaMemcpyHostToDevice, st));
+      if (!t.h[bg].empty()) t.d[bg] = up.put(t.h[bg]);
     }
     t.norms = S.get<double>(2 * (size_t)t.size());
   }
-  CK(cudaStreamSynchronize(st));  // the host vectors have been read
 }
 
 template <typename T, bool BG>
@@ -997,7 +1023,8 @@ static void build_hier(Scope &S, Hier<T> &H, std::vector<Problem> &P, double cap
   H.next.assign(H.depth, {});
   H.coarsest.assign(H.depth, {});
   H.all.assign(H.depth, {});
-  plan_tails(S, H, tail_min, st);
+  Upload up(S, st);
+  plan_tails(S, H, tail_min, up);
   for (int pi = 0; pi < np; pi++) {
     int nl = P[pi].nl;
     for (int l = 0; l < nl; l++) {
@@ -1012,11 +1039,12 @@ static void build_hier(Scope &S, Hier<T> &H, std::vector<Problem> &P, double cap
     }
   }
   for (int l = 0; l < H.depth; l++) {
-    upload_set(S, H.cont[l], st, tiling, stile);
-    upload_set(S, H.next[l], st, tiling, stile);
-    upload_set(S, H.coarsest[l], st, tiling, stile);
-    upload_set(S, H.all[l], st, tiling, stile);
+    upload_set(S, H.cont[l], up, tiling, stile);
+    upload_set(S, H.next[l], up, tiling, stile);
+    upload_set(S, H.coarsest[l], up, tiling, stile);
+    upload_set(S, H.all[l], up, tiling, stile);
   }
+  up.flush();
 }
 
 // ---------------------------------------------------------------------------
@@ -1633,14 +1661,27 @@ static void fused_fine_norms(frmg_ctx *ctx, Hier<T> &H, int np, cudaStream_t st,
   const int ng = C.empty() ? 0 : C.size(), nt = Q.size();
   if (ng + nt == 0) return;
   double *hp = pinned_buf(ctx, 2 * (size_t)(ng + nt));
-  if (ng) {
-    const int *offs = H.cont[0].rr_tiled ? H.cont[0].d_off_rr : C.d_off_fine;
-    k_reduce_partials<<<ng, 256, 0, st>>>(C.partial, offs, ng, C.red);
-    CK_LAUNCH(ctx);
-    CK(cudaMemcpyAsync(hp, C.red, 2 * ng * sizeof(double), cudaMemcpyDeviceToHost, st));
+  // the kernel that sums the partials writes them to the host buffer itself
+  double *hpd = nullptr;
+  if (cudaHostGetDevicePointer((void **)&hpd, hp, 0) != cudaSuccess) {
+    cudaGetLastError();
+    hpd = nullptr;
   }
-  if (nt)
-    CK(cudaMemcpyAsync(hp + 2 * ng, Q.norms, 2 * nt * sizeof(double), cudaMemcpyDeviceToHost, st));
+  double *red = hpd ? hpd : C.red;
+  const int *offs = !ng ? nullptr : (H.cont[0].rr_tiled ? H.cont[0].d_off_rr : C.d_off_fine);
+  if (hpd) {
+    k_reduce_partials<<<ng + nt, 256, 0, st>>>(C.partial, offs, ng, red, Q.norms);
+    CK_LAUNCH(ctx);
+  } else {
+    if (ng) {
+      k_reduce_partials<<<ng, 256, 0, st>>>(C.partial, offs, ng, red);
+      CK_LAUNCH(ctx);
+      CK(cudaMemcpyAsync(hp, red, 2 * ng * sizeof(double), cudaMemcpyDeviceToHost, st));
+    }
+    if (nt)
+      CK(cudaMemcpyAsync(hp + 2 * ng, Q.norms, 2 * nt * sizeof(double), cudaMemcpyDeviceToHost,
+                         st));
+  }
   CK(cudaStreamSynchronize(st));
   prof_harvest(ctx);
   for (int g = 0; g < ng; g++) {
@@ -2118,8 +2159,8 @@ static void solve_mixed_df(frmg_ctx *ctx, std::vector<Problem> &P, const SolveCf
   }
   double *partial = S.get<double>(2 * (size_t)boff[np]);
   double *red = S.get<double>(2 * (size_t)np);
-  int *d_boff = S.get<int>(np + 1);
-  CK(cudaMemcpyAsync(d_boff, boff.data(), (np + 1) * sizeof(int), cudaMemcpyHostToDevice, st));
+  Upload up(S, st);
+  int *d_boff = up.put(boff);
   // the fine-grid steps of a batch take all its grids in one launch
   const bool many = np > 1;
   bool wide = false;  // a grid of 2^31 cells or more
@@ -2144,11 +2185,10 @@ static void solve_mixed_df(frmg_ctx *ctx, std::vector<Problem> &P, const SolveCf
       j.check_rho = P[pi].check_rho;
       wide = wide || D[pi].ncell >= (1ll << 31);
     }
-    jobs = S.get<DFJob>(np);
+    jobs = up.put(hj);
     d_fpar = S.get<int>(np);
-    CK(cudaMemcpyAsync(jobs, hj.data(), np * sizeof(DFJob), cudaMemcpyHostToDevice, st));
-    CK(cudaStreamSynchronize(st));  // hj has been read
   }
+  up.flush();
   // a zero start that the caller declared (initial_guess = 0) reads no u and
   // sets the state up in one fused pass below; otherwise u is scanned for a
   // non-zero value
@@ -2359,7 +2399,7 @@ static void solve_mixed_df(frmg_ctx *ctx, std::vector<Problem> &P, const SolveCf
         int hb = 0;
         CK(cudaMemcpyAsync(&hb, rho_bad, sizeof(int), cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
-        if (hb) throw FrError{FR_EINVAL, "density has NaN/Inf or negative values"};
+        if (hb) throw FrError{FR_EINVAL, kBadDensity};
       }
       std::vector<double> r0(np);
       for (int pi = 0; pi < np; pi++) {
@@ -2531,7 +2571,7 @@ static void validate_density(frmg_ctx *ctx, Scope &S, const double *rho, long lo
   int hb = 0;
   CK(cudaMemcpyAsync(&hb, bad, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
-  if (hb) einval("density has NaN/Inf or negative values");
+  if (hb) einval(kBadDensity);
 }
 
 static fr_opts resolve_opts(const fr_opts *o) {
@@ -2717,11 +2757,10 @@ __global__ void k_patch_faces(const double *up, int p0, int p1, int p2, int peri
   }
 }
 
-static void patch_bc_dev(frmg_ctx *ctx, Scope &S, const double *up, const int np_[3], int periodic,
-                         const int org[3], const int n[3], double *u_init, double *ub,
-                         cudaStream_t st) {
-  int *bad = S.get<int>(1);
-  CK(cudaMemsetAsync(bad, 0, sizeof(int), st));
+// Sets *bad where the stencil leaves the parent.
+static void patch_bc_launch(frmg_ctx *ctx, const double *up, const int np_[3], int periodic,
+                            const int org[3], const int n[3], double *u_init, double *ub,
+                            int *bad, cudaStream_t st) {
   long long nc = (long long)n[0] * n[1] * n[2];
   k_patch_init<<<nblocks(nc), 256, 0, st>>>(up, np_[0], np_[1], np_[2], periodic, org[0], org[1],
                                             org[2], n[0], n[1], n[2], u_init, bad);
@@ -2730,10 +2769,18 @@ static void patch_bc_dev(frmg_ctx *ctx, Scope &S, const double *up, const int np
   k_patch_faces<<<nblocks(nf), 256, 0, st>>>(up, np_[0], np_[1], np_[2], periodic, org[0],
                                              org[1], org[2], n[0], n[1], n[2], u_init, ub, bad);
   CK_LAUNCH(ctx);
+}
+
+static void patch_bc_dev(frmg_ctx *ctx, Scope &S, const double *up, const int np_[3], int periodic,
+                         const int org[3], const int n[3], double *u_init, double *ub,
+                         cudaStream_t st) {
+  int *bad = S.get<int>(1);
+  CK(cudaMemsetAsync(bad, 0, sizeof(int), st));
+  patch_bc_launch(ctx, up, np_, periodic, org, n, u_init, ub, bad, st);
   int hb = 0;
   CK(cudaMemcpyAsync(&hb, bad, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
-  if (hb) einval("patch interpolation stencil leaves its parent (needs a 1-parent-cell margin)");
+  if (hb) einval(kBadStencil);
 }
 
 // y += s * x
@@ -3259,18 +3306,25 @@ int fr_solve_levels(frmg_ctx *ctx, const double *density, const int dims[3], dou
     for (int lv = 1; lv <= maxlev; lv++) {
       std::vector<Problem> P;
       std::vector<int> ids;
+      // the checks of all patches of the level are read back together: per
+      // patch the density's and the interpolation stencil's flag
+      int *bad = S.get<int>(2 * (size_t)npatch);
+      CK(cudaMemsetAsync(bad, 0, 2 * (size_t)npatch * sizeof(int), st));
       for (int i = 0; i < npatch; i++) {
         if (level[i] != lv) continue;
         fr_patch &pp = patches[i];
         long long pn = (long long)pp.n[0] * pp.n[1] * pp.n[2];
         const double *prho = stage(S, back, pp.density, pn, true, false, st);
         pu[i] = stage(S, back, pp.u, pn, false, true, st);
-        validate_density(ctx, S, prho, pn, o.allow_negative_density, st);
+        k_check_density<<<nblocks(pn), 256, 0, st>>>(prho, pn, o.allow_negative_density,
+                                                     bad + 2 * i);
+        CK_LAUNCH(ctx);
         double *ub = S.get<double>(face_total(pp.n));
         const double *up = pp.parent < 0 ? du : pu[pp.parent];
         const int *pdim = pp.parent < 0 ? dims : pdims[pp.parent].data();
         double hpar = pp.parent < 0 ? 1.0 / dims[0] : ph[pp.parent];
-        patch_bc_dev(ctx, S, up, pdim, pp.parent < 0, pp.origin, pp.n, pu[i], ub, st);
+        patch_bc_launch(ctx, up, pdim, pp.parent < 0, pp.origin, pp.n, pu[i], ub, bad + 2 * i + 1,
+                        st);
         ph[i] = 0.5 * hpar;
         Problem p;
         memset(&p, 0, sizeof(p));
@@ -3285,6 +3339,13 @@ int fr_solve_levels(frmg_ctx *ctx, const double *density, const int dims[3], dou
         p.bnd = ub;
         P.push_back(p);
         ids.push_back(i);
+      }
+      std::vector<int> hb(2 * (size_t)npatch);
+      CK(cudaMemcpyAsync(hb.data(), bad, hb.size() * sizeof(int), cudaMemcpyDeviceToHost, st));
+      CK(cudaStreamSynchronize(st));
+      for (int i : ids) {
+        if (hb[2 * i]) einval(kBadDensity);
+        if (hb[2 * i + 1]) einval(kBadStencil);
       }
       std::vector<fr_stats> sv(P.size());
       memset(sv.data(), 0, sv.size() * sizeof(fr_stats));
