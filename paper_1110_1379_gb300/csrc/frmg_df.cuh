@@ -105,9 +105,8 @@ __device__ __forceinline__ void df_update(const DFGrid &G, const float *delta, f
     const df2 B = df_mul2(df2{make_float2(Bo.x, Bo.z), make_float2(Bo.y, Bo.w)}, q);
     Bn = make_float4(B.h.x, B.l.x, B.h.y, B.l.y);
   } else {
-    const df b0 = df_exp(df{u.h.x, u.l.x}, ln2h, ln2l);
-    const df b1 = df_exp(df{u.h.y, u.l.y}, ln2h, ln2l);
-    Bn = make_float4(b0.h, b0.l, b1.h, b1.l);
+    const df2 b = df_exp2(u, ln2h, ln2l);
+    Bn = make_float4(b.h.x, b.l.x, b.h.y, b.l.y);
   }
   B4[t] = Bn;
 }

@@ -82,17 +82,20 @@ __device__ __forceinline__ df df_rsqrt(df a) {
 
 // e^u for u = (h, l) (|u| < 80): u = n ln2 + r, e^r from its Taylor series at
 // r/16 (degree 7, truncation below 1e-17 relative) squared four times, scaled
-// by 2^n.  ln2 enters as the double-float pair (ln2h, ln2l) supplied by the host.
+// by 2^n.  The series is 1 + s (1 + s/2 (1 + s/3 (1 + s/4 (1 + tau)))), tau =
+// s/5 (1 + s/6 (1 + s/7)) in FP32: its rounding enters through s^4/24 < 1e-8,
+// below 3e-18 of the result.  ln2 enters as the double-float pair (ln2h,
+// ln2l) supplied by the host.
 __device__ __forceinline__ df df_exp(df u, float ln2h, float ln2l) {
   float n = rintf(u.h * 1.44269504f);  // nearest integer to u / ln2
   df nl = df_add(two_prod(n, ln2h), two_prod(n, ln2l));
   df r = df_sub(u, nl);
   r.h *= 0.0625f;  // exact scaling by 2^-4
   r.l *= 0.0625f;
-  // Horner: 1 + r (1 + r/2 (1 + r/3 (... (1 + r/7))))
-  df t = {1.0f, 0.0f};
+  const float tau = (r.h * 0.2f) * fmaf(r.h * (1.0f / 6.0f), fmaf(r.h, 1.0f / 7.0f, 1.0f), 1.0f);
+  df t = fast_two_sum(1.0f, tau);
 #pragma unroll
-  for (int k = 7; k >= 1; k--) {
+  for (int k = 4; k >= 1; k--) {
     t = df_mul(t, r);
     // t = 1 + t / k: q = t.h (1/k) rounded, then the remainder t - q k (exact
     // by FMA) divided by k gives the low part (two-step division by a float)
@@ -194,6 +197,30 @@ __device__ __forceinline__ df2 df_diff2(df2 ui, df2 uj) {
   float2 e = sub2(sub2(uj.h, sub2(s, bb)), add2(ui.h, bb));
   e = add2(e, sub2(uj.l, ui.l));
   return fast_two_sum2(s, e);
+}
+// df_exp lane by lane
+__device__ __forceinline__ df2 df_exp2(df2 u, float ln2h, float ln2l) {
+  const float2 n = make_float2(rintf(u.h.x * 1.44269504f), rintf(u.h.y * 1.44269504f));
+  const df2 nl = df_add2(two_prod2(n, splat2(ln2h)), two_prod2(n, splat2(ln2l)));
+  df2 r = df_sub2(u, nl);
+  r.h = mul2(r.h, splat2(0.0625f));
+  r.l = mul2(r.l, splat2(0.0625f));
+  float2 p = fma2(r.h, splat2(1.0f / 7.0f), splat2(1.0f));
+  p = fma2(mul2(r.h, splat2(1.0f / 6.0f)), p, splat2(1.0f));
+  df2 t = fast_two_sum2(splat2(1.0f), mul2(mul2(r.h, splat2(0.2f)), p));
+#pragma unroll
+  for (int k = 4; k >= 1; k--) {
+    t = df_mul2(t, r);
+    const float rk = 1.0f / (float)k;
+    const float2 q = mul2(t.h, splat2(rk));
+    const float2 rem = add2(fma2(q, splat2(-(float)k), t.h), t.l);
+    t = df_add_f2(df2{q, mul2(rem, splat2(rk))}, 1.0f);
+  }
+#pragma unroll
+  for (int k = 0; k < 4; k++) t = df_mul2(t, t);
+  const int n0 = (int)n.x, n1 = (int)n.y;
+  return {make_float2(ldexpf(t.h.x, n0), ldexpf(t.h.y, n1)),
+          make_float2(ldexpf(t.l.x, n0), ldexpf(t.l.y, n1))};
 }
 // df_rsqrt lane by lane: the FP32 estimate per lane, the Newton step packed
 __device__ __forceinline__ df2 df_rsqrt2(df2 a) {

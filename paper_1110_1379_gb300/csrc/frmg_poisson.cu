@@ -696,46 +696,63 @@ struct PFine {
   long long foff[6];
   int n0, n1, n2;
   long long ncell;
-  FastDiv fd0, fd1;
+  FastDiv fdh, fd1;    // division by n0 / 2 and n1
   float ih2h, ih2l;    // 1/h^2 as a double-float pair
 };
 
-__device__ __forceinline__ df ldf(const float2 *p, long long c) {
-  const float2 v = p[c];
-  return {v.x, v.y};
-}
-
-// Sum of two double-float values across a warp; lane 0 holds the total.
+// Sum of double-float values across a warp, on every lane.
 __device__ __forceinline__ df warp_df_sum(df v) {
   for (int o = 16; o > 0; o >>= 1) {
-    df w = {__shfl_down_sync(0xffffffffu, v.h, o), __shfl_down_sync(0xffffffffu, v.l, o)};
+    df w = {__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)};
     v = df_add(v, w);
   }
   return v;
 }
 
 // Block (sum, max) of a double-float per-thread value: partial[2 b] = sum
-// (as FP64), partial[2 b + 1] = max |value| (the max is taken on the high parts).
+// (as FP64), partial[2 b + 1] = max |value| (the max is taken on the high
+// parts).  No FP64 arithmetic: the warp sums are added as pairs too.
 __device__ __forceinline__ void block_df_partial(df v, float amax, double *partial) {
-  __shared__ double ws[kNT / 32];
+  __shared__ float2 ws[kNT / 32];
   __shared__ float wm[kNT / 32];
   v = warp_df_sum(v);
-  for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_down_sync(0xffffffffu, amax, o));
-  if ((threadIdx.x & 31) == 0) {
-    ws[threadIdx.x >> 5] = join_bits(v.h, v.l);
+  for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+  const int lane = threadIdx.x & 31;
+  if (lane == 0) {
+    ws[threadIdx.x >> 5] = make_float2(v.h, v.l);
     wm[threadIdx.x >> 5] = amax;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    float m = 0.0f;
-    for (int w = 0; w < kNT / 32; w++) {
-      s += ws[w];
-      m = fmaxf(m, wm[w]);
+  if (threadIdx.x < 32) {
+    const float2 w = lane < kNT / 32 ? ws[lane] : make_float2(0.f, 0.f);
+    v = warp_df_sum(df{w.x, w.y});
+    amax = lane < kNT / 32 ? wm[lane] : 0.0f;
+    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+    if (lane == 0) {
+      partial[2 * blockIdx.x] = join_bits(v.h, v.l);
+      partial[2 * blockIdx.x + 1] = (double)amax;
     }
-    partial[2 * blockIdx.x] = s;
-    partial[2 * blockIdx.x + 1] = (double)m;
   }
+}
+
+// The double-float passes over the fine grid work on x-pairs (every n0 is
+// even), the pair arithmetic on packed FP32 pairs; the sums take kPP pairs per
+// thread, 256 apart, so that their block reduction (about 150 instructions) is
+// shared by 2 kPP cells.  At 512^3: source 3.20 -> 1.98 ms, sum of phi 0.80 ->
+// 0.18 ms, defect 1.47 -> 1.13 ms (one cell per thread before).
+constexpr int kPP = 2;
+
+__device__ __forceinline__ df2 ld_df2(const float2 *p, long long pair) {
+  const float4 v = reinterpret_cast<const float4 *>(p)[pair];
+  return {make_float2(v.x, v.z), make_float2(v.y, v.w)};
+}
+__device__ __forceinline__ void st_df2(float2 *p, long long pair, const df2 &v) {
+  reinterpret_cast<float4 *>(p)[pair] = make_float4(v.h.x, v.l.x, v.h.y, v.l.y);
+}
+// cells c0 and c1 of an FP64 array of the caller's (aligned to 8 bytes only)
+__device__ __forceinline__ df2 split2(const double *p, long long c0, long long c1) {
+  const df a = split_bits(p[c0]), b = split_bits(p[c1]);
+  return {make_float2(a.h, b.h), make_float2(a.l, b.l)};
 }
 
 // s = 2 gamma (rho - 1) - (beta/2)(e^{-u/2} - 1) and phi = phi0, both as
@@ -743,65 +760,108 @@ __device__ __forceinline__ void block_df_partial(df v, float amax, double *parti
 __global__ void __launch_bounds__(kNT)
     k_psource(PFine P, const double *rho, const double *u, const double *phi0, float g2h,
               float g2l, float bh, float bl, float ln2h, float ln2l, double *partial) {
-  const long long t = (long long)blockIdx.x * kNT + threadIdx.x;
-  df v = {0.f, 0.f};
+  df2 v = {splat2(0.f), splat2(0.f)};
   float am = 0.0f;
-  if (t < P.ncell) {
-    const df r = split_bits(rho[t]);
-    const df uu = split_bits(u[t]);
-    const df e = df_exp(df{-0.5f * uu.h, -0.5f * uu.l}, ln2h, ln2l);  // exact halving
-    const df s = df_sub(df_mul(df_add_f(r, -1.0f), df{g2h, g2l}),
-                        df_mul(df_add_f(e, -1.0f), df{bh, bl}));
-    P.s[t] = make_float2(s.h, s.l);
-    const df p = phi0 ? split_bits(phi0[t]) : df{0.f, 0.f};
-    P.phi[t] = make_float2(p.h, p.l);
-    v = s;
-    am = fabsf(s.h);
+#pragma unroll
+  for (int q = 0; q < kPP; q++) {
+    const long long t = ((long long)blockIdx.x * kPP + q) * kNT + threadIdx.x;
+    const long long c0 = 2 * t;
+    if (c0 >= P.ncell) break;
+    // (the last pair of an odd number of cells holds one cell twice)
+    const bool two = c0 + 1 < P.ncell;
+    const long long c1 = two ? c0 + 1 : c0;
+    const df2 r = split2(rho, c0, c1), uu = split2(u, c0, c1);
+    const df2 e = df_exp2(df2{mul2(uu.h, splat2(-0.5f)), mul2(uu.l, splat2(-0.5f))}, ln2h,
+                          ln2l);  // exact halving
+    df2 s = df_sub2(df_mul2(df_add_f2(r, -1.0f), df2{splat2(g2h), splat2(g2l)}),
+                    df_mul2(df_add_f2(e, -1.0f), df2{splat2(bh), splat2(bl)}));
+    const df2 p0 = phi0 ? split2(phi0, c0, c1) : df2{splat2(0.f), splat2(0.f)};
+    if (two) {
+      st_df2(P.s, t, s);
+      st_df2(P.phi, t, p0);
+    } else {
+      P.s[c0] = make_float2(s.h.x, s.l.x);
+      P.phi[c0] = make_float2(p0.h.x, p0.l.x);
+      s.h.y = s.l.y = 0.0f;
+    }
+    v = df_add2(v, s);
+    am = fmaxf(am, fmaxf(fabsf(s.h.x), fabsf(s.h.y)));
   }
-  block_df_partial(v, am, partial);
+  block_df_partial(df_add(df{v.h.x, v.l.x}, df{v.h.y, v.l.y}), am, partial);
 }
 
 // Fine defect d = L(phi) - (s - smean) in double-float; the FP32 correction
-// problem gets f = -d and e = 0.  Per-block partials of (d^2, max |d|).
+// problem gets f = -d and e = 0.  Per-block partials of (d^2, max |d|).  One
+// x-pair per thread.  The sum of the neighbours carries its rounding errors and
+// the low parts in one FP32 sum (TwoSum per neighbour) and is normalised once.
 __global__ void __launch_bounds__(kNT)
     k_pdefect(PFine P, float smh, float sml, float *f32, float *e32, double *partial,
               double *dout) {
   const long long t = (long long)blockIdx.x * kNT + threadIdx.x;
   float ss = 0.0f, mx = 0.0f;
-  if (t < P.ncell) {
-    const unsigned tu = (unsigned)t, q = fdiv(tu, P.fd0), q2 = fdiv(q, P.fd1);
-    const int i = (int)(tu - q * (unsigned)P.n0), j = (int)(q - q2 * (unsigned)P.n1),
-              k = (int)q2;
-    const long long sy = P.n0, sz = (long long)P.n0 * P.n1;
-    const df pi = ldf(P.phi, t);
-    df acc = {0.f, 0.f};
-    int nb = 0;  // neighbours inside
-    auto reg = [&](long long cj) {
-      acc = df_add(acc, ldf(P.phi, cj));
-      nb++;
-    };
-    auto ghost = [&](int f, long long o) {
-      // ghost 2 phi_b - phi_i: phi_b enters here, -phi_i with the diagonal
-      const df b = split_bits(P.phib[P.foff[f] + o]);
-      acc = df_add(acc, df{2.0f * b.h, 2.0f * b.l});
-    };
+  if (t < (P.ncell >> 1)) {
+    const unsigned tu = (unsigned)t, q = fdiv(tu, P.fdh), q2 = fdiv(q, P.fd1);
+    const int i = 2 * (int)(tu - q * (unsigned)(P.n0 >> 1)),
+              j = (int)(q - q2 * (unsigned)P.n1), k = (int)q2;
+    const long long c = 2 * t, sy = P.n0, sz = (long long)P.n0 * P.n1;
+    const df2 pi = ld_df2(P.phi, t);
     const bool pat = P.phib != nullptr;
-    if (i > 0) reg(t - 1); else if (!pat) reg(t + (P.n0 - 1)); else ghost(0, (long long)k * P.n1 + j);
-    if (i < P.n0 - 1) reg(t + 1); else if (!pat) reg(t - (P.n0 - 1)); else ghost(1, (long long)k * P.n1 + j);
-    if (j > 0) reg(t - sy); else if (!pat) reg(t + (P.n1 - 1) * sy); else ghost(2, (long long)k * P.n0 + i);
-    if (j < P.n1 - 1) reg(t + sy); else if (!pat) reg(t - (P.n1 - 1) * sy); else ghost(3, (long long)k * P.n0 + i);
-    if (k > 0) reg(t - sz); else if (!pat) reg(t + (P.n2 - 1) * sz); else ghost(4, (long long)j * P.n0 + i);
-    if (k < P.n2 - 1) reg(t + sz); else if (!pat) reg(t - (P.n2 - 1) * sz); else ghost(5, (long long)j * P.n0 + i);
+    float2 nb = splat2(6.0f);  // neighbours inside
+    // ghost 2 phi_b - phi_i: phi_b enters here, -phi_i with the diagonal
+    auto ghost = [&](int f, long long o) {
+      const df b = split_bits(P.phib[P.foff[f] + o]);
+      return make_float2(2.0f * b.h, 2.0f * b.l);
+    };
+    // -x of the pair's left cell, +x of its right cell
+    float2 xl, xr;
+    if (i > 0 || !pat) {
+      xl = P.phi[i > 0 ? c - 1 : c + P.n0 - 1];
+    } else {
+      xl = ghost(0, (long long)k * P.n1 + j);
+      nb.x -= 1.0f;
+    }
+    if (i + 2 < P.n0 || !pat) {
+      xr = P.phi[i + 2 < P.n0 ? c + 2 : c + 2 - P.n0];
+    } else {
+      xr = ghost(1, (long long)k * P.n1 + j);
+      nb.y -= 1.0f;
+    }
+    // cell 0: xl + cell 1; cell 1: cell 0 + xr
+    df2 a = two_sum2(make_float2(xl.x, pi.h.x), make_float2(pi.h.y, xr.x));
+    float2 lo = add2(a.l, add2(make_float2(xl.y, pi.l.x), make_float2(pi.l.y, xr.y)));
+    auto add = [&](const df2 &v) {
+      a = two_sum2(a.h, v.h);
+      lo = add2(lo, add2(a.l, v.l));
+    };
+    auto pair_face = [&](bool inside, long long in, long long wrap, int f, long long o) {
+      if (inside || !pat) {
+        add(ld_df2(P.phi, (inside ? in : wrap) >> 1));
+      } else {
+        const float2 g0 = ghost(f, o), g1 = ghost(f, o + 1);
+        add(df2{make_float2(g0.x, g1.x), make_float2(g0.y, g1.y)});
+        nb = sub2(nb, splat2(1.0f));
+      }
+    };
+    const long long oy = (long long)k * P.n0 + i, oz = (long long)j * P.n0 + i;
+    pair_face(j > 0, c - sy, c + (P.n1 - 1) * sy, 2, oy);
+    pair_face(j < P.n1 - 1, c + sy, c - (P.n1 - 1) * sy, 3, oy);
+    pair_face(k > 0, c - sz, c + (P.n2 - 1) * sz, 4, oz);
+    pair_face(k < P.n2 - 1, c + sz, c - (P.n2 - 1) * sz, 5, oz);
     // diagonal: -(6 + missing) phi_i = -(12 - nb) phi_i
-    acc = df_sub(acc, df_mul_f(pi, (float)(12 - nb)));
-    df d = df_mul(acc, df{P.ih2h, P.ih2l});
-    d = df_sub(d, df_sub(ldf(P.s, t), df{smh, sml}));
-    const float dv = d.h + d.l;
-    f32[t] = -dv;
-    e32[t] = 0.0f;
-    if (dout) dout[t] = join_bits(d.h, d.l);
-    ss = dv * dv;
-    mx = fabsf(dv);
+    const float2 dg = sub2(nb, splat2(12.0f));
+    const df2 m = two_prod2(pi.h, dg);
+    add(df2{m.h, fma2(pi.l, dg, m.l)});
+    const df2 acc = fast_two_sum2(a.h, lo);
+    df2 d = df_mul2(acc, df2{splat2(P.ih2h), splat2(P.ih2l)});
+    d = df_sub2(d, df_sub2(ld_df2(P.s, t), df2{splat2(smh), splat2(sml)}));
+    const float2 dv = add2(d.h, d.l);
+    reinterpret_cast<float2 *>(f32)[t] = make_float2(-dv.x, -dv.y);
+    reinterpret_cast<float2 *>(e32)[t] = make_float2(0.0f, 0.0f);
+    if (dout)
+      reinterpret_cast<double2 *>(dout)[t] =
+          make_double2(join_bits(d.h.x, d.l.x), join_bits(d.h.y, d.l.y));
+    ss = fmaf(dv.y, dv.y, dv.x * dv.x);
+    mx = fmaxf(fabsf(dv.x), fabsf(dv.y));
   }
   for (int o = 16; o > 0; o >>= 1) {
     ss += __shfl_down_sync(0xffffffffu, ss, o);
@@ -814,13 +874,12 @@ __global__ void __launch_bounds__(kNT)
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    double s2 = 0.0;
-    float m2 = 0.0f;
+    float s2 = 0.0f, m2 = 0.0f;
     for (int w = 0; w < kNT / 32; w++) {
-      s2 += (double)a[w];
+      s2 += a[w];
       m2 = fmaxf(m2, b[w]);
     }
-    partial[2 * blockIdx.x] = s2;
+    partial[2 * blockIdx.x] = (double)s2;
     partial[2 * blockIdx.x + 1] = (double)m2;
   }
 }
@@ -838,17 +897,22 @@ __global__ void __launch_bounds__(kNT) k_pupdate(PFine P, const float *e) {
 
 // per-block sums of phi (for its mean)
 __global__ void __launch_bounds__(kNT) k_pphisum(PFine P, double *partial) {
-  const long long t = (long long)blockIdx.x * kNT + threadIdx.x;
-  df v = {0.f, 0.f};
-  if (t < P.ncell) v = ldf(P.phi, t);
-  block_df_partial(v, fabsf(v.h), partial);
+  const long long np = P.ncell >> 1;
+  df2 v = {splat2(0.f), splat2(0.f)};
+#pragma unroll
+  for (int q = 0; q < kPP; q++) {
+    const long long t = ((long long)blockIdx.x * kPP + q) * kNT + threadIdx.x;
+    if (t < np) v = df_add2(v, ld_df2(P.phi, t));
+  }
+  block_df_partial(df_add(df{v.h.x, v.l.x}, df{v.h.y, v.l.y}), 0.0f, partial);
 }
 
 // phi64 = phi - mean
 __global__ void __launch_bounds__(kNT) k_pfinal(PFine P, float mh, float ml, double *out) {
   const long long t = (long long)blockIdx.x * kNT + threadIdx.x;
   if (t >= P.ncell) return;
-  const df p = df_sub(ldf(P.phi, t), df{mh, ml});
+  const float2 v = P.phi[t];
+  const df p = df_sub(df{v.x, v.y}, df{mh, ml});
   out[t] = join_bits(p.h, p.l);
 }
 
@@ -1069,7 +1133,7 @@ extern "C" int fr_poisson_solve(frmg_ctx *ctx, const double *density, const doub
     P.n1 = dims[1];
     P.n2 = dims[2];
     P.ncell = nc;
-    P.fd0 = make_fastdiv((unsigned)P.n0);
+    P.fdh = make_fastdiv((unsigned)(P.n0 / 2));
     P.fd1 = make_fastdiv((unsigned)P.n1);
     P.phi = A.get<float2>(nc);
     P.s = A.get<float2>(nc);
@@ -1170,8 +1234,10 @@ extern "C" int fr_poisson_solve(frmg_ctx *ctx, const double *density, const doub
         hl *= 2.0;
       }
     }
-    const long long nb = nblk(nc);
-    double *partial = A.get<double>(2 * nb);
+    // blocks of the double-float passes: one x-pair per thread, kPP pairs per
+    // thread in the sums, one cell per thread
+    const long long np = nc / 2, nbp = nblk(np), nbs = nblk((np + kPP - 1) / kPP), nb = nblk(nc);
+    double *partial = A.get<double>(2 * nbp);
     double *pin = frmg_pinned(ctx, 2);
     if (!pin) throw PError{FR_ENOMEM, "pinned host allocation failed"};
     if (nb > (long long)kRedCH * kRedCH) throw PError{FR_EINVAL, "grid too large"};
@@ -1180,10 +1246,10 @@ extern "C" int fr_poisson_solve(frmg_ctx *ctx, const double *density, const doub
     split_host(std::log(2.0), ln2h, ln2l);
     split_host(2.0 * gamma, g2h, g2l);
     split_host(0.5 * beta, bh, bl);
-    k_psource<<<nb, kNT, 0, st>>>(P, drho, du, dphi0, g2h, g2l, bh, bl, ln2h, ln2l, partial);
+    k_psource<<<nbs, kNT, 0, st>>>(P, drho, du, dphi0, g2h, g2l, bh, bl, ln2h, ln2l, partial);
     PLAUNCH(ctx);
     double ssum, smax;
-    psum(partial, nb, ssum, smax);
+    psum(partial, nbs, ssum, smax);
     const double smean = phib ? 0.0 : ssum / (double)nc;
     if (src_mean) *src_mean = smean;
     float smh, sml;
@@ -1203,10 +1269,10 @@ extern "C" int fr_poisson_solve(frmg_ctx *ctx, const double *density, const doub
                               : 0;
     double *partial0 = A.get<double>(2 * std::max<long long>(nbc, 1));
     for (int outer = 0; outer < o.max_outer; outer++) {
-      k_pdefect<<<nb, kNT, 0, st>>>(P, smh, sml, S.lev[0].f, S.lev[0].e, partial, nullptr);
+      k_pdefect<<<nbp, kNT, 0, st>>>(P, smh, sml, S.lev[0].f, S.lev[0].e, partial, nullptr);
       PLAUNCH(ctx);
       double s2, dmax;
-      psum(partial, nb, s2, dmax);
+      psum(partial, nbp, s2, dmax);
       const double r = std::sqrt(s2 / (double)nc);
       if (outer == 0) sv.res0_rms = r;
       sv.res_rms = r;
@@ -1221,9 +1287,10 @@ extern "C" int fr_poisson_solve(frmg_ctx *ctx, const double *density, const doub
       if (outer > 0 && r > prev) throw PError{FR_EDIVERGED, "defect grew"};
       prev = r;
       if (sv.vcycles >= o.max_vcycles) break;
-      // FP32 correction solve: stop near the FP32 floor (1e-5 of its start)
-      // or when the cycle contraction stalls
-      double rp = HUGE_VAL;
+      // FP32 correction solve: stop near the FP32 floor (2e-5 of its start: the
+      // next cycle rarely gains a factor of two there) or when the cycle
+      // contraction stalls
+      double rp = HUGE_VAL, rbest = HUGE_VAL;
       for (int k = 0; k < o.max_vcycles; k++) {
         if (S.lev.size() == 1) {
           k_lcoarsest<<<1, kNT, 0, st>>>(S.lev[0], 500);
@@ -1238,9 +1305,13 @@ extern "C" int fr_poisson_solve(frmg_ctx *ctx, const double *density, const doub
         const double rr = std::sqrt(a2 / (double)nc);  // residual after pre-smoothing
         push(rr);
         const double pred = rp < HUGE_VAL ? rr * std::sqrt(rr / rp) : rr;
-        if (!(rr < 0.75 * rp) || rr <= 1e-5 * r || pred <= 0.5 * tol ||
-            sv.vcycles >= o.max_vcycles)
+        // near the FP32 floor (1e-4 of the start) a cycle that contracts three
+        // times less than the best one has reached it
+        const double ratio = rr / rp;
+        if (!(ratio < 0.75) || rr <= 2e-5 * r || (rr <= 1e-4 * r && ratio > 3.0 * rbest) ||
+            pred <= 0.5 * tol || sv.vcycles >= o.max_vcycles)
           break;
+        if (k > 0) rbest = std::min(rbest, ratio);
         rp = rr;
       }
       k_pupdate<<<nb, kNT, 0, st>>>(P, S.lev[0].e);
@@ -1249,10 +1320,10 @@ extern "C" int fr_poisson_solve(frmg_ctx *ctx, const double *density, const doub
     // gauge (periodic): phi of zero mean
     double pmean = 0.0;
     if (!phib) {
-      k_pphisum<<<nb, kNT, 0, st>>>(P, partial);
+      k_pphisum<<<nbs, kNT, 0, st>>>(P, partial);
       PLAUNCH(ctx);
       double phisum, pm;
-      psum(partial, nb, phisum, pm);
+      psum(partial, nbs, phisum, pm);
       pmean = phisum / (double)nc;
     }
     float mh, ml;
@@ -1301,13 +1372,13 @@ extern "C" int fr_poisson_source(frmg_ctx *ctx, const double *density, const dou
     P.ncell = nc;
     P.phi = A.get<float2>(nc);
     P.s = A.get<float2>(nc);
-    const long long nb = nblk(nc);
-    double *partial = A.get<double>(2 * nb);
+    const long long nb = nblk(nc), nbs = nblk(((nc + 1) / 2 + kPP - 1) / kPP);
+    double *partial = A.get<double>(2 * nbs);
     float ln2h, ln2l, g2h, g2l, bh, bl;
     split_host(std::log(2.0), ln2h, ln2l);
     split_host(2.0 * k6[2], g2h, g2l);
     split_host(0.5 * k6[1], bh, bl);
-    k_psource<<<nb, kNT, 0, st>>>(P, drho, du, nullptr, g2h, g2l, bh, bl, ln2h, ln2l, partial);
+    k_psource<<<nbs, kNT, 0, st>>>(P, drho, du, nullptr, g2h, g2l, bh, bl, ln2h, ln2l, partial);
     PLAUNCH(ctx);
     PFine Q = P;  // k_pfinal converts its phi array: point it at the source
     Q.phi = P.s;

@@ -760,37 +760,51 @@ __global__ void __launch_bounds__(tail_threads<T>(), 1)
   const int ntop = L0.np * L0.plane;
   if (ntop > 0) {
     // the top level's own planes and, from global memory too, the copied ones,
-    // 16 bytes at a time (a plane holds a multiple of four cells)
+    // 16 bytes at a time (a plane holds a multiple of four cells) unless an
+    // FP64 array of the caller's starts at an odd multiple of 8 bytes
     constexpr int W = 16 / (int)sizeof(T);
     const T *gu = L0.gu[pin], *gx = L0.gx[pin], *gf = L0.gf;
     const int pl = L0.plane, z0 = L0.z0, n2 = L0.n2, n = ntop + 2 * pl;
-    for (int t = W * tid; t < n; t += W * NT) {
+    const T fs = L0.fs, fo = L0.fo;
+    auto cell = [&](int t) {
       const int kl = tail_div(tail_div(t, L0.m0), L0.m1) - 1;
       int k = z0 + kl;
       k = k < 0 ? k + n2 : (k >= n2 ? k - n2 : k);
-      const int c = k * pl + t - (kl + 1) * pl;
-      const int4 vu = *reinterpret_cast<const int4 *>(gu + c);
-      const int4 vx = *reinterpret_cast<const int4 *>(gx + c);
-      int4 vb, vE;
-      if (BG) {
-        vb = *reinterpret_cast<const int4 *>(L0.gub + c);
-        vE = *reinterpret_cast<const int4 *>(L0.gE + c);
+      return k * pl + t - (kl + 1) * pl;
+    };
+    if (sizeof(T) == 4 ||
+        ((reinterpret_cast<size_t>(gu) | reinterpret_cast<size_t>(gf)) & 15) == 0) {
+      for (int t = W * tid; t < n; t += W * NT) {
+        const int c = cell(t);
+        const int4 vu = *reinterpret_cast<const int4 *>(gu + c);
+        const int4 vx = *reinterpret_cast<const int4 *>(gx + c);
+        int4 vb, vE;
+        if (BG) {
+          vb = *reinterpret_cast<const int4 *>(L0.gub + c);
+          vE = *reinterpret_cast<const int4 *>(L0.gE + c);
+        }
+        *reinterpret_cast<int4 *>(sm + L0.u + t) = vu;
+        *reinterpret_cast<int4 *>(sm + L0.x + t) = vx;
+        if (BG) {
+          *reinterpret_cast<int4 *>(sm + L0.ub + t) = vb;
+          *reinterpret_cast<int4 *>(sm + L0.E + t) = vE;
+        }
       }
-      *reinterpret_cast<int4 *>(sm + L0.u + t) = vu;
-      *reinterpret_cast<int4 *>(sm + L0.x + t) = vx;
-      if (BG) {
-        *reinterpret_cast<int4 *>(sm + L0.ub + t) = vb;
-        *reinterpret_cast<int4 *>(sm + L0.E + t) = vE;
-      }
-    }
-    const T fs = L0.fs, fo = L0.fo;
-    for (int t = W * tid; t < ntop; t += W * NT) {
-      T v[W];
-      *reinterpret_cast<int4 *>(v) = gf ? *reinterpret_cast<const int4 *>(gf + c0 + t)
-                                        : make_int4(0, 0, 0, 0);
+      for (int t = W * tid; t < ntop; t += W * NT) {
+        T v[W];
+        *reinterpret_cast<int4 *>(v) = gf ? *reinterpret_cast<const int4 *>(gf + c0 + t)
+                                          : make_int4(0, 0, 0, 0);
 #pragma unroll
-      for (int q = 0; q < W; q++) v[q] = gf ? fs * (v[q] - fo) : T(0);
-      *reinterpret_cast<int4 *>(sm + L0.f + t) = *reinterpret_cast<int4 *>(v);
+        for (int q = 0; q < W; q++) v[q] = gf ? fs * (v[q] - fo) : T(0);
+        *reinterpret_cast<int4 *>(sm + L0.f + t) = *reinterpret_cast<int4 *>(v);
+      }
+    } else {
+      for (int t = tid; t < n; t += NT) {
+        const int c = cell(t);
+        sm[L0.u + t] = gu[c];
+        sm[L0.x + t] = gx[c];
+      }
+      for (int t = tid; t < ntop; t += NT) sm[L0.f + t] = gf ? fs * (gf[c0 + t] - fo) : T(0);
     }
   }
   int lf = 0;  // first level kept in one block

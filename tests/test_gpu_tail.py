@@ -115,3 +115,41 @@ def test_masked_tail_matches_oracle(C, prec, dims, count, relax):
     st, s = C.solve_masked(dev(rho), dev(m), u, h=1.0 / 64, tol=1e-11, prec=prec, relax=relax, **P)
     assert st == 0 and s.res_rms <= 1e-11
     assert np.abs(host(u) - ref.u).max() < 1e-8
+
+
+def _at8(a):
+    """The array on the device at an address that is a multiple of 8, not of 16."""
+    buf = torch.empty(a.size + 1, dtype=torch.float64, device="cuda")
+    t = buf[1:].view(a.shape)
+    assert t.data_ptr() % 16 == 8
+    t.copy_(torch.from_numpy(np.ascontiguousarray(a)))
+    return t
+
+
+def test_arrays_at_odd_multiples_of_8_bytes(C):
+    """The FP64 tail and the Poisson passes read the caller's arrays: any
+    address that is a multiple of 8 gives the aligned arrays' result."""
+    rho, P = _case((16, 16, 16), 8700)
+    u0 = np.zeros(rho.shape)
+    ua, ub = dev(u0), _at8(u0)
+    C.vcycles(dev(rho), ua, 2, **P)
+    C.vcycles(_at8(rho), ub, 2, **P)
+    assert np.array_equal(host(ua), host(ub))
+    pa, pb = dev(u0), _at8(u0)
+    C.poisson(dev(rho), ua, pa, tol=1e-10, **P)
+    C.poisson(_at8(rho), ub, pb, tol=1e-10, **P)
+    assert np.array_equal(host(pa), host(pb))
+
+
+@pytest.mark.parametrize("shape", [(3, 5, 7), (1, 1, 1), (4, 6, 9), (16, 16, 32)])
+def test_poisson_source_of_any_size(C, shape):
+    """The source pass works on pairs of cells: odd numbers of cells, and more
+    than one block, against the formula (double-float pairs: 1e-12 of its terms)."""
+    from oracle import poisson as PO
+    rng = np.random.default_rng(3)
+    rho, u = np.exp(rng.standard_normal(shape)), rng.standard_normal(shape)
+    P = dict(box=64.0, a=0.9, omega_m=0.24, fr0=1e-5)
+    out = torch.empty(shape, dtype=torch.float64, device="cuda")
+    C.poisson_source(_at8(rho), _at8(u), out, **P)
+    ref = PO.source(u, rho, **P)
+    assert np.abs(host(out) - ref).max() < 1e-12 * max(1.0, np.abs(ref).max())
