@@ -23,6 +23,7 @@
 // phi += e.  On a periodic grid the equation has a solution only for a source
 // of zero mean, so the source's mean is removed (and reported) and phi is
 // returned with zero mean.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -687,6 +688,367 @@ __global__ void __launch_bounds__(kNT) k_lcoarsest(PLevel L, int maxit) {
   }
 }
 
+// ---- the small levels of a V-cycle in one cluster
+//
+// As the f(R) solver's tail (frmg_tail.cuh): the levels from one of at most
+// kLtCells cells down to the coarsest and back up run in one launch, each
+// level's planes dealt out to the blocks of one thread-block cluster, e and f in
+// shared memory, with copies of the e planes above and below a block's own
+// that their owner keeps up to date; levels of at most kLtLocal cells live in the
+// first block.  A launch per step costs 3 to 4 us of host and launch time on
+// these levels, ten steps per level (V(2,2)).  Same updates as k_lsmooth, k_lresid_restrict,
+// k_lprolong and k_lcoarsest (whose sums are added in another order).
+namespace cg = cooperative_groups;
+
+constexpr int kLtNT = 512, kLtLev = 8, kLtCluster = 16;
+constexpr long long kLtCells = 110592;  // 48^3: what fits 16 blocks' shared memory
+constexpr int kLtLocal = 4096;          // 16^3: a step of one block is shorter than a barrier
+
+struct LtLevel {
+  int n0, n1, n2, hx, plane, zc, local;
+  unsigned e, f, d, g;       // arrays in shared memory: e (with the copies), f, residual,
+                             // the coarser level's correction that the own planes take
+  unsigned mh, m0, m1, mz;   // division by hx, n0, n1, zc: (t m) >> 32
+  float h2;
+  float *ge, *gf;            // the level's arrays in global memory
+  int z0, np, below, above, belowo;
+};
+struct LtDesc {
+  int nl, patch, pre, post;
+  float relax;
+  LtLevel lev[kLtLev];
+};
+
+// Lays out nl levels on clusters of cs blocks; returns the bytes per block.
+size_t lt_layout(LtDesc &D, const PLevel *lev, int nl, int cs) {
+  auto magic = [](int d) {
+    return d <= 1 ? 0u : (unsigned)(((1ull << 32) + (unsigned)d - 1) / (unsigned)d);
+  };
+  unsigned end = 0;
+  D.nl = nl;
+  for (int l = 0; l < nl; l++) {
+    LtLevel &L = D.lev[l];
+    const PLevel &G = lev[l];
+    L.n0 = G.n0;
+    L.n1 = G.n1;
+    L.n2 = G.n2;
+    L.hx = G.n0 / 2;
+    L.plane = G.n0 * G.n1;
+    L.local = G.ncell <= kLtLocal;
+    L.zc = L.local ? G.n2 : (G.n2 + cs - 1) / cs;
+    L.mh = magic(L.hx);
+    L.m0 = magic(L.n0);
+    L.m1 = magic(L.n1);
+    L.mz = magic(L.zc);
+    L.h2 = G.h2;
+    L.ge = G.e;
+    L.gf = G.f;
+    L.e = end;
+    L.f = L.e + (unsigned)((L.zc + 2) * L.plane);
+    L.d = L.f + (unsigned)(L.zc * L.plane);
+    L.g = L.d + (unsigned)(L.zc * L.plane);
+    end = L.g + (unsigned)((L.zc / 2 + 3) * (L.plane / 4 + 1));
+  }
+  return (size_t)end * sizeof(float);
+}
+
+struct LtBlock {
+  LtDesc D;
+  int cs, me;
+  float red[kLtNT / 32], slots[kLtCluster];
+};
+
+__device__ __forceinline__ float *lt_smem() {
+  extern __shared__ __align__(16) float lt_smem_raw[];
+  return lt_smem_raw;
+}
+__device__ __forceinline__ void lt_sync(bool all) {
+  if (all) cg::this_cluster().sync();
+  else __syncthreads();
+}
+__device__ __forceinline__ float *lt_remote(float *p, int r) {
+  return cg::this_cluster().map_shared_rank(p, r);
+}
+__device__ __forceinline__ int lt_div(int t, unsigned m) {
+  return m ? (int)__umulhi((unsigned)t, m) : t;
+}
+
+// Writes e of the own planes, and the neighbours' copies of the outer ones.
+template <bool PATCH>
+struct LtPut {
+  float *sm, *below, *above;
+  int plane, last, belowo;
+  unsigned e;
+  __device__ __forceinline__ explicit LtPut(const LtLevel &L)
+      : sm(lt_smem()), plane(L.plane), last(L.np - 1), belowo(L.belowo), e(L.e) {
+    below = PATCH && L.z0 == 0 ? nullptr : lt_remote(sm, L.below);
+    above = PATCH && L.z0 + L.np == L.n2 ? nullptr : lt_remote(sm, L.above);
+  }
+  __device__ __forceinline__ void operator()(float v, int kl, int q) const {
+    sm[e + (kl + 1) * plane + q] = v;
+    if (kl == 0 && (!PATCH || below)) below[e + belowo + q] = v;
+    if (kl == last && (!PATCH || above)) above[e + q] = v;
+  }
+};
+
+// Sum of the six neighbours (in the grid) of cell (i, j) of own plane kl.
+template <bool PATCH>
+__device__ __forceinline__ float lt_nbsum(const LtLevel &L, int i, int j, int kl, float &own,
+                                          int &nm) {
+  const float *sm = lt_smem();
+  const int n0 = L.n0, pl = L.plane, o = (int)L.e + (kl + 1) * pl + j * n0 + i;
+  const bool b[6] = {i == 0, i == n0 - 1, j == 0, j == L.n1 - 1, L.z0 + kl == 0,
+                     L.z0 + kl == L.n2 - 1};
+  const int wx = n0 - 1, wy = pl - n0;
+  const float v[6] = {sm[b[0] ? o + wx : o - 1],  sm[b[1] ? o - wx : o + 1],
+                      sm[b[2] ? o + wy : o - n0], sm[b[3] ? o - wy : o + n0],
+                      sm[o - pl],                 sm[o + pl]};
+  own = sm[o];
+  float s = 0.0f;
+  nm = 0;
+#pragma unroll
+  for (int q = 0; q < 6; q++) {
+    if (PATCH && b[q]) nm++;
+    else s += v[q];
+  }
+  return s;
+}
+
+template <bool PATCH>
+__device__ __noinline__ void lt_smooth(const LtBlock &B, int l, int sweeps, float relax,
+                                       bool all) {
+  const LtLevel &L = B.D.lev[l];
+  const float *sm = lt_smem();
+  const LtPut<PATCH> put(L);
+  const int n = L.np * L.n1 * L.hx;
+  for (int s = 0; s < 2 * sweeps; s++) {
+    for (int t = threadIdx.x; t < n; t += kLtNT) {
+      const int q = lt_div(t, L.mh), kl = lt_div(q, L.m1), j = q - kl * L.n1;
+      const int i = 2 * (t - q * L.hx) + ((j + L.z0 + kl + s) & 1);
+      float own;
+      int nm;
+      const float sum = lt_nbsum<PATCH>(L, i, j, kl, own, nm);
+      const float gs = gs_value(sum, L.h2 * sm[L.f + kl * L.plane + j * L.n0 + i], nm);
+      put(fmaf(relax, gs - own, own), kl, j * L.n0 + i);
+    }
+    lt_sync(all);
+  }
+}
+
+// d = f - L e on the own planes; returns this thread's sum of d^2.
+template <bool PATCH>
+__device__ __noinline__ float lt_resid(const LtBlock &B, int l) {
+  const LtLevel &L = B.D.lev[l];
+  float *sm = lt_smem();
+  const int n = L.np * L.plane;
+  float ss = 0.0f;
+  for (int t = threadIdx.x; t < n; t += kLtNT) {
+    const int q = lt_div(t, L.m0), kl = lt_div(q, L.m1), j = q - kl * L.n1, i = t - q * L.n0;
+    float own;
+    int nm;
+    const float sum = lt_nbsum<PATCH>(L, i, j, kl, own, nm);
+    const float d = sm[L.f + t] - (sum - (6.0f + (float)nm) * own) / L.h2;
+    sm[L.d + t] = d;
+    ss = fmaf(d, d, ss);
+  }
+  return ss;
+}
+
+// f of level l + 1 = mean of the children's d, e = 0 (own planes and copies)
+__device__ __noinline__ void lt_restrict(const LtBlock &B, int l, bool all) {
+  const LtLevel &F = B.D.lev[l], &C = B.D.lev[l + 1];
+  float *sm = lt_smem();
+  const int n = C.np * C.plane;
+  if (n > 0)
+    for (int t = threadIdx.x; t < n + 2 * C.plane; t += kLtNT) sm[C.e + t] = 0.0f;
+  for (int t = threadIdx.x; t < n; t += kLtNT) {
+    const int q = lt_div(t, C.m0), Kl = lt_div(q, C.m1), J = q - Kl * C.n1, I = t - q * C.n0;
+    float sd = 0.0f;
+#pragma unroll
+    for (int z = 0; z < 2; z++) {
+      const int k = 2 * (C.z0 + Kl) + z, r = lt_div(k, F.mz);
+      const float *p = lt_remote(sm, r) + F.d + (k - r * F.zc) * F.plane + 2 * J * F.n0 + 2 * I;
+      sd += p[0];
+      sd += p[1];
+      sd += p[F.n0];
+      sd += p[F.n0 + 1];
+    }
+    sm[C.f + t] = 0.125f * sd;
+  }
+  lt_sync(all);
+}
+
+template <bool PATCH>
+__device__ __noinline__ void lt_prolong(const LtBlock &B, int l, bool all) {
+  const LtLevel &F = B.D.lev[l], &C = B.D.lev[l + 1];
+  float *sm = lt_smem();
+  const int n = F.np * F.plane, K0 = (F.z0 >> 1) - 1;
+  if (n > 0) {
+    const int ne = (((F.z0 + F.np - 1) >> 1) + 2 - K0) * C.plane;
+    for (int t = threadIdx.x; t < ne; t += kLtNT) {
+      const int s = lt_div(lt_div(t, C.m0), C.m1), q = t - s * C.plane;
+      int K = K0 + s;
+      const bool out = K < 0 || K >= C.n2;
+      K = K < 0 ? K + C.n2 : (K >= C.n2 ? K - C.n2 : K);
+      const int r = lt_div(K, C.mz);
+      const float v = lt_remote(sm, r)[C.e + (K - r * C.zc + 1) * C.plane + q];
+      sm[F.g + t] = PATCH && out ? 0.0f : v;
+    }
+  }
+  __syncthreads();
+  const LtPut<PATCH> put(F);
+  for (int t = threadIdx.x; t < n; t += kLtNT) {
+    const int q = lt_div(t, F.m0), kl = lt_div(q, F.m1), j = q - kl * F.n1, i = t - q * F.n0;
+    const int k = F.z0 + kl, I = i >> 1, J = j >> 1, K = k >> 1;
+    const int di = (i & 1) ? 1 : -1, dj = (j & 1) ? 1 : -1, dk = (k & 1) ? 1 : -1;
+    float acc = 0.0f;
+#pragma unroll
+    for (int c = 0; c < 8; c++) {
+      int ii = I + ((c & 1) ? di : 0), jj = J + (((c >> 1) & 1) ? dj : 0);
+      const int kk = K + ((c >> 2) ? dk : 0);
+      const float w = ((c & 1) ? 0.25f : 0.75f) * (((c >> 1) & 1) ? 0.25f : 0.75f) *
+                      ((c >> 2) ? 0.25f : 0.75f);
+      const bool in = !PATCH || (ii >= 0 && ii < C.n0 && jj >= 0 && jj < C.n1);
+      ii = ii < 0 ? ii + C.n0 : (ii >= C.n0 ? ii - C.n0 : ii);
+      jj = jj < 0 ? jj + C.n1 : (jj >= C.n1 ? jj - C.n1 : jj);
+      const float v = sm[F.g + (kk - K0) * C.plane + jj * C.n0 + ii];
+      if (in) acc = fmaf(w, v, acc);
+    }
+    put(sm[F.e + F.plane + t] + acc, kl, t - kl * F.plane);
+  }
+  lt_sync(all);
+}
+
+// Gauss-Seidel sweeps to k_lcoarsest's stopping rule.
+template <bool PATCH>
+__device__ __noinline__ void lt_coarsest(LtBlock &B, int l, int maxit, bool all) {
+  const float cells = (float)(B.D.lev[l].n2 * B.D.lev[l].plane);
+  float r0 = 0.0f, prev = 0.0f;
+  for (int it = -1; it < maxit; it++) {
+    if (it >= 0) lt_smooth<PATCH>(B, l, 1, 1.0f, all);
+    float ss = lt_resid<PATCH>(B, l);
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) B.red[threadIdx.x >> 5] = ss;
+    __syncthreads();
+    ss = lane < kLtNT / 32 ? B.red[lane] : 0.0f;
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    if (all) {
+      if ((int)threadIdx.x < B.cs) lt_remote(B.slots, threadIdx.x)[B.me] = ss;
+      lt_sync(true);
+      ss = 0.0f;
+      for (int q = 0; q < B.cs; q++) ss += B.slots[q];
+    }
+    const float r = sqrtf(ss / cells);
+    lt_sync(all);  // the sums have been read
+    if (it < 0) r0 = r;
+    else if (r <= 1e-3f * r0 || !(r < prev)) return;
+    prev = r;
+  }
+}
+
+template <bool PATCH>
+__global__ void __launch_bounds__(kLtNT, 1) k_ltail(const LtDesc *desc) {
+  __shared__ LtBlock B;
+  float *sm = lt_smem();
+  const int tid = threadIdx.x;
+  const int cs = (int)cg::this_cluster().num_blocks(), me = (int)cg::this_cluster().block_rank();
+  {
+    const int *src = reinterpret_cast<const int *>(desc);
+    int *dst = reinterpret_cast<int *>(&B.D);
+    for (int t = tid; t < (int)(sizeof(LtDesc) / sizeof(int)); t += kLtNT) dst[t] = src[t];
+  }
+  __syncthreads();
+  const int nl = B.D.nl, pre = B.D.pre, post = B.D.post;
+  const float relax = B.D.relax;
+  if (tid < nl) {
+    LtLevel &L = B.D.lev[tid];
+    L.z0 = min(me * L.zc, L.n2);
+    L.np = min(L.zc, L.n2 - L.z0);
+    const int lo = L.z0 > 0 ? L.z0 - 1 : L.n2 - 1;
+    const int hi = L.z0 + L.np < L.n2 ? L.z0 + L.np : 0;
+    L.below = lt_div(lo, L.mz);
+    L.above = lt_div(hi, L.mz);
+    L.belowo = (lo - L.below * L.zc + 2) * L.plane;
+  }
+  if (tid == 0) {
+    B.cs = cs;
+    B.me = me;
+  }
+  __syncthreads();
+  const LtLevel &T = B.D.lev[0];
+  const long long c0 = (long long)T.z0 * T.plane;
+  const int ntop = T.np * T.plane;
+  // the top level: f from global memory, e = 0
+  for (int t = tid; t < ntop; t += kLtNT) sm[T.f + t] = T.gf[c0 + t];
+  if (ntop > 0)
+    for (int t = tid; t < ntop + 2 * T.plane; t += kLtNT) sm[T.e + t] = 0.0f;
+  int lf = 0;  // first level kept in one block
+  while (lf < nl && !B.D.lev[lf].local) lf++;
+  lt_sync(true);
+  for (int l = 0; l < lf; l++) {
+    if (l == nl - 1) {
+      lt_coarsest<PATCH>(B, l, 500, true);
+      break;
+    }
+    lt_smooth<PATCH>(B, l, pre, relax, true);
+    lt_resid<PATCH>(B, l);
+    lt_sync(true);
+    if (l + 1 < lf) lt_restrict(B, l, true);
+  }
+  if (lf < nl) {
+    if (me == 0) {
+      if (lf > 0) lt_restrict(B, lf - 1, false);
+      for (int l = lf; l < nl - 1; l++) {
+        lt_smooth<PATCH>(B, l, pre, relax, false);
+        lt_resid<PATCH>(B, l);
+        __syncthreads();
+        lt_restrict(B, l, false);
+      }
+      lt_coarsest<PATCH>(B, nl - 1, 500, false);
+      for (int l = nl - 2; l >= lf; l--) {
+        lt_prolong<PATCH>(B, l, false);
+        lt_smooth<PATCH>(B, l, post, relax, false);
+      }
+    }
+    lt_sync(true);
+  }
+  for (int l = min(lf, nl - 1) - 1; l >= 0; l--) {
+    lt_prolong<PATCH>(B, l, true);
+    lt_smooth<PATCH>(B, l, post, relax, true);
+  }
+  for (int t = tid; t < ntop; t += kLtNT) T.ge[c0 + t] = sm[T.e + T.plane + t];
+}
+
+// Blocks per cluster the device takes (16 where it can).
+constexpr size_t kLtSmem = 220 * 1024;
+template <bool PATCH>
+int lt_cluster() {
+  static int best = 0;
+  if (!best) {
+    auto *k = k_ltail<PATCH>;
+    PCK(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    PCK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLtSmem));
+    for (int cs = kLtCluster; cs > 0 && !best; cs /= 2) {
+      cudaLaunchConfig_t c = {};
+      c.gridDim = dim3(cs);
+      c.blockDim = dim3(kLtNT);
+      c.dynamicSmemBytes = kLtSmem;
+      cudaLaunchAttribute a[1];
+      a[0].id = cudaLaunchAttributeClusterDimension;
+      a[0].val.clusterDim.x = cs;
+      a[0].val.clusterDim.y = a[0].val.clusterDim.z = 1;
+      c.attrs = a;
+      c.numAttrs = 1;
+      int n = 0;
+      if (cudaOccupancyMaxActiveClusters(&n, k, &c) == cudaSuccess && n > 0) best = cs;
+      else cudaGetLastError();
+    }
+    if (!best) best = 1;
+  }
+  return best;
+}
+
 // ---- double-float fine level
 
 struct PFine {
@@ -1030,6 +1392,56 @@ struct PoissonSolver {
   std::vector<int> kc_p, nblk_p;  // tiled prolongation onto a level: coarse planes per block
                                   // and blocks (0: one thread per fine cell)
   std::vector<int> kc_r, nblk_r;  // tiled residual + restriction from a level (same layout)
+  int tail = 1 << 30;     // first level of the one-cluster tail (none)
+  LtDesc *tail_d = nullptr;
+  int tail_cs = 1;
+  size_t tail_smem = 0;
+
+  // The tail begins at the first level below the finest whose levels fit it.
+  void set_tail(Arena &A) {
+    const int nl = (int)lev.size();
+    const bool patch = lev[0].patch != 0;
+    // a coarsest grid of odd sides keeps the launched levels (x-pairs)
+    if (lev.back().n0 % 2 || lev.back().n1 % 2 || lev.back().n2 % 2) return;
+    const int cs = patch ? lt_cluster<true>() : lt_cluster<false>();
+    LtDesc D, best;
+    memset(&D, 0, sizeof(D));
+    D.patch = patch;
+    D.pre = pre;
+    D.post = post;
+    D.relax = lev[0].relax;
+    int at = nl;
+    for (int l = nl - 1; l >= 1 && nl - l <= kLtLev && lev[l].ncell <= kLtCells; l--) {
+      const int c = lev[l].ncell <= kLtLocal ? 1 : cs;
+      const size_t b = lt_layout(D, &lev[l], nl - l, c);
+      if (b > kLtSmem) break;
+      at = l;
+      best = D;
+      tail_cs = c;
+      tail_smem = b;
+    }
+    if (at == nl) return;
+    tail = at;
+    tail_d = A.get<LtDesc>(1);
+    PCK(cudaMemcpyAsync(tail_d, &best, sizeof(best), cudaMemcpyHostToDevice, st));
+    PCK(cudaStreamSynchronize(st));  // best has been read
+  }
+  template <bool PATCH>
+  void run_tail() {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3((unsigned)tail_cs);
+    c.blockDim = dim3(kLtNT);
+    c.dynamicSmemBytes = tail_smem;
+    c.stream = st;
+    cudaLaunchAttribute a[1];
+    a[0].id = cudaLaunchAttributeClusterDimension;
+    a[0].val.clusterDim.x = tail_cs;
+    a[0].val.clusterDim.y = a[0].val.clusterDim.z = 1;
+    c.attrs = a;
+    c.numAttrs = 1;
+    PCK(cudaLaunchKernelEx(&c, k_ltail<PATCH>, (const LtDesc *)tail_d));
+    PLAUNCH(ctx);
+  }
 
   void smooth(int l, int n) {
     for (int it = 0; it < n; it++) {
@@ -1050,6 +1462,11 @@ struct PoissonSolver {
     }
   }
   void vcycle(int l, double *partial0) {
+    if (l == tail) {
+      if (lev[l].patch) run_tail<true>();
+      else run_tail<false>();
+      return;
+    }
     if (l == (int)lev.size() - 1) {
       k_lcoarsest<<<1, kNT, 0, st>>>(lev[l], 500);
       PLAUNCH(ctx);
@@ -1234,6 +1651,7 @@ extern "C" int fr_poisson_solve(frmg_ctx *ctx, const double *density, const doub
         hl *= 2.0;
       }
     }
+    S.set_tail(A);
     // blocks of the double-float passes: one x-pair per thread, kPP pairs per
     // thread in the sums, one cell per thread
     const long long np = nc / 2, nbp = nblk(np), nbs = nblk((np + kPP - 1) / kPP), nb = nblk(nc);
