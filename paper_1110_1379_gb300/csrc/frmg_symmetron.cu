@@ -152,6 +152,13 @@ __device__ __forceinline__ T sy_rhs(const SLevel<T> &L, long long c) {
   return L.f ? L.f[c] : T(0);
 }
 
+// Newton step -w r / dN.  FP32 by the hardware reciprocal (the step's last bits
+// do not move the solution; an IEEE division is about ten instructions).
+__device__ __forceinline__ double sy_step(double r, double dN, double w) { return -w * r / dN; }
+__device__ __forceinline__ float sy_step(float r, float dN, float w) {
+  return __fdividef(-w * r, dN);
+}
+
 // One colour of a red-black Newton-Gauss-Seidel sweep (red = (i + j + k) even).
 template <typename T, bool CORR>
 __global__ void __launch_bounds__(kNT) k_sy_smooth(SLevel<T> L, int colour) {
@@ -163,7 +170,7 @@ __global__ void __launch_bounds__(kNT) k_sy_smooth(SLevel<T> L, int colour) {
   T N, dN;
   sy_op<T, CORR>(L, i, j, k, N, dN);
   const long long c = ((long long)k * L.n1 + j) * L.n0 + i;
-  T du = -L.relax * (N - sy_rhs(L, c)) / dN;
+  T du = sy_step(N - sy_rhs(L, c), dN, L.relax);
   du = du > L.cap ? L.cap : (du < -L.cap ? -L.cap : du);
   L.u[c] += du;
 }
@@ -335,7 +342,7 @@ __global__ void __launch_bounds__(kNT) k_sy_coarsest(SLevel<T> L, double rel, do
         T N, dN;
         sy_op<T, CORR>(L, i, j, k, N, dN);
         const long long c = ((long long)k * L.n1 + j) * L.n0 + i;
-        T du = -L.relax * (N - sy_rhs(L, c)) / dN;
+        T du = sy_step(N - sy_rhs(L, c), dN, L.relax);
         du = du > L.cap ? L.cap : (du < -L.cap ? -L.cap : du);
         L.u[c] += du;
       }
@@ -470,7 +477,7 @@ __global__ void __launch_bounds__(kNT, 3)
     const float lap = (lf - d) + (rt - d) + (ym - d) + (yp - d) + (zm - d) + (zp - d);
     const float N = A * lap - d * (c.y + d * (c.z + d));
     const float dN = -6.0f * A - (c.y + d * (2.0f * c.z + 3.0f * d));
-    float du = -relax * (N - c.w) / dN;
+    float du = sy_step(N - c.w, dN, relax);
     du = fminf(fmaxf(du, -cap), cap);
     return d + du;
   };
@@ -533,23 +540,46 @@ __global__ void __launch_bounds__(kNT, 3)
   }
 }
 
-// 8-child average of an array (coarse dims c0 x c1 x c2).
-template <typename S, typename D>
-__global__ void __launch_bounds__(kNT) k_sy_restrict(const S *fine, D *coarse, int c0, int c1,
-                                                     int c2) {
+// 8-child average of an array (coarse dims c0 x c1 x c2).  FP32: the children's
+// sum with its rounding errors carried along (TwoSum), as good as an FP64 sum
+// without the FP64 pipe (0.55 ms at 512^3 with FP64 conversions and additions).
+template <typename T>
+__global__ void __launch_bounds__(kNT) k_sy_restrict(const T *fine, T *coarse, int c0, int c1,
+                                                     int c2, frmg::FastDiv fd0,
+                                                     frmg::FastDiv fd1) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long nc = (long long)c0 * c1 * c2;
   if (t >= nc) return;
-  const int I = (int)(t % c0);
-  const long long r = t / c0;
-  const int J = (int)(r % c1), K = (int)(r / c1);
-  const int f0 = 2 * c0, f1 = 2 * c1;
-  double s = 0.0;
-  for (int q = 0; q < 8; q++) {
-    const int i = 2 * I + (q & 1), j = 2 * J + ((q >> 1) & 1), k = 2 * K + (q >> 2);
-    s += (double)fine[((long long)k * f1 + j) * f0 + i];
+  int I, J, K;
+  if (nc < (1ll << 31)) {
+    const unsigned tu = (unsigned)t, q = frmg::fdiv(tu, fd0), q2 = frmg::fdiv(q, fd1);
+    I = (int)(tu - q * (unsigned)c0);
+    J = (int)(q - q2 * (unsigned)c1);
+    K = (int)q2;
+  } else {
+    I = (int)(t % c0);
+    const long long r = t / c0;
+    J = (int)(r % c1);
+    K = (int)(r / c1);
   }
-  coarse[t] = (D)(s * 0.125);
+  const long long f0 = 2 * c0, f1 = 2 * c1;
+  T s = T(0), e = T(0);
+#pragma unroll
+  for (int q = 0; q < 4; q++) {
+    const T *row = fine + ((2ll * K + (q >> 1)) * f1 + 2 * J + (q & 1)) * f0 + 2 * I;
+    const T v[2] = {row[0], row[1]};
+#pragma unroll
+    for (int x = 0; x < 2; x++) {
+      if constexpr (sizeof(T) == 4) {
+        const frmg::df w = frmg::two_sum(s, v[x]);
+        s = w.h;
+        e += w.l;
+      } else {
+        s += v[x];
+      }
+    }
+  }
+  coarse[t] = (s + e) * T(0.125);
 }
 
 // FP64 residual of the full equation, d = L(chi), with norm partials.
@@ -572,25 +602,44 @@ __global__ void __launch_bounds__(kNT) k_sy_fill(double *v, double x, long long 
   if (t < n) v[t] = x;
 }
 
-template <typename S, typename D>
-__global__ void __launch_bounds__(kNT) k_sy_convert(const S *in, D *out, long long n) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < n) out[t] = (D)in[t];
-}
-
 // ---- double-float outer loop of the mixed solve (FP64 accuracy on the FP32
-// pipes, see frmg_dfmath.cuh): chi and rho are held as (hi, lo) pairs.
+// pipes, see frmg_dfmath.cuh): chi and rho are held as (hi, lo) pairs, split and
+// joined with integer operations.
 __global__ void __launch_bounds__(kNT) k_sy_split(const double *v, float2 *p, long long n) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
-  const double x = v[t];
-  const float h = (float)x;
-  p[t] = make_float2(h, (float)(x - (double)h));
+  const frmg::df x = frmg::split_bits(v[t]);
+  p[t] = make_float2(x.h, x.l);
+}
+
+__global__ void __launch_bounds__(kNT) k_sy_fill2(float2 *p, float h, float l, long long n) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < n) p[t] = make_float2(h, l);
+}
+
+// The density in one pass: its check (finite and, being a mass density, >= 0),
+// its pairs and its FP32 copy.  (Three passes, the split on the FP64 pipe, took
+// 1.67 ms at 512^3.)
+__device__ __forceinline__ bool sy_bad_rho(double r) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(r);
+  return ((b >> 52) & 0x7ffu) == 0x7ffu || ((b >> 63) && (b << 1) != 0);
+}
+__global__ void __launch_bounds__(kNT) k_sy_rho(const double *rho, float2 *p, float *f,
+                                                long long n, int *bad) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  const double r = rho[t];
+  if (sy_bad_rho(r)) atomicOr(bad, 1);
+  const frmg::df x = frmg::split_bits(r);
+  p[t] = make_float2(x.h, x.l);
+  f[t] = x.h;
 }
 
 __global__ void __launch_bounds__(kNT) k_sy_join(const float2 *p, double *v, long long n) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < n) v[t] = (double)p[t].x + (double)p[t].y;
+  if (t >= n) return;
+  const float2 x = p[t];
+  v[t] = frmg::join_bits(x.x, x.y);
 }
 
 // Defect of chi in double-float, two cells (an x-pair; every grid has an even
@@ -671,33 +720,18 @@ __global__ void __launch_bounds__(kNT) k_sy_reduce_chunks(const double *in, long
 // density check: finite and, the model's density being a mass density, >= 0
 __global__ void __launch_bounds__(kNT) k_sy_check_rho(const double *rho, long long n, int *bad) {
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < n) {
-    const double r = rho[t];
-    if (!(r >= 0.0) || isinf(r)) atomicOr(bad, 1);
-  }
+  if (t < n && sy_bad_rho(rho[t])) atomicOr(bad, 1);
 }
 
 // sum and max of per-block partial pairs, one block, fixed order
 __global__ void __launch_bounds__(kNT) k_sy_reduce(const double *part, long long nb,
                                                    double *out) {
-  __shared__ double ss[kNT], sm[kNT];
   double s = 0.0, m = 0.0;
   for (long long b = threadIdx.x; b < nb; b += kNT) {
     s += part[2 * b];
     m = fmax(m, part[2 * b + 1]);
   }
-  ss[threadIdx.x] = s;
-  sm[threadIdx.x] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double ts = 0.0, tm = 0.0;
-    for (int q = 0; q < kNT; q++) {
-      ts += ss[q];
-      tm = fmax(tm, sm[q]);
-    }
-    out[0] = ts;
-    out[1] = tm;
-  }
+  sy_block_norms<double>(s, m, out);
 }
 
 long long nblk(long long n) { return (n + kNT - 1) / kNT; }
@@ -819,20 +853,30 @@ extern "C" int fr_symmetron_solve(frmg_ctx *ctx, const double *density, const in
     double *chi = chi_inout;
     if (!chi_dev) chi = A.get<double>(nc);
     const double s = std::pow(a_ssb / a, 3.0);
+    // the homogeneous solution on the positive branch (1 before symmetry
+    // breaking, from where the field relaxes to its symmetric value 0)
+    const double chib = s < 1.0 ? std::sqrt(1.0 - s) : 1.0;
+    const bool mixed = o.prec == FR_MIXED;
     if (o.initial_guess) {
       if (!chi_dev)
         SCK(cudaMemcpyAsync(chi, chi_inout, nc * sizeof(double), cudaMemcpyHostToDevice, st));
-    } else {
-      // the homogeneous solution on the positive branch (1 before symmetry
-      // breaking, from where the field relaxes to its symmetric value 0)
-      const double chib = s < 1.0 ? std::sqrt(1.0 - s) : 1.0;
+    } else if (!mixed) {
       k_sy_fill<<<(unsigned)nblk(nc), kNT, 0, st>>>(chi, chib, nc);
       SLAUNCH(ctx);
     }
+    // the density's check; the mixed solve's pairs and FP32 copy come with it
+    float2 *rho2 = nullptr;
+    float *rho32 = nullptr;
     {
       int *bad = A.get<int>(1);
       SCK(cudaMemsetAsync(bad, 0, sizeof(int), st));
-      k_sy_check_rho<<<(unsigned)nblk(nc), kNT, 0, st>>>(rho, nc, bad);
+      if (mixed) {
+        rho2 = A.get<float2>(nc);
+        rho32 = A.get<float>(nc);
+        k_sy_rho<<<(unsigned)nblk(nc), kNT, 0, st>>>(rho, rho2, rho32, nc, bad);
+      } else {
+        k_sy_check_rho<<<(unsigned)nblk(nc), kNT, 0, st>>>(rho, nc, bad);
+      }
       SLAUNCH(ctx);
       int hb = 0;
       SCK(cudaMemcpyAsync(&hb, bad, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -923,8 +967,8 @@ extern "C" int fr_symmetron_solve(frmg_ctx *ctx, const double *density, const in
         L.uR = A.get<double>(L.nc);
         L.f = A.get<double>(L.nc);
         double *r = A.get<double>(L.nc);
-        k_sy_restrict<double, double><<<(unsigned)nblk(L.nc), kNT, 0, st>>>(
-            H.lev[l - 1].rho, r, L.n0, L.n1, L.n2);
+        k_sy_restrict<<<(unsigned)nblk(L.nc), kNT, 0, st>>>(H.lev[l - 1].rho, r, L.n0, L.n1,
+                                                            L.n2, L.fd0, L.fd1);
         SLAUNCH(ctx);
         L.rho = r;
         H.lev.push_back(L);
@@ -993,15 +1037,14 @@ extern "C" int fr_symmetron_solve(frmg_ctx *ctx, const double *density, const in
             L.u2 = A.get<float>(L.nc);
           }
         }
-        float *r = A.get<float>(L.nc);
-        if (l == 0) {
-          k_sy_convert<double, float><<<(unsigned)nblk(L.nc), kNT, 0, st>>>(rho, r, L.nc);
-        } else {
-          k_sy_restrict<float, float><<<(unsigned)nblk(L.nc), kNT, 0, st>>>(
-              H.lev[l - 1].rho, r, L.n0, L.n1, L.n2);
+        L.rho = rho32;
+        if (l > 0) {
+          float *r = A.get<float>(L.nc);
+          k_sy_restrict<<<(unsigned)nblk(L.nc), kNT, 0, st>>>(H.lev[l - 1].rho, r, L.n0, L.n1,
+                                                              L.n2, L.fd0, L.fd1);
+          SLAUNCH(ctx);
+          L.rho = r;
         }
-        SLAUNCH(ctx);
-        L.rho = r;
         gl[l] = A.get<float>(L.nc);
         L.g = gl[l];
         H.lev.push_back(L);
@@ -1010,10 +1053,13 @@ extern "C" int fr_symmetron_solve(frmg_ctx *ctx, const double *density, const in
       double *part_in = nl > 1 ? A.get<double>(2 * nb1) : nullptr;
       H.part0 = part_in;
       // chi and rho as double-float pairs for the outer loop
-      float2 *chi2 = A.get<float2>(nc), *rho2 = A.get<float2>(nc);
-      k_sy_split<<<(unsigned)nblk(nc), kNT, 0, st>>>(chi, chi2, nc);
-      SLAUNCH(ctx);
-      k_sy_split<<<(unsigned)nblk(nc), kNT, 0, st>>>(rho, rho2, nc);
+      float2 *chi2 = A.get<float2>(nc);
+      if (o.initial_guess) {
+        k_sy_split<<<(unsigned)nblk(nc), kNT, 0, st>>>(chi, chi2, nc);
+      } else {
+        const float ch = (float)chib;
+        k_sy_fill2<<<(unsigned)nblk(nc), kNT, 0, st>>>(chi2, ch, (float)(chib - (double)ch), nc);
+      }
       SLAUNCH(ctx);
       const float Ah = (float)Al[0], Alo = (float)(Al[0] - (double)Ah);
       const float sh = (float)s, slo = (float)(s - (double)sh);
@@ -1040,8 +1086,8 @@ extern "C" int fr_symmetron_solve(frmg_ctx *ctx, const double *density, const in
         // correction problem of this outer step: N(delta) = -d on g = fp32(chi)
         // (fine level set up by the defect pass)
         for (int l = 1; l < nl; l++) {
-          k_sy_restrict<float, float><<<(unsigned)nblk(ncell(l)), kNT, 0, st>>>(
-              gl[l - 1], gl[l], ns[l][0], ns[l][1], ns[l][2]);
+          k_sy_restrict<<<(unsigned)nblk(ncell(l)), kNT, 0, st>>>(
+              gl[l - 1], gl[l], ns[l][0], ns[l][1], ns[l][2], H.lev[l].fd0, H.lev[l].fd1);
           SLAUNCH(ctx);
         }
         // inner V-cycles until the fine correction residual (after
