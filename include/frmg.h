@@ -478,9 +478,8 @@ int fr_solve_masked(frmg_ctx *ctx, const double *density, const double *mask, co
  * solution sqrt(1 - s), or 1 before symmetry breaking), solution out.  Host
  * or device pointers.  opts: pre, post, newton_step_cap, relax, max_vcycles,
  * max_outer, initial_guess, tiling (FR_MIXED: the FP32 sweeps of a level run
- * as one register-column kernel per sweep on 64 x 8 tiles where the level
- * fills the GPU with tiles (0), wherever it is at least 16 cells a side (1),
- * or never (-1: one launch per colour)), prec: FR_FP64 = every step in FP64; FR_MIXED =
+ * as one register-column kernel per sweep on 64 x 16 tiles wherever it is at
+ * least 16 cells a side (0, 1), or never (-1: one launch per colour)), prec: FR_FP64 = every step in FP64; FR_MIXED =
  * the residual, the update of chi and the convergence test in double-float
  * (chi and rho as pairs of FP32 values, ~48-bit significands, on the FP32
  * pipes) around FP32 FAS V-cycles of

@@ -369,7 +369,7 @@ __device__ __forceinline__ int wrapmod_sy(int v, int n) {
 
 // One red-black sweep of the FP32 correction form with register-resident
 // z-columns (periodic grids of at least 16 cells a side): the layout and
-// march of the f(R) solver's register-column smoother on 64 x 8 tiles with a
+// march of the f(R) solver's register-column smoother on 64 x 16 tiles with a
 // halo of two cells.  Every x-pair of the tile plus halo has one owner
 // thread that keeps, for the last four planes, the pair's red and black cell
 // (delta and the cell's coefficients c1 = s rho - 1 + 3 g^2, c2 = 3 g and
@@ -382,14 +382,19 @@ __device__ __forceinline__ int wrapmod_sy(int v, int n) {
 // coefficients are recomputed from rho and g at every load).  Reads buffer
 // uin, writes uout (halos come from the unmodified input), so the sweep is
 // the same as two launches of k_sy_smooth up to FP32 rounding order.
-constexpr int kSyTX = 64, kSyTY = 8, kSyPX = kSyTX / 2 + 2, kSyLY = kSyTY + 4;
-constexpr int kSyPP = kSyPX * kSyLY, kSyNHR = 4 * (kSyTX / 2), kSyNHALO = kSyNHR + 2 * kSyLY;
-static_assert(kSyNHALO <= kNT, "halo pairs per thread");
+// Bound: instruction issue.  64 x 16 tiles (two interior pairs per thread, 128
+// registers, 2 blocks per SM) update and load 1.33 times the tile's cells with
+// its halo, 64 x 8 tiles (80 registers, 3 blocks) 1.59 times: a 512^3 solve takes
+// 39.7 and 45.0 ms with them.
+constexpr int kSyTX = 64, kSyTY = 16, kSyPX = kSyTX / 2 + 2;
 
-__global__ void __launch_bounds__(kNT, 3)
+__global__ void __launch_bounds__(kNT, 2)
     k_sy_smooth_rc(SLevel<float> L, const float *__restrict__ uin, float *__restrict__ uout,
                    int zc) {
-  constexpr int NSL = 2;  // one interior pair, one halo pair
+  constexpr int kSyLY = kSyTY + 4, kSyPP = kSyPX * kSyLY;
+  constexpr int kSyNHR = 4 * (kSyTX / 2), kSyNHALO = kSyNHR + 2 * kSyLY;
+  static_assert(kSyNHALO <= kNT, "halo pairs per thread");
+  constexpr int NIN = kSyTY / 8, NSL = NIN + 1;  // interior pairs and one halo pair per thread
   __shared__ float sbk[2][kSyPP], srd[2][kSyPP];
   const int n0 = L.n0, n1 = L.n1, n2 = L.n2;
   const int ntx = (n0 + kSyTX - 1) / kSyTX, nty = (n1 + kSyTY - 1) / kSyTY;
@@ -412,10 +417,10 @@ __global__ void __launch_bounds__(kNT, 3)
 #pragma unroll
   for (int sl = 0; sl < NSL; sl++) {
     int px = -1, ly = -1;
-    const bool interior = sl == 0;
+    const bool interior = sl < NIN;
     if (interior) {
       px = 1 + lane;
-      ly = 2 + w;
+      ly = 2 + w + 8 * sl;
     } else if ((int)threadIdx.x < kSyNHALO) {
       const int t = threadIdx.x;
       if (t < kSyNHR) {
@@ -503,7 +508,7 @@ __global__ void __launch_bounds__(kNT, 3)
 #pragma unroll
         for (int sl = 0; sl < NSL; sl++) {
           const bool odd = (ro[sl] ^ PK1) != 0;
-          if (!((sl == 0) || (fl[sl] & (odd ? 8u : 4u)))) continue;
+          if (!((sl < NIN) || (fl[sl] & (odd ? 8u : 4u)))) continue;
           const float *bk = &sbk[PK1][q[sl]];
           const float nx = bk[odd ? 1 : -1];
           const float in = B[sl][K1].x;
@@ -517,16 +522,20 @@ __global__ void __launch_bounds__(kNT, 3)
     {
       const int m = p - 2;
       if (m >= Z0 && m < Z1) {
-        const bool odd = (ro[0] ^ PK2) == 0;  // black cell is the odd one
-        const float *rd = &srd[PK2][q[0]];
-        const float nx = rd[odd ? 1 : -1];
-        const float in = R[0][K2].x;
-        const float dn = newton(B[0][K2], odd ? in : nx, odd ? nx : in, rd[-kSyPX], rd[kSyPX],
-                                R[0][K3].x, R[0][K1].x);
-        B[0][K2].x = dn;
-        if (fl[0] & 2u) {
-          const float de = odd ? R[0][K2].x : dn, dd = odd ? dn : R[0][K2].x;
-          *reinterpret_cast<float2 *>(uout + (long long)m * plane + roff[0]) = make_float2(de, dd);
+#pragma unroll
+        for (int sl = 0; sl < NIN; sl++) {
+          const bool odd = (ro[sl] ^ PK2) == 0;  // black cell is the odd one
+          const float *rd = &srd[PK2][q[sl]];
+          const float nx = rd[odd ? 1 : -1];
+          const float in = R[sl][K2].x;
+          const float dn = newton(B[sl][K2], odd ? in : nx, odd ? nx : in, rd[-kSyPX], rd[kSyPX],
+                                  R[sl][K3].x, R[sl][K1].x);
+          B[sl][K2].x = dn;
+          if (fl[sl] & 2u) {
+            const float de = odd ? R[sl][K2].x : dn, dd = odd ? dn : R[sl][K2].x;
+            *reinterpret_cast<float2 *>(uout + (long long)m * plane + roff[sl]) =
+                make_float2(de, dd);
+          }
         }
       }
     }
@@ -1017,25 +1026,24 @@ extern "C" int fr_symmetron_solve(frmg_ctx *ctx, const double *density, const in
         L.u = A.get<float>(L.nc);
         L.f = A.get<float>(L.nc);
         if (l > 0) L.uR = A.get<float>(L.nc);
-        // the register-column smoother on levels of at least 16 cells a side
-        // with enough tiles to fill the GPU (else one colour per launch)
+        // the register-column smoother on every level of at least 16 cells a
+        // side (whole solves, one colour per launch against it: 32^3 1.11 and
+        // 1.01 ms, 64^3 1.44 and 1.35, 128^3 2.15 and 1.93, 256^3 7.26 and 6.37)
         if (o.tiling >= 0 && L.n0 >= 16 && L.n1 >= 16 && L.n2 >= 16) {
           const long long tiles = (long long)((L.n0 + kSyTX - 1) / kSyTX) *
                                   ((L.n1 + kSyTY - 1) / kSyTY);
-          const long long slots = 3ll * sm_count_sy();
-          if (o.tiling == 1 || tiles * ((L.n2 + 31) / 32) >= slots) {
-            double best = 1e300;
-            for (int c = 1; c <= L.n2; c++) {
-              const int z = (L.n2 + c - 1) / c;
-              const long long nbk = tiles * ((L.n2 + z - 1) / z);
-              const double cost = std::ceil((double)nbk / slots) * (z + 4);
-              if (cost < best - 1e-9) {
-                best = cost;
-                L.zc = z;
-              }
+          const long long slots = 2ll * sm_count_sy();
+          double best = 1e300;
+          for (int c = 1; c <= L.n2; c++) {
+            const int z = (L.n2 + c - 1) / c;
+            const long long nbk = tiles * ((L.n2 + z - 1) / z);
+            const double cost = std::ceil((double)nbk / slots) * (z + 4);
+            if (cost < best - 1e-9) {
+              best = cost;
+              L.zc = z;
             }
-            L.u2 = A.get<float>(L.nc);
           }
+          L.u2 = A.get<float>(L.nc);
         }
         L.rho = rho32;
         if (l > 0) {
