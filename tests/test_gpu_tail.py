@@ -171,3 +171,19 @@ def test_poisson_tail_matches_fft(C, shape, pre, post, relax):
     ref, _ = PO.solve_periodic(PO.source(u, rho, **P), 1.0 / shape[2])
     assert st == 0 and s.res_rms <= 1e-10
     assert np.abs(host(phi) - ref).max() < 1e-9
+
+
+@pytest.mark.parametrize("shape", [(24, 40, 72), (2, 18, 66), (24, 512, 1280)])
+def test_symmetron_prolongation_tiles(C, shape):
+    """One FP64 V-cycle on grids whose coarse level ends inside a prolongation
+    tile, has one plane, and has a short last chunk of planes: the oracle's
+    iterate up to rounding.  (Coarsest grids of even sides: on odd ones cells of
+    one colour are neighbours across the boundary.)"""
+    from oracle import symmetron as SY
+    P = dict(a=1.0, a_ssb=0.5, lambda0=1.0)
+    rho = synth.lognormal_density(shape, 77, sigma=1.0)
+    ref = SY.solve(rho, box=0.5 * shape[2], tol=1e-30, max_cycles=1, **P)
+    chi = torch.empty(shape, dtype=torch.float64, device="cuda")
+    C.symmetron(dev(rho), chi, box=0.5 * shape[2], tol=1e-30, prec="fp64", initial_guess=0,
+                max_vcycles=1, **P)
+    assert np.abs(host(chi) - ref.chi).max() < 1e-10
