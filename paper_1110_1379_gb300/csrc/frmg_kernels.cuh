@@ -2411,6 +2411,14 @@ __device__ __forceinline__ void cp_async8(void *smem, const void *gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sa), "l"(gmem) : "memory");
 }
+__device__ __forceinline__ void cp_async4(void *smem, const void *gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sa), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() {
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
@@ -2420,53 +2428,51 @@ __device__ __forceinline__ void cp_async_wait() {
 }
 
 // Tiled FP32 residual + restriction (same result as k_resid_restrict).
-// A block owns a TX x TY fine tile and an even chunk of zc fine planes, marches
-// along z with a ring of 4 planes (tile plus a halo of 2 cells in x, so that
-// 8-byte x-pairs stay aligned, and 1 in y) in shared memory, and each thread
-// owns one coarse column of the tile: per fine plane it evaluates the residual
-// of its 2x2 fine cells from shared memory, and after every second plane it
-// writes its coarse cell (u^H = uR = mean u^h, x^H = expm1(u^H),
-// f^H <- mean d^h) and accumulates the fine residual norm.  Plane m+2 is
-// fetched into registers while plane m is evaluated.
-template <int TX, int TY>
+// A block owns a 64 x 16 fine tile and an even chunk of zc fine planes and
+// marches along z; a thread owns the 2 x 2 fine cells of one coarse column.
+// The planes arrive by asynchronous copies in a ring of four in shared memory,
+// two ahead of the one in use; each thread copies its own cells and the cells
+// beyond the tile that only it needs, and keeps its cells of planes m - 1, m,
+// m + 1 in registers, so that shared memory is read for the arriving plane and
+// the rows above and below only (x neighbours come by shuffles) and one barrier
+// per plane suffices.  Without a patch's ghost faces the two cells of an x-pair
+// are evaluated as one packed pair.  After every second plane a thread writes
+// its coarse cell (u^H = uR = mean u^h, x^H = expm1(u^H), f^H <- mean d^h); the
+// fine residual norm is accumulated on the way.
+//
+// 512^3: 0.379 ms plain, 0.715 ms in the correction form (3 and 5 arrays read,
+// 0.28 and 0.44 ms of memory time); with every neighbour of a cell read from
+// shared memory, which left one or two blocks per SM, 0.477 and 0.824 ms.
+// Bound by instruction issue (packed FP32, shuffles) at 16 and 24 warps per SM.
+template <bool BG>
 struct RRCfg {
-  // planes in flight beyond the three being read; ring of A + 4 slots (the
-  // slot being refilled was last read two iterations earlier)
-#ifndef FR_RR_AHEAD
-#define FR_RR_AHEAD 2
-#endif
-  static constexpr int A = FR_RR_AHEAD;
-  static constexpr int LX = TX + 4, LY = TY + 2, PL = LX * LY, NS = 4 + A;
-  static constexpr int PXR = LX / 2, NPAIR = PXR * LY;
-  static constexpr int CX = TX / 2, NT = (TX / 2) * (TY / 2);
-  static constexpr int K = (NPAIR + NT - 1) / NT;
-  static constexpr size_t smem(bool bg) { return (size_t)NS * PL * sizeof(float) * (bg ? 5 : 3); }
+  static constexpr int TX = 64, TY = 16, NT = 256, NW = NT / 32;
+  static_assert(TY == 2 * NW && TX == 64, "two rows per warp, one pair per lane");
+  static constexpr int NA = BG ? 4 : 2;  // arrays: u, x [, ub, E]
+  static constexpr int NS = 4;           // planes in the ring: m, m + 1 and two on their way
+  // rows -1 .. 16 of an array, then the columns left and right of the tile; f
+  // without either
+  static constexpr int EC = (TY + 2) * TX, AN = EC + 2 * TY, PL = NA * AN + TY * TX;
+  static constexpr int MINB = BG ? 2 : 3;
+  static constexpr size_t smem = (size_t)NS * PL * sizeof(float);
 };
 
-template <bool BG, bool DIR, int TX, int TY>
-__global__ void __launch_bounds__(RRCfg<TX, TY>::NT)
+template <bool BG, bool DIR>
+__global__ void __launch_bounds__(RRCfg<BG>::NT, RRCfg<BG>::MINB)
     k_resid_restrict_tiled(const Grid<float> *fine, const Grid<float> *coarse, const int *off,
                            int ngrid, int zc, const int *active, int fpar, int cpar,
                            double *partial) {
-  using C = RRCfg<TX, TY>;
-  constexpr int LX = C::LX, PL = C::PL, NS = C::NS, NT = C::NT, CX = C::CX;
-  constexpr int PXR = C::PXR, NPAIR = C::NPAIR, K = C::K;
+  using C = RRCfg<BG>;
+  constexpr int TX = C::TX, TY = C::TY, NT = C::NT, NA = C::NA;
+  constexpr bool CV = BG && !DIR;  // (x, E) are published and kept as (P, B)
   extern __shared__ float smem[];
-  float *sd = smem;
-  float *sx = smem + NS * PL;
-  float *sf = smem + 2 * NS * PL;
-  float *sub = smem + 3 * NS * PL;
-  float *sE = smem + 4 * NS * PL;
   const int g = find_grid(off, ngrid, blockIdx.x);
   const Grid<float> &Fg = fine[g];
   const Grid<float> &Cg = coarse[g];
   float ss = 0.0f, mx = 0.0f;
   if (grid_active(active, Fg.field)) {
-    const float *__restrict__ uin = fpar ? Fg.u2 : Fg.u;
-    const float *__restrict__ xin = fpar ? Fg.x2 : Fg.x;
+    const float *__restrict__ in[4] = {fpar ? Fg.u2 : Fg.u, fpar ? Fg.x2 : Fg.x, Fg.ubg, Fg.Ebg};
     const float *__restrict__ fin = Fg.f;
-    const float *__restrict__ ubin = Fg.ubg;
-    const float *__restrict__ Ein = Fg.Ebg;
     const float ah = Fg.ah, beta = Fg.beta;
     const int n0 = Fg.n0, n1 = Fg.n1, n2 = Fg.n2;
     const int c0 = Cg.n0, c1 = Cg.n1;
@@ -2482,168 +2488,265 @@ __global__ void __launch_bounds__(RRCfg<TX, TY>::NT)
     b /= nty;
     const int Z0 = b * zc;
     const int Z1 = min(Z0 + zc, n2);
-    // the pairs this thread loads: global pair start (wrapped) per slot, -1 if none
-    long long pg[K];
-    int po[K];
-#pragma unroll
-    for (int k = 0; k < K; k++) {
-      const int c = threadIdx.x + k * NT;
-      pg[k] = -1;
-      po[k] = 0;
-      if (c < NPAIR) {
-        const int yy = c / PXR, px = c - yy * PXR;
-        int gxx = X0 - 2 + 2 * px, gyy = Y0 - 1 + yy;
-        po[k] = yy * LX + 2 * px;
-        bool in = true;
-        if (DIR) {
-          in = gxx >= 0 && gxx < n0 && gyy >= 0 && gyy < n1;
-        } else {
-          // the tile (TX + 4 wide) may span more than two periods of a small grid
-          gxx = wrapmod(gxx, n0);
-          gyy = wrapmod(gyy, n1);
-        }
-        if (in) pg[k] = (long long)gyy * n0 + gxx;
-      }
-    }
-    // copies of plane p into ring slot (p - (Z0 - 1)) mod NS: one commit
-    // group per call (empty when the plane is outside a patch)
-    const bool hasf = fin != nullptr;
-    int pwz = DIR ? Z0 - 1 : wrapmod(Z0 - 1, n2);  // wrapped index of the next plane
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int gx = X0 + 2 * lane, gy = Y0 + 2 * w;
+    const bool valid = gx < n0 && gy < n1;
     const long long fplane = (long long)n0 * n1;
-    auto issue = [&](int p, int slot) {
-      if (!DIR || (p >= 0 && p < n2)) {
-        const long long zo = (long long)pwz * fplane;
-        const int base = slot * PL;
+    // What a lane copies of a plane (offsets, -1: none).  Rows of whole quads:
+    // 16 bytes of row 2 w (lanes 0 - 15) or 2 w + 1, and of the row beyond the
+    // tile (first and last warp); else pairs of both rows.  The first and last
+    // lane also copy the cells left and right of the tile.
+    auto at = [&](int x, int y) -> int {
+      if (DIR) return x >= 0 && x < n0 && y >= 0 && y < n1 ? y * n0 + x : -1;
+      return wrapmod(y, n1) * n0 + wrapmod(x, n0);
+    };
+    const bool quad = !(n0 & 3);
+    const int lx = quad ? 4 * (lane & 15) : 2 * lane, ly = quad ? lane >> 4 : 0;
+    const int o0 = at(X0 + lx, gy + ly);
+    const int oh = w == 0 && !(quad && ly) ? at(X0 + lx, gy - 1)
+                   : (w == C::NW - 1 && !(quad && ly) ? at(X0 + lx, gy + 2) : -1);
+    const int ex = lane == 0 ? X0 - 1 : X0 + TX;
+    const bool edge = lane == 0 || lane == 31;
+    const int oe = edge ? at(ex, gy) : -1;  // (and the row above: n1 is even)
+    // their places in an array's tile, and the own pair of row 2 w
+    const int qc = (2 * w + 1 + ly) * TX + lx;
+    const int qh = (w == 0 ? 0 : TY + 1) * TX + lx;
+    const int qe = C::EC + (lane == 0 ? 0 : TY) + 2 * w;
+    const int q0 = (2 * w + 1) * TX + 2 * lane;
+    auto inz = [&](int p) { return !DIR || (p >= 0 && p < n2); };
+    auto wrapz = [&](int p) { return DIR ? p : (p < 0 ? p + n2 : (p >= n2 ? p - n2 : p)); };
+
+    float2 r[4][NA][2];  // plane (m - 1, m, m + 1 live), array, row
 #pragma unroll
-        for (int k = 0; k < K; k++) {
-          if (pg[k] < 0) continue;
-          const long long gi = zo + pg[k];
-          const int o = base + po[k];
-          cp_async8(sd + o, uin + gi);
-          cp_async8(sx + o, xin + gi);
-          if (hasf) cp_async8(sf + o, fin + gi);
-          if (BG) {
-            cp_async8(sub + o, ubin + gi);
-            cp_async8(sE + o, Ein + gi);
+    for (int k = 0; k < 4; k++)
+#pragma unroll
+      for (int a = 0; a < NA; a++)
+        r[k][a][0] = r[k][a][1] = make_float2(a == 3 ? 1.f : 0.f, a == 3 ? 1.f : 0.f);
+    auto ld2 = [](const float *p) { return *reinterpret_cast<const float2 *>(p); };
+    // copies of plane p into its slot, one commit group
+    auto fetch = [&](int p) {
+      if (p <= Z1 && inz(p)) {
+        const bool own = p >= Z0 && p < Z1;
+        const long long zo = (long long)wrapz(p) * fplane;
+        float *h = smem + ((p - Z0 + 1) & 3) * C::PL;
+#pragma unroll
+        for (int a = 0; a < NA; a++) {
+          const float *v = in[a] + zo;
+          float *ha = h + a * C::AN;
+          if (quad) {
+            if (o0 >= 0) cp_async16(ha + qc, v + o0);
+            if (own && oh >= 0) cp_async16(ha + qh, v + oh);
+          } else {
+            if (o0 >= 0) {
+              cp_async8(ha + qc, v + o0);
+              cp_async8(ha + qc + TX, v + o0 + n0);
+            }
+            if (own && oh >= 0) cp_async8(ha + qh, v + oh);
+          }
+          if (own && oe >= 0) {
+            cp_async4(ha + qe, v + oe);
+            cp_async4(ha + qe + 1, v + oe + n0);
+          }
+        }
+        if (fin && own && o0 >= 0) {
+          float *hf = h + NA * C::AN + qc - TX;
+          if (quad) {
+            cp_async16(hf, fin + zo + o0);
+          } else {
+            cp_async8(hf, fin + zo + o0);
+            cp_async8(hf + TX, fin + zo + o0 + n0);
           }
         }
       }
       cp_async_commit();
-      pwz = DIR ? pwz + 1 : (pwz + 1 == n2 ? 0 : pwz + 1);
     };
-    const int ci = threadIdx.x % CX, cj = threadIdx.x / CX;
-    const int lx = 2 + 2 * ci, ly = 1 + 2 * cj;
-    const int gx = X0 + 2 * ci, gy = Y0 + 2 * cj;
-    const bool valid = gx < n0 && gy < n1;
-    float su = 0.f, sdd = 0.f;
-    constexpr int A = C::A;
-    // prologue: planes Z0-1 .. Z0+A (slots 0 .. A+1)
+    // (x, E) -> (P, B), P = E x, B = E + P
+    auto conv = [](float2 &x, float2 &E) {
+      x = mul2(E, x);
+      E = add2(E, x);
+    };
+    float2 su = make_float2(0.f, 0.f), sd = su, s2 = su;
+
+    auto step = [&](auto Kc, int p) {
+      constexpr int K = decltype(Kc)::value;  // ring slot of plane p
+      constexpr int K1 = (K + 3) & 3, K2 = (K + 2) & 3;
+      // 1. plane p + 2 on its way (into the slot of plane p - 2, last read in
+      // the step before the last barrier), plane p from its slot
+      fetch(p + 2);
+      cp_async_wait<2>();
+      __syncwarp();  // a warp's rows are copied by all of its lanes
+      const float *sp = smem + K * C::PL;
 #pragma unroll
-    for (int d = 0; d < A + 2; d++) issue(Z0 - 1 + d, d);
-    int sl = 1;  // ring slot of plane m
-    for (int m = Z0; m < Z1; m++) {
-      // plane m+1+A into the slot of plane m-3 (last read by iteration m-2,
-      // before the barrier of iteration m-1); planes m-1, m, m+1 must have landed
-      {
-        const int pz = m + 1 + A;
-        if (pz <= Z1) issue(pz, (sl + A + 1) % NS);
-        else cp_async_commit();
+      for (int a = 0; a < NA; a++) {
+        r[K][a][0] = ld2(sp + a * C::AN + q0);
+        r[K][a][1] = ld2(sp + a * C::AN + q0 + TX);
       }
-      cp_async_wait<A>();
-      __syncthreads();
-      if (valid) {
-        const int slm = sl == 0 ? NS - 1 : sl - 1, slp = sl + 1 == NS ? 0 : sl + 1;
-        // the 2 x 2 cells of this thread (rows ly, ly + 1; columns lx, lx + 1)
-        // and their neighbours as aligned pairs: left, own and right pair of
-        // each row, the pairs of rows ly - 1 and ly + 2, and the own pairs of
-        // planes m - 1 and m + 1 (same values and face order as cell by cell)
-        const int r0 = sl * PL + ly * LX + lx, r1 = r0 + LX;
-        const int zm0 = slm * PL + ly * LX + lx, zp0 = slp * PL + ly * LX + lx;
-        auto pr = [&](const float *a, int o) { return *reinterpret_cast<const float2 *>(a + o); };
-        struct Nb {
-          float2 L[2], C[2], R[2], D, U, M[2], P[2];
-        };
-        auto gather = [&](const float *a) {
-          Nb n;
-          n.L[0] = pr(a, r0 - 2);
-          n.C[0] = pr(a, r0);
-          n.R[0] = pr(a, r0 + 2);
-          n.L[1] = pr(a, r1 - 2);
-          n.C[1] = pr(a, r1);
-          n.R[1] = pr(a, r1 + 2);
-          n.D = pr(a, r0 - LX);
-          n.U = pr(a, r1 + LX);
-          n.M[0] = pr(a, zm0);
-          n.M[1] = pr(a, zm0 + LX);
-          n.P[0] = pr(a, zp0);
-          n.P[1] = pr(a, zp0 + LX);
-          return n;
-        };
-        const Nb nu = gather(sd), nx = gather(sx);
-        Nb nb, ne;
-        if (BG) {
-          nb = gather(sub);
-          ne = gather(sE);
-        }
-        const float2 f0 = hasf ? pr(sf, r0) : make_float2(0.f, 0.f);
-        const float2 f1 = hasf ? pr(sf, r1) : make_float2(0.f, 0.f);
-        auto lane = [](const float2 &v, int a) { return a ? v.y : v.x; };
+      // 2. residual of plane m = p - 1
+      const int m = p - 1;
+      if (m >= Z0) {
+        const float *sm = smem + K1 * C::PL;
+        float2 O[NA][2];
 #pragma unroll
-        for (int q = 0; q < 4; q++) {
-          const int ax = q & 1, ay = q >> 1;
-          const int gxq = gx + ax, gyq = gy + ay;
-          // value of array n at neighbour k of the cell: 0 -x, 1 +x, 2 -y, 3 +y, 4 -z, 5 +z
-          auto at = [&](const Nb &n, int k) -> float {
-            switch (k) {
-              case 0: return ax ? n.C[ay].x : n.L[ay].y;
-              case 1: return ax ? n.R[ay].x : n.C[ay].y;
-              case 2: return ay ? lane(n.C[0], ax) : lane(n.D, ax);
-              case 3: return ay ? lane(n.U, ax) : lane(n.C[1], ax);
-              case 4: return lane(n.M[ay], ax);
-              default: return lane(n.P[ay], ax);
-            }
-          };
-          const float di = lane(nu.C[ay], ax), xi = lane(nx.C[ay], ax);
-          const float Ei = BG ? lane(ne.C[ay], ax) : 1.0f;
-          const float ubi = BG ? lane(nb.C[ay], ax) : 0.0f;
-          const float Bi = BG ? Ei + Ei * xi : 1.0f + xi;
-          OpAcc<float, BG> A(di, Ei, xi, Bi, ubi);
-#define FR_NB(K) A.reg(at(nu, K), at(nx, K), BG ? at(nb, K) : 0.0f, BG ? at(ne, K) : 1.0f)
-          if (DIR && gxq == 0) A.ghost(face_value(Fg, 0, gxq, gyq, m));
-          else FR_NB(0);
-          if (DIR && gxq == n0 - 1) A.ghost(face_value(Fg, 1, gxq, gyq, m));
-          else FR_NB(1);
-          if (DIR && gyq == 0) A.ghost(face_value(Fg, 2, gxq, gyq, m));
-          else FR_NB(2);
-          if (DIR && gyq == n1 - 1) A.ghost(face_value(Fg, 3, gxq, gyq, m));
-          else FR_NB(3);
-          if (DIR && m == 0) A.ghost(face_value(Fg, 4, gxq, gyq, m));
-          else FR_NB(4);
-          if (DIR && m == n2 - 1) A.ghost(face_value(Fg, 5, gxq, gyq, m));
-          else FR_NB(5);
-#undef FR_NB
-          float acc, dacc, N, dN;
-          A.done(acc, dacc);
-          finish_op(xi, Ei, acc, dacc, ah, beta, BG, N, dN);
-          const float d = N - lane(ay ? f1 : f0, ax);  // FP32 grids: fs (f - fo) = f
-          sdd += d;
-          su += di;
-          ss = fmaf(d, d, ss);
-          mx = fmaxf(mx, fabsf(d));
+        for (int a = 0; a < NA; a++) {
+          O[a][0] = r[K1][a][0];
+          O[a][1] = r[K1][a][1];
         }
-        if ((m - Z0) & 1) {
+        if (CV) {
+          conv(O[1][0], O[NA - 1][0]);
+          conv(O[1][1], O[NA - 1][1]);
+        }
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+          // left and right neighbours of the pair, and the row below (k = 0)
+          // or above (k = 1) the own two
+          float2 L[NA], R[NA], V[NA];
+          float lo[NA], hi[NA];
+#pragma unroll
+          for (int a = 0; a < NA; a++) {
+            lo[a] = __shfl_up_sync(0xffffffffu, O[a][k].y, 1);
+            hi[a] = __shfl_down_sync(0xffffffffu, O[a][k].x, 1);
+          }
+          if (edge) {
+            float e[NA];
+#pragma unroll
+            for (int a = 0; a < NA; a++) e[a] = sm[a * C::AN + qe + k];
+            if (CV) {
+              e[1] = __fmul_rn(e[NA - 1], e[1]);
+              e[NA - 1] = __fadd_rn(e[NA - 1], e[1]);
+            }
+#pragma unroll
+            for (int a = 0; a < NA; a++) (lane == 0 ? lo[a] : hi[a]) = e[a];
+          }
+#pragma unroll
+          for (int a = 0; a < NA; a++) {
+            L[a] = make_float2(lo[a], O[a][k].x);
+            R[a] = make_float2(O[a][k].y, hi[a]);
+            V[a] = ld2(sm + a * C::AN + q0 + (k ? 2 * TX : -TX));
+          }
+          if (CV) conv(V[1], V[NA - 1]);
+          const float2 di = r[K1][0][k], xi = r[K1][1][k];
+          const float2 f =
+              fin ? ld2(sm + NA * C::AN + q0 + (k - 1) * TX) : make_float2(0.f, 0.f);
+          float2 d;
+          if constexpr (!DIR) {
+            float2 Zm[NA], Zp[NA];
+#pragma unroll
+            for (int a = 0; a < NA; a++) {
+              Zm[a] = r[K2][a][k];
+              Zp[a] = r[K][a][k];
+            }
+            if (CV) conv(Zp[1], Zp[NA - 1]);
+            float2 S1, S2;
+            [[maybe_unused]] float2 G1, G2;  // of the correction form
+            auto face = [&](const float2 (&v)[NA], bool first) {
+              const float2 dd = sub2(v[0], di);
+              S1 = first ? dd : add2(S1, dd);
+              S2 = first ? mul2(v[NA - 1], dd) : fma2(v[NA - 1], dd, S2);
+              if constexpr (BG) {
+                const float2 gg = sub2(v[2], r[K1][NA - 2][k]);
+                G1 = first ? gg : add2(G1, gg);
+                G2 = first ? mul2(v[1], gg) : fma2(v[1], gg, G2);
+              }
+            };
+            auto other = [&]() {
+              float2 t[NA];
+#pragma unroll
+              for (int a = 0; a < NA; a++) t[a] = O[a][1 - k];
+              face(t, false);
+            };
+            face(L, true);
+            face(R, false);
+            if (k == 0) face(V, false);
+            other();
+            if (k == 1) face(V, false);
+            face(Zm, false);
+            face(Zp, false);
+            float2 acc;
+            if constexpr (BG) {
+              const float2 Ei = r[K1][NA - 1][k];
+              acc = add2(fma2(O[1][k], G1, G2), fma2(fma2(Ei, xi, Ei), S1, S2));
+            } else {
+              acc = fma2(add2(add2(splat2(1.0f), xi), splat2(1.0f)), S1, S2);
+            }
+            // N of finish_op, in pairs
+            const float2 B1 = add2(splat2(1.0f), xi);
+            const float2 rs = make_float2(sfu_rsqrt(B1.x), sfu_rsqrt(B1.y));
+            const float2 den = add2(B1, mul2(B1, rs));
+            const float2 y = mul2(neg2(xi), make_float2(sfu_rcp(den.x), sfu_rcp(den.y)));
+            float2 bF = splat2(beta);
+            if constexpr (BG) {
+              const float2 Ei = r[K1][NA - 1][k];
+              bF = mul2(bF, make_float2(sfu_rsqrt(Ei.x), sfu_rsqrt(Ei.y)));
+            }
+            d = sub2(fma2(splat2(ah), acc, mul2(bF, y)), f);
+          } else {
+            // cell by cell, with the ghost faces of a patch
+#pragma unroll
+            for (int ax = 0; ax < 2; ax++) {
+              auto lane_of = [&](const float2 &v) { return ax ? v.y : v.x; };
+              const int gxq = gx + ax, gyq = gy + k;
+              const float dc = lane_of(di), xc = lane_of(xi);
+              const float Ei = BG ? lane_of(r[K1][NA - 1][k]) : 1.0f;
+              const float ubi = BG ? lane_of(r[K1][NA - 2][k]) : 0.0f;
+              const float Bi = BG ? Ei + Ei * xc : 1.0f + xc;
+              OpAcc<float, BG> A(dc, Ei, xc, Bi, ubi);
+              auto nb = [&](auto get) {
+                A.reg(lane_of(get(0)), lane_of(get(1)), BG ? lane_of(get(NA - 2)) : 0.0f,
+                      BG ? lane_of(get(NA - 1)) : 1.0f);
+              };
+              if (gxq == 0) A.ghost(face_value(Fg, 0, gxq, gyq, m));
+              else nb([&](int a) { return L[a]; });
+              if (gxq == n0 - 1) A.ghost(face_value(Fg, 1, gxq, gyq, m));
+              else nb([&](int a) { return R[a]; });
+              if (gyq == 0) A.ghost(face_value(Fg, 2, gxq, gyq, m));
+              else nb([&](int a) { return k ? O[a][0] : V[a]; });
+              if (gyq == n1 - 1) A.ghost(face_value(Fg, 3, gxq, gyq, m));
+              else nb([&](int a) { return k ? V[a] : O[a][1]; });
+              if (m == 0) A.ghost(face_value(Fg, 4, gxq, gyq, m));
+              else nb([&](int a) { return r[K2][a][k]; });
+              if (m == n2 - 1) A.ghost(face_value(Fg, 5, gxq, gyq, m));
+              else nb([&](int a) { return r[K][a][k]; });
+              float acc, dacc, N, dN;
+              A.done(acc, dacc);
+              finish_op(xc, Ei, acc, dacc, ah, beta, BG, N, dN);
+              (ax ? d.y : d.x) = N - lane_of(f);
+            }
+          }
+          if (valid) {
+            sd = add2(sd, d);
+            su = add2(su, di);
+            s2 = fma2(d, d, s2);
+            mx = fmaxf(mx, fmaxf(fabsf(d.x), fabsf(d.y)));
+          }
+        }
+        if (((m - Z0) & 1) && valid) {
           const long long cidx = ((long long)(m >> 1) * c1 + (gy >> 1)) * c0 + (gx >> 1);
-          const float uh = su * 0.125f;
+          const float uh = (su.x + su.y) * 0.125f;
           cR[cidx] = uh;
           cu[cidx] = uh;
           cx[cidx] = m_expm1(uh);
-          cf[cidx] = sdd * 0.125f;
-          su = 0.f;
-          sdd = 0.f;
+          cf[cidx] = (sd.x + sd.y) * 0.125f;
+          su = sd = make_float2(0.f, 0.f);
         }
       }
-      sl = sl + 1 == NS ? 0 : sl + 1;
+      if (CV) {  // plane p - 1 becomes the plane below
+        conv(r[K1][1][0], r[K1][NA - 1][0]);
+        conv(r[K1][1][1], r[K1][NA - 1][1]);
+      }
+      __syncthreads();
+    };
+    // planes Z0 - 1 .. Z1; the number of planes is even (zc and n2 are)
+    fetch(Z0 - 1);
+    fetch(Z0);
+    for (int p = Z0 - 1; p <= Z1; p += 4) {
+      step(std::integral_constant<int, 0>{}, p);
+      step(std::integral_constant<int, 1>{}, p + 1);
+      if (p + 2 <= Z1) {
+        step(std::integral_constant<int, 2>{}, p + 2);
+        step(std::integral_constant<int, 3>{}, p + 3);
+      }
     }
+    ss = s2.x + s2.y;
     cp_async_wait<0>();
   }
   if (partial) block_reduce2f<NT>(ss, mx, &partial[2 * blockIdx.x], &partial[2 * blockIdx.x + 1]);

@@ -1097,15 +1097,16 @@ static void launch_tiled_k(frmg_ctx *ctx, LevelSet<float> &s, const int *active,
 template <bool BG, bool DIR>
 static void launch_rr_k(frmg_ctx *ctx, LevelSet<float> &F, LevelSet<float> &C, const int *active,
                         int fpar, int cpar, double *partial, cudaStream_t st) {
-  using RC = RRCfg<kTX, kTY>;
-  size_t sm = RC::smem(BG);
+  using RC = RRCfg<BG>;
+  static_assert(RC::TX == kTX && RC::TY == kTY, "tile");
+  const size_t sm = RC::smem;
   static bool attr_set = false;
   if (!attr_set) {
-    CK(cudaFuncSetAttribute(k_resid_restrict_tiled<BG, DIR, kTX, kTY>,
+    CK(cudaFuncSetAttribute(k_resid_restrict_tiled<BG, DIR>,
                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     attr_set = true;
   }
-  k_resid_restrict_tiled<BG, DIR, kTX, kTY><<<F.nblk_rr, RC::NT, sm, st>>>(
+  k_resid_restrict_tiled<BG, DIR><<<F.nblk_rr, RC::NT, sm, st>>>(
       F.d, C.d, F.d_off_rr, F.size(), F.zc_rr, active, fpar, cpar, partial);
 }
 
@@ -1236,9 +1237,9 @@ template <bool DIR>
 static long long rr_slots() {
   static long long slots = 0;
   if (!slots) {
-    using RC = RRCfg<kTX, kTY>;
+    using RC = RRCfg<false>;
     slots = (long long)sm_count() *
-            resident_blocks(k_resid_restrict_tiled<false, DIR, kTX, kTY>, RC::NT, RC::smem(false));
+            resident_blocks(k_resid_restrict_tiled<false, DIR>, RC::NT, RC::smem);
   }
   return slots;
 }

@@ -187,3 +187,43 @@ def test_symmetron_prolongation_tiles(C, shape):
     C.symmetron(dev(rho), chi, box=0.5 * shape[2], tol=1e-30, prec="fp64", initial_guess=0,
                 max_vcycles=1, **P)
     assert np.abs(host(chi) - ref.chi).max() < 1e-10
+
+
+@pytest.mark.parametrize("bg", [False, True])
+@pytest.mark.parametrize("shape", [(40, 34, 66), (40, 36, 132), (64, 52, 36), (34, 50, 70)])
+def test_tiled_residual_and_restriction(C, shape, bg):
+    """Tiles that end within the grid in x and y, rows of whole quads and not,
+    several chunks: two V-cycles (the second after an outer step in the
+    correction form) with the tiled kernels and with one thread per cell give
+    the same iterate up to FP32 rounding.  The sums of a residual's terms round
+    to 6 eps of |u| <= 20 each; a neighbour mixed up changes u by its
+    variation between cells, of order 1e-2 and more."""
+    rho, P = _case(shape, 8900)
+    out = []
+    for tiling in (-1, 1):
+        u = torch.zeros(shape, dtype=torch.float64, device="cuda")
+        C.solve(dev(rho), u, tol=1e-30, prec="mixed", tiling=tiling, fmg=0,
+                max_vcycles=12 if bg else 2, **P)
+        out.append(host(u))
+    assert np.abs(out[0]).max() > 0.1
+    assert np.abs(out[0] - out[1]).max() < 12 * 6e-8 * 20
+
+
+def test_tiled_patch_of_pairs(C):
+    """A patch whose rows are not whole quads and end within a tile."""
+    n = 48
+    rho, P = _case((n,) * 3, 8901)
+    prho = synth.lognormal_density((40, 36, 70), 8902, sigma=1.0)
+    org = (4, 4, 6)
+    dom, pres = O.solve_levels(rho, [dict(parent=-1, origin=org, rho=prho)], tol=1e-11, **P)
+    u0 = torch.zeros((n,) * 3, dtype=torch.float64, device="cuda")
+    vc = []
+    for tiling in (-1, 1):
+        u0.zero_()
+        g = dict(parent=-1, origin=org, density=dev(prho),
+                 u=torch.zeros(prho.shape, dtype=torch.float64, device="cuda"))
+        st, stats = C.solve_levels(dev(rho), u0, [g], tol=1e-11, prec="mixed", tiling=tiling, **P)
+        assert st == 0
+        assert np.abs(host(g["u"]) - pres[0].u).max() < 1e-8
+        vc.append(sum(s.vcycles for s in stats))
+    assert abs(vc[0] - vc[1]) <= 1
