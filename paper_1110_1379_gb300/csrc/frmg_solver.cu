@@ -1229,7 +1229,7 @@ static long long fr_slots() {
 template <bool DIR>
 static long long pl_slots() {
   static long long slots = 0;
-  if (!slots) slots = (long long)sm_count() * resident_blocks(k_prolong_tiled<DIR>, 256, 0);
+  if (!slots) slots = (long long)sm_count() * resident_blocks(k_prolong_tiled<DIR, false>, 256, 0);
   return slots;
 }
 
@@ -1324,7 +1324,7 @@ static void smooth_set(frmg_ctx *ctx, LevelSet<T> &s, int sweeps, const std::vec
 
 // u^h += P (u^H - R u^h) from depth l + 1 onto depth l (tiled where the
 // depth's sets have the tiled schedule).
-template <typename T>
+template <typename T, bool BG>
 static void prolong_level(frmg_ctx *ctx, Hier<T> &H, int l, const int *active, cudaStream_t st) {
   auto &F = H.cont[l];
   auto &C = H.next[l];
@@ -1333,11 +1333,11 @@ static void prolong_level(frmg_ctx *ctx, Hier<T> &H, int l, const int *active, c
   if constexpr (sizeof(T) == 4) {
     if (F.rr_tiled && F.nblk_pl > 0) {
       if (F.dirichlet)
-        k_prolong_tiled<true><<<F.nblk_pl, 256, 0, st>>>(F.d, C.d, F.d_off_pl, F.size(),
-                                                         F.kc_pl, active, H.par[l], H.par[l + 1]);
+        k_prolong_tiled<true, BG><<<F.nblk_pl, 256, 0, st>>>(
+            F.d, C.d, F.d_off_pl, F.size(), F.kc_pl, active, H.par[l], H.par[l + 1]);
       else
-        k_prolong_tiled<false><<<F.nblk_pl, 256, 0, st>>>(F.d, C.d, F.d_off_pl, F.size(),
-                                                          F.kc_pl, active, H.par[l], H.par[l + 1]);
+        k_prolong_tiled<false, BG><<<F.nblk_pl, 256, 0, st>>>(
+            F.d, C.d, F.d_off_pl, F.size(), F.kc_pl, active, H.par[l], H.par[l + 1]);
       done = true;
     }
   }
@@ -1490,7 +1490,7 @@ static void vcycle_launched(frmg_ctx *ctx, Hier<T> &H, int l, const CycleOpts &o
       return;
     }
   }
-  prolong_level<T>(ctx, H, l, active, st);
+  prolong_level<T, BG>(ctx, H, l, active, st);
   smooth_set<T, BG>(ctx, F, o.post, tiled_ok ? &plan_post : nullptr, active, H.par[l], st,
                     l == 0);
 }
@@ -1520,7 +1520,7 @@ static void fmg_start(frmg_ctx *ctx, Hier<float> &H, const CycleOpts &co, const 
     CK(cudaMemsetAsync(lev[l + 1].uR, 0, lev[l + 1].ncell * sizeof(float), st));
     CK(cudaMemsetAsync(H.cur_u(0, l), 0, lev[l].ncell * sizeof(float), st));
     CK(cudaMemsetAsync(H.cur_x(0, l), 0, lev[l].ncell * sizeof(float), st));
-    prolong_level<float>(ctx, H, l, active, st);
+    prolong_level<float, false>(ctx, H, l, active, st);
     vcycle<float, false>(ctx, H, l, co, active, st);
   }
 }

@@ -227,3 +227,20 @@ def test_tiled_patch_of_pairs(C):
         assert np.abs(host(g["u"]) - pres[0].u).max() < 1e-8
         vc.append(sum(s.vcycles for s in stats))
     assert abs(vc[0] - vc[1]) <= 1
+
+
+@pytest.mark.parametrize("tiled", [1, 8, 16])
+@pytest.mark.parametrize("c", [-6.0, -2.1, -0.7, -0.35, -0.05, 0.05, 0.36, 1.1])
+def test_sweeps_over_the_range_of_u(C, tiled, c):
+    """The sweeps' e^u - 1 on both sides of the ends of its reduction (u = +-ln2
+    / 2, multiples of ln2) and near zero: two FP32 sweeps against the FP64
+    oracle, to a few hundred FP32 roundings of u (at least 1)."""
+    shape = (24, 20, 36)
+    rng = np.random.default_rng(29)
+    P = dict(box=128.0, a=1.0, omega_m=0.24, fr0=1e-5, h=1.0 / 40)
+    f32 = lambda a: a.astype(np.float32).astype(np.float64)  # noqa: E731
+    u0, f = f32(c + 0.04 * rng.standard_normal(shape)), f32(rng.standard_normal(shape) * 0.05)
+    ref = O.smooth(u0, np.ones(shape), 2, f=f, **P)
+    u = torch.from_numpy(u0.astype(np.float32)).cuda()
+    C.smooth_f32(u, 2, f=torch.from_numpy(f.astype(np.float32)).cuda(), tiled=tiled, **P)
+    assert np.abs(host(u) - ref).max() < 2e-5 * max(1.0, abs(c))
