@@ -301,7 +301,10 @@ struct OpAcc<float, true> {
       : di(d), Ei(E), xi(x), Bi(B), ubi(ub) {}
   __device__ __forceinline__ void reg(float dj, float xj, float ubj, float Ej) {
     const float Pj = __fmul_rn(Ej, xj);
-    const float Bj = __fadd_rn(Ej, Pj);
+    reg_pb(dj, Pj, ubj, __fadd_rn(Ej, Pj));
+  }
+  // the neighbour's P = E x and B = E + P formed beforehand
+  __device__ __forceinline__ void reg_pb(float dj, float Pj, float ubj, float Bj) {
     const float dd = __fsub_rn(dj, di), g = __fsub_rn(ubj, ubi);
     G1 = __fadd_rn(G1, g);
     G2 = fmaf(Pj, g, G2);
@@ -415,8 +418,8 @@ __device__ __forceinline__ float2 m_expm1_2(float2 d) {
 // keep their relative accuracy.  n is clamped to [-127, 127]
 // (2^-127 counts as 0; r, and with it the result, grow beyond).  Relative error
 // <= 1.6e-7 for |d| < 4, m_expm1 9.2e-7 (expf(d) - 1 just above its threshold).
-// Sweep with prolongation at 512^3 0.896 -> 0.851 ms; on strongly clustered
-// batches of 256^3 0.337 -> 0.288, sweeps 0.215 -> 0.201.
+// Sweep with prolongation at 512^3 0.896 -> 0.851 ms; on a batch of 48 grids of
+// 32^3 to 128^3 0.337 -> 0.288, its plain sweeps 0.215 -> 0.201.
 __device__ __forceinline__ float2 m_expm1_full2(float2 d) {
   const float magic = 12582912.0f;  // 1.5 2^23: the sum's low bits are n
   float2 t = fma2(d, splat2(1.44269504f), splat2(magic));
@@ -1837,6 +1840,12 @@ __global__ void __launch_bounds__(RBCfg<TY>::NT, RBCfg<TY>::minb(BG))
 // compile-time indices; which cell of a pair is red is a per-slot bit flipped
 // every plane, applied with selects, so an update is straight-line code and
 // the updates of a thread's slots interleave.
+// In the correction form a cell is kept and published as its neighbours use it,
+// (u, P = E x, ub, B = E + P), and the x and E that only its own update needs
+// wait in the thread's own shared memory: bound by issue (60 % of slots), the
+// two operations per face saved are 3 % of a sweep (512^3 1.081 -> 1.054 ms).
+// 64 x 16 tiles of 512 threads (one block per SM, a sixth fewer halo updates)
+// took as long, and planes arriving by 8-byte asynchronous copies 1.67 ms.
 // Thread layout (256 threads, 8 warps): warp w owns the interior pairs
 // px = 1 + lane of rows 2 + w + 8 j (j < TY / 8), and thread t < NHALO also
 // one halo pair: the four halo rows for t < 128, the two halo columns above.
@@ -1859,9 +1868,11 @@ struct RCCfg {
   // coarse tile of the prolongation (fine tile plus halo, +-1 coarse cell)
   static constexpr int CXE = TX / 2 + 4, CYE = TY / 2 + 4, CE = CXE * CYE;
   static constexpr size_t smem(bool prl = false) {
-    return (size_t)4 * PP * sizeof(Cell) + (prl ? (size_t)2 * CE * sizeof(float) : 0);
+    return (size_t)4 * PP * sizeof(Cell) + (prl ? (size_t)2 * CE * sizeof(float) : 0) +
+           (BG ? NT * (4 * sizeof(float2) + 2 * sizeof(float)) : 0);
   }
   static_assert(TY % NW == 0 && NHALO <= NT, "tile height");
+  static_assert(!BG || NI == 1, "the correction form keeps the x of one pair per thread");
 };
 
 template <bool BG, bool DIR, int TY, bool PRL = false>
@@ -1878,6 +1889,11 @@ __global__ void __launch_bounds__(RCCfg<TY, BG>::NT, RCCfg<TY, BG>::MINB)
   Cell *const srd = sbk + 2 * PP;
   float *const sez = reinterpret_cast<float *>(srd + 2 * PP);  // [2][CE] (PRL)
   constexpr int CXE = C::CXE, CE = C::CE;
+  // correction form: (x, E) of the thread's black cells [4][NT], x of its
+  // updated red cells [2][NT]
+  [[maybe_unused]] float2 *const sxe = reinterpret_cast<float2 *>(srd + 2 * PP) + threadIdx.x;
+  [[maybe_unused]] float *const sxr =
+      reinterpret_cast<float *>(reinterpret_cast<float2 *>(srd + 2 * PP) + 4 * C::NT) + threadIdx.x;
   const int g = find_grid(off, ngrid, blockIdx.x);
   const Grid<float> &Gg = grids[g];
   if (!grid_active(active, Gg.field)) return;
@@ -2103,7 +2119,12 @@ __global__ void __launch_bounds__(RCCfg<TY, BG>::NT, RCCfg<TY, BG>::MINB)
     const float Ei = bgv(own).y, ubi = bgv(own).x;
     const float Bi = BG ? Ei + Ei * xi : 1.0f + xi;
     OpAcc<float, BG> A(di, Ei, xi, Bi, ubi);
-    auto nb = [&](const Cell &c) { A.reg(c.x, c.y, bgv(c).x, bgv(c).y); };
+    auto nb = [&](const Cell &c) {
+      if constexpr (BG)
+        A.reg_pb(c.x, c.y, c.z, c.w);
+      else
+        A.reg(c.x, c.y, 0.0f, 1.0f);
+    };
     if (DIR && gx == 0)
       A.ghost(face_value(Gg, 0, gx, gy, m));
     else
@@ -2190,8 +2211,9 @@ __global__ void __launch_bounds__(RCCfg<TY, BG>::NT, RCCfg<TY, BG>::MINB)
         if constexpr (BG) {
           R[s][K] = make_float4(ur, needr ? xr : 0.0f,
                                 odd ? pb[s].y : pb[s].x, odd ? pe[s].y : pe[s].x);
-          B[s][K] = make_float4(ub, xb, odd ? pb[s].x : pb[s].y,
-                                odd ? pe[s].x : pe[s].y);
+          const float Eb = odd ? pe[s].x : pe[s].y, Pb = __fmul_rn(Eb, xb);
+          B[s][K] = make_float4(ub, Pb, odd ? pb[s].x : pb[s].y, __fadd_rn(Eb, Pb));
+          if (s < NI) sxe[K * C::NT] = make_float2(xb, Eb);
         } else {
           R[s][K] = make_float2(ur, needr ? xr : 0.0f);
           B[s][K] = make_float2(ub, xb);
@@ -2252,7 +2274,13 @@ __global__ void __launch_bounds__(RCCfg<TY, BG>::NT, RCCfg<TY, BG>::MINB)
           const float un = newton(R[s][K1], FR[s][K1], sel(odd, B[s][K1], nx),
                                   sel(odd, nx, B[s][K1]), ym, yp, B[s][K2], B[s][K],
                                   gxe[s] + (odd ? 1 : 0), gyv[s], m);
-          R[s][K1] = with_u(R[s][K1], un);
+          if constexpr (BG) {
+            const float xn = ex(un), Er = R[s][K1].w, Pr = __fmul_rn(Er, xn);
+            R[s][K1] = make_float4(un, Pr, R[s][K1].z, __fadd_rn(Er, Pr));
+            if (s < NI) sxr[PK1 * C::NT] = xn;
+          } else {
+            R[s][K1] = with_u(R[s][K1], un);
+          }
           srd[PK1 * PP + q[s]] = R[s][K1];
         }
       }
@@ -2294,12 +2322,20 @@ __global__ void __launch_bounds__(RCCfg<TY, BG>::NT, RCCfg<TY, BG>::MINB)
             const Cell *rd = srd + PK2 * PP + q[s];
             const Cell ym = rd[-PX], yp = rd[PX];
             const Cell nx = rd[odd ? 1 : -1];
-            const float un = newton(B[s][K2], FB[s][K2], sel(odd, R[s][K2], nx), sel(odd, nx, R[s][K2]), ym,
+            Cell own = B[s][K2];
+            if constexpr (BG) {
+              const float2 xe = sxe[K2 * C::NT];
+              own.y = xe.x;
+              own.w = xe.y;
+            }
+            const float un = newton(own, FB[s][K2], sel(odd, R[s][K2], nx), sel(odd, nx, R[s][K2]), ym,
                         yp, R[s][K3], R[s][K1], gxe[s] + (odd ? 1 : 0), gyv[s], m);
             B[s][K2] = with_u(B[s][K2], un);
           }
           if (fl[s] & 2u) {
-            const Cell e = sel(odd, R[s][K2], B[s][K2]), o = sel(odd, B[s][K2], R[s][K2]);
+            Cell rr = R[s][K2];
+            if constexpr (BG) rr.y = sxr[PK2 * C::NT];
+            const Cell e = sel(odd, rr, B[s][K2]), o = sel(odd, B[s][K2], rr);
             const long long oo = (long long)m * plane + roff[s];
             *reinterpret_cast<float2 *>(uout + oo) = make_float2(e.x, o.x);
             *reinterpret_cast<float2 *>(xout + oo) = make_float2(e.y, o.y);
