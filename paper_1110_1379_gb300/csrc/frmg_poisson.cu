@@ -31,6 +31,7 @@
 #include <cmath>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "frmg.h"
@@ -356,132 +357,189 @@ __global__ void __launch_bounds__(kNT) k_lresid_restrict(PLevel F, PLevel C, dou
   }
 }
 
-// Tiled residual + restriction (the arithmetic of k_lresid_restrict): a block
+// Asynchronous global-to-shared copies of 4, 8 and 16 bytes (PTX cp.async).
+template <int N>
+__device__ __forceinline__ void cp_async(void *smem, const void *gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  if constexpr (N == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(sa), "l"(gmem), "n"(N)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() {
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Tiled residual + restriction (the residuals of k_lresid_restrict): a block
 // owns a 64 x 16 fine tile (32 x 8 coarse cells, one per thread) and a chunk
-// of kc coarse planes, and keeps a ring of four fine planes of e (tile plus a
-// one-cell halo) in shared memory: coarse plane K needs fine planes 2K-1 ..
-// 2K+2, and each step loads the next two (prefetched into registers while the
-// residuals of the current pair of fine planes are formed).  f is read by
-// each thread for its own 2 x 2 x 2 children.  Optional per-block norm
-// partials (sum d^2, max |d|).
+// of kc coarse planes, and marches over its fine planes.  They arrive by
+// asynchronous copies in a ring of four, two ahead of the one in use (16 bytes
+// a lane where rows are whole quads, else pairs); a thread keeps its 2 x 2 cells
+// of three planes in registers, takes x neighbours by shuffles and the rows
+// above and below from shared memory, and evaluates x-pairs as packed FP32
+// pairs.  On a patch the cells outside are zeros, and counted.  Bound by HBM and
+// the copies' latency; eight cells one by one from shared memory, f by scalar
+// loads and a division each took 0.363 ms at 512^3, this 0.196 (the memory time
+// of e, f and the coarse arrays is 0.18).  Optional per-block norm partials
+// (sum d^2, max |d|).
 constexpr int kLrTX = 64, kLrTY = 16;
 template <bool PATCH>
-__global__ void __launch_bounds__(256) k_lresid_restrict_tiled(PLevel F, PLevel C, int kc,
-                                                               double *partial) {
-  constexpr int LX = kLrTX + 2, LY = kLrTY + 2, PC = LX * LY, NT = 256;
-  constexpr int NLD = (PC + NT - 1) / NT;
-  __shared__ float se[4 * PC];
+__global__ void __launch_bounds__(256, 4) k_lresid_restrict_tiled(PLevel F, PLevel C, int kc,
+                                                                  double *partial) {
+  constexpr int TX = kLrTX, TY = kLrTY, NT = 256, NW = NT / 32;
+  static_assert(TY == 2 * NW && TX == 64, "two rows per warp, one pair per lane");
+  // a slot: rows -1 .. 16 of e, the columns left and right of the tile, rows 0 .. 15 of f
+  constexpr int EC = (TY + 2) * TX, AN = EC + 2 * TY, PL = AN + TY * TX;
+  __shared__ __align__(16) float smem[4 * PL];
   const int n0 = F.n0, n1 = F.n1, n2 = F.n2;
-  const int ntx = (n0 + kLrTX - 1) / kLrTX, nty = (n1 + kLrTY - 1) / kLrTY;
+  const int ntx = (n0 + TX - 1) / TX, nty = (n1 + TY - 1) / TY;
   int b = blockIdx.x;
-  const int X0 = (b % ntx) * kLrTX;
+  const int X0 = (b % ntx) * TX;
   b /= ntx;
-  const int Y0 = (b % nty) * kLrTY;
+  const int Y0 = (b % nty) * TY;
   b /= nty;
-  const int K0 = b * kc, K1 = min(K0 + kc, C.n2);
+  const int Z0 = 2 * b * kc, Z1 = min(Z0 + 2 * kc, n2);
   const long long plane = (long long)n0 * n1;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int gx = X0 + 2 * lane, gy = Y0 + 2 * w;
+  const bool valid = gx < n0 && gy < n1;
   auto wrapm = [](int v, int n) {
     int r = v % n;
     return r < 0 ? r + n : r;
   };
-  int roff[NLD];
-  bool lok[NLD];
-#pragma unroll
-  for (int k = 0; k < NLD; k++) {
-    const int q = threadIdx.x + k * NT;
-    roff[k] = 0;
-    lok[k] = false;
-    if (q < PC) {
-      const int gx = X0 - 1 + q % LX, gy = Y0 - 1 + q / LX;
-      if (PATCH) {
-        lok[k] = gx >= 0 && gx < n0 && gy >= 0 && gy < n1;
-        roff[k] = lok[k] ? gy * n0 + gx : 0;
-      } else {
-        lok[k] = true;
-        roff[k] = wrapm(gy, n1) * n0 + wrapm(gx, n0);
-      }
-    }
+  // What a lane copies of a plane (offsets, -1: none): 16 bytes of row 2 w
+  // (lanes 0 - 15) or 2 w + 1, and of the row beyond the tile (first and last
+  // warp), or pairs of both rows; the first and last lane also the cells left
+  // and right of the tile.
+  auto at = [&](int x, int y) -> int {
+    if (PATCH) return x >= 0 && x < n0 && y >= 0 && y < n1 ? y * n0 + x : -1;
+    return wrapm(y, n1) * n0 + wrapm(x, n0);
+  };
+  const bool quad = !(n0 & 3);
+  const int lx = quad ? 4 * (lane & 15) : 2 * lane, ly = quad ? lane >> 4 : 0;
+  const int o0 = at(X0 + lx, gy + ly);
+  const int oh = w == 0 && !(quad && ly) ? at(X0 + lx, gy - 1)
+                 : (w == NW - 1 && !(quad && ly) ? at(X0 + lx, gy + 2) : -1);
+  const int ex = lane == 0 ? X0 - 1 : X0 + TX;
+  const bool edge = lane == 0 || lane == 31;
+  const int oe = edge ? at(ex, gy) : -1;  // (and the row above: n1 is even)
+  const int qc = (2 * w + 1 + ly) * TX + lx;
+  const int qh = (w == 0 ? 0 : TY + 1) * TX + lx;
+  const int qe = EC + (lane == 0 ? 0 : TY) + 2 * w;
+  const int q0 = (2 * w + 1) * TX + 2 * lane;
+  auto inz = [&](int p) { return !PATCH || (p >= 0 && p < n2); };
+  if (PATCH) {  // what lies outside the grid is never copied to
+    for (int q = threadIdx.x; q < 4 * PL; q += NT) smem[q] = 0.0f;
+    __syncthreads();
   }
-  float pv[2][NLD];
-  // fine plane z (may lie outside a patch: never read then) into registers
-  auto fetch = [&](int r, int z) {
-    const bool vz = !PATCH || (z >= 0 && z < n2);
-    const long long zo = (long long)(PATCH ? z : wrapm(z, n2)) * plane;
-#pragma unroll
-    for (int k = 0; k < NLD; k++) pv[r][k] = (vz && lok[k]) ? F.e[zo + roff[k]] : 0.0f;
-  };
-  auto commit = [&](int r, int slot) {
-#pragma unroll
-    for (int k = 0; k < NLD; k++) {
-      const int q = threadIdx.x + k * NT;
-      if (q < PC) se[slot * PC + q] = pv[r][k];
-    }
-  };
-  // this thread's coarse cell of the tile
-  const int cx = threadIdx.x & 31, cy = threadIdx.x >> 5;
-  const int I = X0 / 2 + cx, J = Y0 / 2 + cy;
-  const bool own = 2 * I < n0 && 2 * J < n1;
-  float ss = 0.0f, mx = 0.0f;
-  // planes 2K0-1 .. 2K0+2 into slots 0..3 (slot of fine plane z: (z - 2K0 + 1) & 3)
-  fetch(0, 2 * K0 - 1);
-  fetch(1, 2 * K0);
-  commit(0, 0);
-  commit(1, 1);
-  fetch(0, 2 * K0 + 1);
-  fetch(1, 2 * K0 + 2);
-  commit(0, 2);
-  commit(1, 3);
-  __syncthreads();
-  for (int K = K0; K < K1; K++) {
-    const bool more = K + 1 < K1;
-    if (more) {
-      fetch(0, 2 * K + 3);
-      fetch(1, 2 * K + 4);
-    }
-    if (own) {
-      float sd = 0.0f;
-#pragma unroll
-      for (int q = 0; q < 8; q++) {
-        const int dx = q & 1, dy = (q >> 1) & 1, dz = q >> 2;
-        const int i = 2 * I + dx, j = 2 * J + dy, k = 2 * K + dz;
-        const int lx = 1 + 2 * cx + dx, ly = 1 + 2 * cy + dy;
-        const int sm = ((k - 1 - 2 * K0 + 1) & 3) * PC, sc = ((k - 2 * K0 + 1) & 3) * PC,
-                  sp = ((k + 1 - 2 * K0 + 1) & 3) * PC;
-        const int o = ly * LX + lx;
-        float s = 0.0f;
-        int nm = 0;
-        if (PATCH) {
-          if (i > 0) s += se[sc + o - 1]; else nm++;
-          if (i < n0 - 1) s += se[sc + o + 1]; else nm++;
-          if (j > 0) s += se[sc + o - LX]; else nm++;
-          if (j < n1 - 1) s += se[sc + o + LX]; else nm++;
-          if (k > 0) s += se[sm + o]; else nm++;
-          if (k < n2 - 1) s += se[sp + o]; else nm++;
-        } else {
-          s += se[sc + o - 1];
-          s += se[sc + o + 1];
-          s += se[sc + o - LX];
-          s += se[sc + o + LX];
-          s += se[sm + o];
-          s += se[sp + o];
+  auto fetch = [&](int p) {
+    if (p <= Z1 && inz(p)) {
+      const bool own = p >= Z0 && p < Z1;
+      const long long zo = (long long)(PATCH ? p : (p < 0 ? p + n2 : (p >= n2 ? p - n2 : p))) * plane;
+      float *h = smem + ((p - Z0 + 1) & 3) * PL;
+      const float *v = F.e + zo, *fv = F.f + zo;
+      if (quad) {
+        if (o0 >= 0) {
+          cp_async<16>(h + qc, v + o0);
+          if (own) cp_async<16>(h + AN + qc - TX, fv + o0);
         }
-        const long long c = (long long)k * plane + (long long)j * n0 + i;
-        const float d = F.f[c] - (s - (6.0f + (float)nm) * se[sc + o]) / F.h2;
-        sd += d;
-        ss = fmaf(d, d, ss);
-        mx = fmaxf(mx, fabsf(d));
+        if (own && oh >= 0) cp_async<16>(h + qh, v + oh);
+      } else {
+        if (o0 >= 0) {
+          cp_async<8>(h + qc, v + o0);
+          cp_async<8>(h + qc + TX, v + o0 + n0);
+          if (own) {
+            cp_async<8>(h + AN + qc - TX, fv + o0);
+            cp_async<8>(h + AN + qc, fv + o0 + n0);
+          }
+        }
+        if (own && oh >= 0) cp_async<8>(h + qh, v + oh);
       }
-      const long long t = ((long long)K * C.n1 + J) * C.n0 + I;
-      C.f[t] = 0.125f * sd;
-      C.e[t] = 0.0f;
+      if (own && oe >= 0) {
+        cp_async<4>(h + qe, v + oe);
+        cp_async<4>(h + qe + 1, v + oe + n0);
+      }
+    }
+    cp_async_commit();
+  };
+  auto ld2 = [](const float *p) { return *reinterpret_cast<const float2 *>(p); };
+  const float h2 = F.h2, rh2 = 1.0f / h2;
+  float2 sd = make_float2(0.f, 0.f), s2 = sd;
+  float mx = 0.0f;
+  float2 r[4][2];  // the own rows of planes m - 1, m, m + 1 (by plane modulo 4)
+  r[3][0] = r[3][1] = r[2][0] = r[2][1] = sd;
+
+  auto step = [&](auto Kc, int p) {
+    constexpr int K = decltype(Kc)::value, K1 = (K + 3) & 3, K2 = (K + 2) & 3;
+    fetch(p + 2);  // into the slot of plane p - 2, last read before the last barrier
+    cp_async_wait<2>();
+    __syncwarp();  // a warp's rows are copied by all of its lanes
+#pragma unroll
+    for (int k = 0; k < 2; k++)
+      r[K][k] = inz(p) ? ld2(smem + K * PL + q0 + k * TX) : make_float2(0.f, 0.f);
+    const int m = p - 1;
+    if (m >= Z0) {
+      const float *sm = smem + K1 * PL;
+#pragma unroll
+      for (int k = 0; k < 2; k++) {
+        const float2 own = r[K1][k];
+        float lo = __shfl_up_sync(0xffffffffu, own.y, 1);
+        float hi = __shfl_down_sync(0xffffffffu, own.x, 1);
+        if (edge) (lane == 0 ? lo : hi) = sm[qe + k];
+        const float2 V = ld2(sm + q0 + (k ? 2 * TX : -TX));
+        float2 R = make_float2(own.y, hi);
+        float2 cnt = make_float2(6.0f, 6.0f);
+        if (PATCH) {
+          // lanes at the end of a ragged row: the pair beyond it holds zeros
+          const float my = (float)((gy + k == 0) + (gy + k == n1 - 1) + (m == 0) + (m == n2 - 1));
+          cnt.x += my + (float)(gx == 0);
+          cnt.y += my + (float)(gx + 2 == n0);
+        }
+        float2 t = add2(make_float2(lo, own.x), R);
+        t = add2(t, k ? r[K1][0] : V);
+        t = add2(t, k ? V : r[K1][1]);
+        t = add2(t, r[K2][k]);
+        t = add2(t, r[K][k]);
+        // one rounding, as in k_lresid_restrict: with 6 e rounded first, a large
+        // constant part of e (free on a periodic grid) left a residual of its own
+        t = fma2(make_float2(-cnt.x, -cnt.y), own, t);
+        // t / h^2: the product with the rounded reciprocal and one correction
+        // by its exact remainder (Markstein 1990)
+        float2 q = mul2(t, splat2(rh2));
+        q = fma2(fma2(q, splat2(-h2), t), splat2(rh2), q);
+        const float2 d = sub2(ld2(sm + AN + q0 + (k - 1) * TX), q);
+        if (valid) {
+          sd = add2(sd, d);
+          s2 = fma2(d, d, s2);
+          mx = fmaxf(mx, fmaxf(fabsf(d.x), fabsf(d.y)));
+        }
+      }
+      if (((m - Z0) & 1) && valid) {
+        const long long t = ((long long)(m >> 1) * C.n1 + (gy >> 1)) * C.n0 + (gx >> 1);
+        C.f[t] = 0.125f * (sd.x + sd.y);
+        C.e[t] = 0.0f;
+        sd = make_float2(0.f, 0.f);
+      }
     }
     __syncthreads();
-    if (more) {
-      commit(0, (2 * K + 3 - 2 * K0 + 1) & 3);
-      commit(1, (2 * K + 4 - 2 * K0 + 1) & 3);
+  };
+  fetch(Z0 - 1);
+  fetch(Z0);
+  for (int p = Z0 - 1; p <= Z1; p += 4) {  // an even number of planes
+    step(std::integral_constant<int, 0>{}, p);
+    step(std::integral_constant<int, 1>{}, p + 1);
+    if (p + 2 <= Z1) {
+      step(std::integral_constant<int, 2>{}, p + 2);
+      step(std::integral_constant<int, 3>{}, p + 3);
     }
-    __syncthreads();
   }
+  cp_async_wait<0>();
+  float ss = s2.x + s2.y;
   if (partial) {
     for (int o = 16; o > 0; o >>= 1) {
       ss += __shfl_down_sync(0xffffffffu, ss, o);
@@ -1617,35 +1675,38 @@ extern "C" int fr_poisson_solve(frmg_ctx *ctx, const double *density, const doub
         }
         S.zc.push_back(zcl);
         S.nblk_t.push_back(nbt);
-        // tiled prolongation onto this level (from the next coarser one) where
-        // its 64 x 16 tiles times coarse-plane chunks fill the GPU: chunks of
-        // kc coarse planes minimise (waves of 8 resident blocks per SM) x (kc + 1)
-        int kcp = 0, nbp = 0;
+        // tiled prolongation onto this level (from the next coarser one) and
+        // residual + restriction from it, where the 64 x 16 tiles times chunks
+        // of coarse planes fill the GPU: the chunk minimises (waves of resident
+        // blocks, 8 and 4 per SM) x (chunk + the planes read beyond it)
+        int kcp = 0, nbp = 0, kcr = 0, nbr = 0;
         if (l + 1 < nl && nbt > 0) {
           int sms = 0, dev = 0;
           PCK(cudaGetDevice(&dev));
           PCK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-          const long long slots = 8ll * std::max(sms, 1);
           const long long tiles = (long long)((m[0] + 63) / 64) * ((m[1] + 15) / 16);
           const int c2 = m[2] / 2;
-          double best = 1e300;
-          for (int c = 1; c <= c2; c++) {
-            const int z = (c2 + c - 1) / c;
-            const long long blocks = tiles * ((c2 + z - 1) / z);
-            const double cost = std::ceil((double)blocks / slots) * (z + 1);
-            if (cost < best - 1e-9) {
-              best = cost;
-              kcp = z;
+          auto pick = [&](int per_sm, int beyond, int &kc, int &nb) {
+            const long long slots = (long long)per_sm * std::max(sms, 1);
+            double best = 1e300;
+            for (int c = 1; c <= c2; c++) {
+              const int z = (c2 + c - 1) / c;
+              const long long blocks = tiles * ((c2 + z - 1) / z);
+              const double cost = std::ceil((double)blocks / slots) * (z + beyond);
+              if (cost < best - 1e-9) {
+                best = cost;
+                kc = z;
+              }
             }
-          }
-          nbp = (int)(tiles * ((c2 + kcp - 1) / kcp));
+            nb = (int)(tiles * ((c2 + kc - 1) / kc));
+          };
+          pick(8, 1, kcp, nbp);
+          pick(4, 2, kcr, nbr);
         }
         S.kc_p.push_back(kcp);
         S.nblk_p.push_back(nbp);
-        // the residual + restriction from this level uses the same tiles and
-        // coarse-plane chunks (blocks of 256 threads, one per coarse cell)
-        S.kc_r.push_back(kcp);
-        S.nblk_r.push_back(nbp);
+        S.kc_r.push_back(kcr);
+        S.nblk_r.push_back(nbr);
         S.lev.push_back(L);
         for (int d = 0; d < 3; d++) m[d] /= 2;
         hl *= 2.0;

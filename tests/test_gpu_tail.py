@@ -244,3 +244,42 @@ def test_sweeps_over_the_range_of_u(C, tiled, c):
     u = torch.from_numpy(u0.astype(np.float32)).cuda()
     C.smooth_f32(u, 2, f=torch.from_numpy(f.astype(np.float32)).cuda(), tiled=tiled, **P)
     assert np.abs(host(u) - ref).max() < 2e-5 * max(1.0, abs(c))
+
+
+@pytest.mark.parametrize("shape,patch", [((36, 34, 132), True), ((96, 48, 64), False),
+                                         ((32, 64, 96), False), ((96, 96, 96), False)])
+def test_poisson_tiled_residual_and_restriction(C, shape, patch):
+    """Tiles that end within the grid, and periodic grids whose coarsest sides of
+    3 amplify a residual that does not sum to zero: the oracle's equation is
+    met to the tolerance, in the number of cycles multigrid takes."""
+    from oracle import poisson as PO
+    rho, P = _case(shape, 9000)
+    u = 0.3 * np.random.default_rng(9001).standard_normal(shape)
+    h = 1.0 / 256 if patch else 1.0 / shape[2]
+    s = PO.source(u, rho, **P)
+    phi = torch.zeros(shape, dtype=torch.float64, device="cuda")
+    kw = {}
+    if patch:
+        phib = np.random.default_rng(9002).uniform(-1e-3, 1e-3, sum(O.face_sizes(shape)))
+        kw = dict(phib=dev(phib), h=h)
+    st, stats, _ = C.poisson(dev(rho), dev(u), phi, tol=1e-9, **kw, **P)
+    assert st == 0 and stats.res_rms <= 1e-9 and stats.vcycles <= 25
+    if patch:
+        assert np.sqrt(np.mean(PO.residual(host(phi), s, h, phib) ** 2)) <= 2e-9
+    else:
+        ref, _ = PO.solve_periodic(s, h)
+        assert np.abs(host(phi) - ref).max() <= 1e-7 / 39.0
+
+
+@pytest.mark.parametrize("shape", [(36, 34, 66), (24, 36, 130), (34, 36, 70)])
+def test_poisson_tiled_rows_of_pairs(C, shape):
+    """Rows that are not whole quads (their coarsest grids are odd, so these
+    solves stall later): the first cycles contract as multigrid does, a factor
+    of 10 or more each."""
+    rho, P = _case(shape, 9000)
+    u = 0.3 * np.random.default_rng(9001).standard_normal(shape)
+    phib = np.random.default_rng(9002).uniform(-1e-3, 1e-3, sum(O.face_sizes(shape)))
+    phi = torch.zeros(shape, dtype=torch.float64, device="cuda")
+    _, s, _ = C.poisson(dev(rho), dev(u), phi, tol=1e-9, phib=dev(phib), h=1.0 / 256, **P)
+    h = [abs(v) for v in list(s.hist)[:4]]
+    assert h[3] <= 1e-3 * h[0], h
