@@ -1766,10 +1766,9 @@ extern "C" int fr_poisson_solve(frmg_ctx *ctx, const double *density, const doub
       if (outer > 0 && r > prev) throw PError{FR_EDIVERGED, "defect grew"};
       prev = r;
       if (sv.vcycles >= o.max_vcycles) break;
-      // FP32 correction solve: stop near the FP32 floor (2e-5 of its start: the
-      // next cycle rarely gains a factor of two there) or when the cycle
-      // contraction stalls
-      double rp = HUGE_VAL, rbest = HUGE_VAL;
+      // FP32 correction solve: stop near the FP32 floor (1e-5 of its start)
+      // or when the cycle contraction stalls
+      double rp = HUGE_VAL;
       for (int k = 0; k < o.max_vcycles; k++) {
         if (S.lev.size() == 1) {
           k_lcoarsest<<<1, kNT, 0, st>>>(S.lev[0], 500);
@@ -1784,13 +1783,9 @@ extern "C" int fr_poisson_solve(frmg_ctx *ctx, const double *density, const doub
         const double rr = std::sqrt(a2 / (double)nc);  // residual after pre-smoothing
         push(rr);
         const double pred = rp < HUGE_VAL ? rr * std::sqrt(rr / rp) : rr;
-        // near the FP32 floor (1e-4 of the start) a cycle that contracts three
-        // times less than the best one has reached it
-        const double ratio = rr / rp;
-        if (!(ratio < 0.75) || rr <= 2e-5 * r || (rr <= 1e-4 * r && ratio > 3.0 * rbest) ||
-            pred <= 0.5 * tol || sv.vcycles >= o.max_vcycles)
+        if (!(rr < 0.75 * rp) || rr <= 1e-5 * r || pred <= 0.5 * tol ||
+            sv.vcycles >= o.max_vcycles)
           break;
-        if (k > 0) rbest = std::min(rbest, ratio);
         rp = rr;
       }
       k_pupdate<<<nb, kNT, 0, st>>>(P, S.lev[0].e);
