@@ -249,6 +249,24 @@ __global__ void __launch_bounds__(kNT) k_sy_fas_rhs(SLevel<T> Cs) {
   Cs.f[t] = N - Cs.f[t];
 }
 
+// An x-pair of a level's u.
+__device__ __forceinline__ void sy_ld2(const float *p, float (&v)[2]) {
+  const float2 w = *reinterpret_cast<const float2 *>(p);
+  v[0] = w.x;
+  v[1] = w.y;
+}
+__device__ __forceinline__ void sy_st2(float *p, const float (&v)[2]) {
+  *reinterpret_cast<float2 *>(p) = make_float2(v[0], v[1]);
+}
+__device__ __forceinline__ void sy_ld2(const double *p, double (&v)[2]) {
+  v[0] = p[0];
+  v[1] = p[1];
+}
+__device__ __forceinline__ void sy_st2(double *p, const double (&v)[2]) {
+  p[0] = v[0];
+  p[1] = v[1];
+}
+
 // u^h += P(u^H - R u^h): the trilinear 27/9/3/1 prolongation (Sec. V.A.3) of
 // the coarse correction onto every fine cell, periodic.  A block owns 32 x 8
 // coarse columns and zc coarse planes: e = u^H - uR of a plane (with a halo of
@@ -257,11 +275,11 @@ __global__ void __launch_bounds__(kNT) k_sy_fas_rhs(SLevel<T> Cs) {
 // is one multiply-add per child.  Bound by memory (u read and written, u^H and
 // uR read).  One thread per coarse cell reading its 27 neighbours of both
 // arrays through the L1 was bound by those 54 loads: 0.437 ms per 512^3 level,
-// now 0.21.
+// now 0.21.  FP32 u is read and written as x-pairs; FP64 u, which on the finest
+// level may be the caller's array (aligned to 8 bytes only), cell by cell.
 template <typename T>
 __global__ void __launch_bounds__(kNT) k_sy_prolong(SLevel<T> F, SLevel<T> Cs, int zc) {
   constexpr int PX = kPrX + 2, PP = PX * (kPrY + 2), NS = (PP + kNT - 1) / kNT;
-  using T2 = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
   __shared__ T se[2][PP];
   const int c0 = Cs.n0, c1 = Cs.n1, c2 = Cs.n2;
   const int ntx = (c0 + kPrX - 1) / kPrX, nty = (c1 + kPrY - 1) / kPrY;
@@ -303,11 +321,11 @@ __global__ void __launch_bounds__(kNT) k_sy_prolong(SLevel<T> F, SLevel<T> Cs, i
       if (off[r] >= 0) sb[threadIdx.x + r * kNT] = e[r];
     if (k < K1) load(k + 1);
     const bool out = own && k > K0;  // the children of plane k - 1 are complete
-    T2 fu[4];
-    T2 *fp = reinterpret_cast<T2 *>(F.u + (2 * (k - 1) * fplane + 2ll * J * F.n0 + 2 * I));
+    T fu[4][2];
+    T *fp = F.u + (2 * (k - 1) * fplane + 2ll * J * F.n0 + 2 * I);
     if (out) {
 #pragma unroll
-      for (int r = 0; r < 4; r++) fu[r] = fp[((r >> 1) * fplane + (r & 1) * F.n0) / 2];
+      for (int r = 0; r < 4; r++) sy_ld2(fp + (r >> 1) * fplane + (r & 1) * F.n0, fu[r]);
     }
     __syncthreads();
     const T *s = sb + (ly + 1) * PX + lx + 1;
@@ -327,9 +345,9 @@ __global__ void __launch_bounds__(kNT) k_sy_prolong(SLevel<T> F, SLevel<T> Cs, i
       for (int r = 0; r < 4; r++) {
         const int cz = r >> 1, q = 2 * (r & 1);
         const T *m = a[1], *z = cz ? a[2] : a[0];
-        fu[r].x += (T(3) * m[q] + z[q]) * T(1.0 / 64.0);
-        fu[r].y += (T(3) * m[q + 1] + z[q + 1]) * T(1.0 / 64.0);
-        fp[((r >> 1) * fplane + (r & 1) * F.n0) / 2] = fu[r];
+        fu[r][0] += (T(3) * m[q] + z[q]) * T(1.0 / 64.0);
+        fu[r][1] += (T(3) * m[q + 1] + z[q + 1]) * T(1.0 / 64.0);
+        sy_st2(fp + (r >> 1) * fplane + (r & 1) * F.n0, fu[r]);
       }
     }
   }

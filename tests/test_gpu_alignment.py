@@ -1,0 +1,43 @@
+"""Caller's device arrays at the smallest alignment their type has (a slice of a
+larger tensor): the same results, bit for bit, as with aligned arrays."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from gpu_common import ctx, dev, host  # noqa: E402
+from paper_1110_1379_gb300 import synth  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def C():
+    c = ctx()
+    yield c
+    c.close()
+
+
+def offset(a, dtype=torch.float64):
+    """The array on the device one element past an aligned address."""
+    buf = torch.empty(a.size + 1, dtype=dtype, device="cuda")
+    t = buf[1:].view(a.shape)
+    assert t.data_ptr() % (2 * t.element_size()) == t.element_size()
+    t.copy_(torch.from_numpy(np.ascontiguousarray(a)))
+    return t
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("shape", [(16, 16, 16), (24, 40, 72)])
+def test_symmetron_arrays_at_odd_multiples_of_8_bytes(C, prec, shape):
+    """The FP64 V-cycle works on the caller's chi itself."""
+    P = dict(a=1.0, a_ssb=0.5, lambda0=1.0, box=0.5 * shape[2])
+    rho = synth.lognormal_density(shape, 7, sigma=1.0)
+    chi0 = 0.5 + 0.1 * np.random.default_rng(8).standard_normal(shape)
+    out = []
+    for put in (dev, offset):
+        chi = put(chi0)
+        C.symmetron(put(rho), chi, tol=1e-30, prec=prec, initial_guess=1, max_vcycles=3, **P)
+        out.append(host(chi))
+    assert not np.array_equal(out[0], chi0)
+    assert np.array_equal(out[0], out[1])
