@@ -264,9 +264,10 @@ __device__ __forceinline__ void df_defect(const DFGrid &G, float *r32, float *ub
     reinterpret_cast<float2 *>(E32)[t] = make_float2(expf(ui.h.x), expf(ui.h.y));
     reinterpret_cast<float2 *>(delta)[t] = make_float2(0.0f, 0.0f);
     reinterpret_cast<float2 *>(x32)[t] = make_float2(0.0f, 0.0f);
-    if (dout)
-      reinterpret_cast<double2 *>(dout)[t] =
-          make_double2(join_bits(d.h.x, d.l.x), join_bits(d.h.y, d.l.y));
+    if (dout) {  // the caller's array, aligned to 8 bytes only
+      dout[2 * t] = join_bits(d.h.x, d.l.x);
+      dout[2 * t + 1] = join_bits(d.h.y, d.l.y);
+    }
     s2 = fmaf(dv.y, dv.y, dv.x * dv.x);
     mx = fmaxf(fabsf(dv.x), fabsf(dv.y));
   }

@@ -1215,8 +1215,7 @@ __global__ void __launch_bounds__(kNT)
 // x-pair per thread.  The sum of the neighbours carries its rounding errors and
 // the low parts in one FP32 sum (TwoSum per neighbour) and is normalised once.
 __global__ void __launch_bounds__(kNT)
-    k_pdefect(PFine P, float smh, float sml, float *f32, float *e32, double *partial,
-              double *dout) {
+    k_pdefect(PFine P, float smh, float sml, float *f32, float *e32, double *partial) {
   const long long t = (long long)blockIdx.x * kNT + threadIdx.x;
   float ss = 0.0f, mx = 0.0f;
   if (t < (P.ncell >> 1)) {
@@ -1277,9 +1276,6 @@ __global__ void __launch_bounds__(kNT)
     const float2 dv = add2(d.h, d.l);
     reinterpret_cast<float2 *>(f32)[t] = make_float2(-dv.x, -dv.y);
     reinterpret_cast<float2 *>(e32)[t] = make_float2(0.0f, 0.0f);
-    if (dout)
-      reinterpret_cast<double2 *>(dout)[t] =
-          make_double2(join_bits(d.h.x, d.l.x), join_bits(d.h.y, d.l.y));
     ss = fmaf(dv.y, dv.y, dv.x * dv.x);
     mx = fmaxf(fabsf(dv.x), fabsf(dv.y));
   }
@@ -1748,7 +1744,7 @@ extern "C" int fr_poisson_solve(frmg_ctx *ctx, const double *density, const doub
                               : 0;
     double *partial0 = A.get<double>(2 * std::max<long long>(nbc, 1));
     for (int outer = 0; outer < o.max_outer; outer++) {
-      k_pdefect<<<nbp, kNT, 0, st>>>(P, smh, sml, S.lev[0].f, S.lev[0].e, partial, nullptr);
+      k_pdefect<<<nbp, kNT, 0, st>>>(P, smh, sml, S.lev[0].f, S.lev[0].e, partial);
       PLAUNCH(ctx);
       double s2, dmax;
       psum(partial, nbp, s2, dmax);

@@ -41,3 +41,18 @@ def test_symmetron_arrays_at_odd_multiples_of_8_bytes(C, prec, shape):
         out.append(host(chi))
     assert not np.array_equal(out[0], chi0)
     assert np.array_equal(out[0], out[1])
+
+
+def test_residual_df_arrays_at_odd_multiples_of_8_bytes(C):
+    """The double-float defect is written to the caller's d."""
+    shape = (12, 16, 20)
+    P = dict(box=40.0, a=1.0, omega_m=0.24, fr0=1e-5)
+    rho = synth.lognormal_density(shape, 9, sigma=1.0)
+    u = 0.3 * np.random.default_rng(10).standard_normal(shape)
+    out = []
+    for put in (dev, offset):
+        d = put(np.zeros(shape))
+        C.residual_df(put(u), put(rho), d, **P)
+        out.append(host(d))
+    assert np.abs(out[0]).max() > 0
+    assert np.array_equal(out[0], out[1])
