@@ -3471,10 +3471,19 @@ int fr_smooth_f32(frmg_ctx *ctx, float *u, const float *bg, const float *f, cons
     G.x = S.get<float>(nc);
     k_expm1<float><<<nblocks(nc), 256, 0, st>>>(G.u, G.x, nc);
     CK_LAUNCH(ctx);
-    G.f = stage(S, back, f, nc, true, false, st);
+    // the sweeps read these arrays as x-pairs: a copy where the caller's starts
+    // at an odd multiple of 4 bytes
+    auto pairs = [&](const float *p) -> const float * {
+      const float *v = stage(S, back, p, nc, true, false, st);
+      if (!(reinterpret_cast<size_t>(v) & 7)) return v;
+      float *w = S.get<float>(nc);
+      CK(cudaMemcpyAsync(w, v, nc * sizeof(float), cudaMemcpyDeviceToDevice, st));
+      return w;
+    };
+    G.f = pairs(f);
     G.bnd = stage(S, back, ub, ub ? face_total(dims) : 0, true, false, st);
     if (bg) {
-      G.ubg = stage(S, back, bg, nc, true, false, st);
+      G.ubg = pairs(bg);
       float *E = S.get<float>(nc);
       k_expf<<<nblocks(nc), 256, 0, st>>>(G.ubg, E, nc);
       CK_LAUNCH(ctx);

@@ -56,3 +56,22 @@ def test_residual_df_arrays_at_odd_multiples_of_8_bytes(C):
         out.append(host(d))
     assert np.abs(out[0]).max() > 0
     assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("tiled", [0, 1, 8, 16])
+@pytest.mark.parametrize("corr", [False, True])
+def test_smooth_f32_arrays_at_odd_multiples_of_4_bytes(C, tiled, corr):
+    """The tiled FP32 sweeps read the caller's right-hand side and background."""
+    shape = (20, 24, 36)
+    P = dict(box=40.0, a=1.0, omega_m=0.24, fr0=1e-5)
+    rng = np.random.default_rng(11)
+    u0 = 0.1 * rng.standard_normal(shape).astype(np.float32)
+    bg = rng.standard_normal(shape).astype(np.float32) if corr else None
+    f = 0.05 * rng.standard_normal(shape).astype(np.float32)
+    out = []
+    for put in (lambda a: torch.from_numpy(a).cuda(), lambda a: offset(a, torch.float32)):
+        u = put(u0)
+        C.smooth_f32(u, 2, f=put(f), bg=None if bg is None else put(bg), tiled=tiled, **P)
+        out.append(host(u))
+    assert not np.array_equal(out[0], u0)
+    assert np.array_equal(out[0], out[1])
