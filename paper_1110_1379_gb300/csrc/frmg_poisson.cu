@@ -37,6 +37,7 @@
 #include "frmg.h"
 #include "frmg_dfmath.cuh"
 #include "frmg_internal.h"
+#include "frmg_perdevice.h"
 
 using namespace frmg;
 
@@ -1078,16 +1079,19 @@ __global__ void __launch_bounds__(kLtNT, 1) k_ltail(const LtDesc *desc) {
   for (int t = tid; t < ntop; t += kLtNT) T.ge[c0 + t] = sm[T.e + T.plane + t];
 }
 
-// Blocks per cluster the device takes (16 where it can).
+// Blocks per cluster the current device takes (16 where it can); also sets the
+// kernel's attributes there.
 constexpr size_t kLtSmem = 220 * 1024;
 template <bool PATCH>
 int lt_cluster() {
-  static int best = 0;
-  if (!best) {
+  static PerDevice<int> best;
+  int dev = 0;
+  PCK(cudaGetDevice(&dev));
+  return best.get(dev, []() {
     auto *k = k_ltail<PATCH>;
     PCK(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     PCK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLtSmem));
-    for (int cs = kLtCluster; cs > 0 && !best; cs /= 2) {
+    for (int cs = kLtCluster; cs > 0; cs /= 2) {
       cudaLaunchConfig_t c = {};
       c.gridDim = dim3(cs);
       c.blockDim = dim3(kLtNT);
@@ -1099,12 +1103,11 @@ int lt_cluster() {
       c.attrs = a;
       c.numAttrs = 1;
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, k, &c) == cudaSuccess && n > 0) best = cs;
-      else cudaGetLastError();
+      if (cudaOccupancyMaxActiveClusters(&n, k, &c) == cudaSuccess && n > 0) return cs;
+      cudaGetLastError();
     }
-    if (!best) best = 1;
-  }
-  return best;
+    return 1;
+  });
 }
 
 // ---- double-float fine level

@@ -30,6 +30,7 @@
 
 #include "frmg.h"
 #include "frmg_internal.h"
+#include "frmg_perdevice.h"
 #include "frmg_kernels.cuh"
 #include "frmg_tail.cuh"
 #include "frmg_df.cuh"
@@ -553,15 +554,30 @@ static int red_chunks(const std::vector<int> &off) {
   return maxc <= 2 * kRedChunk ? 0 : (maxc + kRedChunk - 1) / kRedChunk;
 }
 
+static int current_device() {
+  int dev = 0;
+  CK(cudaGetDevice(&dev));
+  return dev;
+}
+
 static int sm_count() {
-  static int n = 0;
-  if (n <= 0) {
-    int dev = 0;
-    CK(cudaGetDevice(&dev));
+  static PerDevice<int> count;
+  const int dev = current_device();
+  return count.get(dev, [&]() {
+    int n = 0;
     CK(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
-    if (n <= 0) n = 1;
-  }
-  return n;
+    return std::max(n, 1);
+  });
+}
+
+// Allows a kernel `smem` bytes of dynamic shared memory on the current device,
+// once per device (set: the kernel's own).
+template <typename K>
+static void allow_smem(PerDevice<bool> &set, K kernel, size_t smem) {
+  set.get(current_device(), [&]() {
+    CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    return true;
+  });
 }
 
 // Resident blocks per SM of a kernel launched with `threads` threads and
@@ -848,15 +864,16 @@ struct Hier {
   T *cur_x(int pi, int l) const { return par[l] ? lev[pi][l].x2 : lev[pi][l].x; }
 };
 
-// Most blocks per cluster that a tail may use with `smem` bytes each.
+// Most blocks per cluster that a tail may use with `smem` bytes each (it also
+// sets the kernel's attributes on the current device).
 template <typename T, bool BG, bool DIR>
 static int tail_cluster(size_t smem) {
-  static int best = 0;
-  if (!best) {
+  static PerDevice<int> best;
+  return best.get(current_device(), [&]() {
     auto *k = k_tail<T, BG, DIR>;
     CK(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    for (int cs = kTailCluster; cs > 0 && !best; cs /= 2) {
+    for (int cs = kTailCluster; cs > 0; cs /= 2) {
       cudaLaunchConfig_t c = {};
       c.gridDim = dim3(cs);
       c.blockDim = dim3(tail_threads<T>());
@@ -868,12 +885,11 @@ static int tail_cluster(size_t smem) {
       c.attrs = a;
       c.numAttrs = 1;
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, k, &c) == cudaSuccess && n > 0) best = cs;
-      else cudaGetLastError();
+      if (cudaOccupancyMaxActiveClusters(&n, k, &c) == cudaSuccess && n > 0) return cs;
+      cudaGetLastError();
     }
-    if (!best) best = 1;
-  }
-  return best;
+    return 1;
+  });
 }
 
 // Shared memory a tail's block may use (227 KB per block less the static part).
@@ -1084,12 +1100,8 @@ static void launch_tiled_k(frmg_ctx *ctx, LevelSet<float> &s, const int *active,
                            cudaStream_t st) {
   using TC = TileCfg<S, kTX, kTY>;
   size_t sm = TC::smem(BG);
-  static bool attr_set = false;
-  if (!attr_set) {
-    CK(cudaFuncSetAttribute(k_smooth_tiled<BG, DIR, S, kTX, kTY>,
-                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    attr_set = true;
-  }
+  static PerDevice<bool> set;
+  allow_smem(set, k_smooth_tiled<BG, DIR, S, kTX, kTY>, sm);
   k_smooth_tiled<BG, DIR, S, kTX, kTY><<<s.nblk_tile, TC::NT, sm, st>>>(s.d, s.d_off_tile,
                                                                         s.size(), s.zc, active, par);
 }
@@ -1100,12 +1112,8 @@ static void launch_rr_k(frmg_ctx *ctx, LevelSet<float> &F, LevelSet<float> &C, c
   using RC = RRCfg<BG>;
   static_assert(RC::TX == kTX && RC::TY == kTY, "tile");
   const size_t sm = RC::smem;
-  static bool attr_set = false;
-  if (!attr_set) {
-    CK(cudaFuncSetAttribute(k_resid_restrict_tiled<BG, DIR>,
-                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    attr_set = true;
-  }
+  static PerDevice<bool> set;
+  allow_smem(set, k_resid_restrict_tiled<BG, DIR>, sm);
   k_resid_restrict_tiled<BG, DIR><<<F.nblk_rr, RC::NT, sm, st>>>(
       F.d, C.d, F.d_off_rr, F.size(), F.zc_rr, active, fpar, cpar, partial);
 }
@@ -1126,12 +1134,8 @@ static void launch_rc_k(LevelSet<float> &s, const int *active, int par, cudaStre
   using RC = RCCfg<TY, BG>;
   constexpr int v = BG ? 1 : 0;
   const size_t sm = RC::smem(PRL);
-  static bool attr_set = false;
-  if (!attr_set) {
-    CK(cudaFuncSetAttribute(k_smooth_rc<BG, DIR, TY, PRL>,
-                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    attr_set = true;
-  }
+  static PerDevice<bool> set;
+  allow_smem(set, k_smooth_rc<BG, DIR, TY, PRL>, sm);
   k_smooth_rc<BG, DIR, TY, PRL><<<s.nblk_rc[v], RC::NT, sm, st>>>(
       s.d, s.d_off_rc[v], s.size(), s.zc_rc[v], active, par, coarse, cpar);
 }
@@ -1171,12 +1175,8 @@ static void launch_rb_k(frmg_ctx *ctx, LevelSet<float> &s, const int *active, in
   constexpr int TY = kRbTY;
   using RC = RBCfg<TY>;
   size_t sm = RC::smem(BG);
-  static bool attr_set = false;
-  if (!attr_set) {
-    CK(cudaFuncSetAttribute(k_smooth_rb<BG, DIR, TY>,
-                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    attr_set = true;
-  }
+  static PerDevice<bool> set;
+  allow_smem(set, k_smooth_rb<BG, DIR, TY>, sm);
   constexpr int v = BG ? 1 : 0;
   k_smooth_rb<BG, DIR, TY><<<s.nblk_rb[v], RC::NT, sm, st>>>(s.d, s.d_off_rb[v], s.size(),
                                                               s.zc_rb[v], active, par);
@@ -1186,12 +1186,8 @@ template <bool BG, bool DIR>
 static void launch_fas_rhs_tiled(frmg_ctx *ctx, LevelSet<float> &s, const int *active, int par,
                                  cudaStream_t st) {
   const size_t sm = fas_rhs_tiled_smem(BG);
-  static bool attr_set = false;
-  if (!attr_set) {
-    CK(cudaFuncSetAttribute(k_fas_rhs_tiled<BG, DIR>,
-                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    attr_set = true;
-  }
+  static PerDevice<bool> set;
+  allow_smem(set, k_fas_rhs_tiled<BG, DIR>, sm);
   constexpr int v = BG ? 1 : 0;
   k_fas_rhs_tiled<BG, DIR><<<s.nblk_fr[v], 256, sm, st>>>(s.d, s.d_off_fr[v], s.size(),
                                                          s.zc_fr[v], active, par);
@@ -1199,49 +1195,49 @@ static void launch_fas_rhs_tiled(frmg_ctx *ctx, LevelSet<float> &s, const int *a
 
 template <bool BG, bool DIR>
 static long long rb_slots() {
-  static long long slots = 0;
-  if (!slots) {
+  static PerDevice<long long> slots;
+  return slots.get(current_device(), []() {
     using RC = RBCfg<kRbTY>;
-    slots = (long long)sm_count() *
-            resident_blocks(k_smooth_rb<BG, DIR, kRbTY>, RC::NT, RC::smem(BG));
-  }
-  return slots;
+    return (long long)sm_count() *
+           resident_blocks(k_smooth_rb<BG, DIR, kRbTY>, RC::NT, RC::smem(BG));
+  });
 }
 
 template <bool BG, bool DIR, int TY>
 static long long rc_slots() {
-  static long long slots = 0;
-  if (!slots)
-    slots = (long long)sm_count() *
-            resident_blocks(k_smooth_rc<BG, DIR, TY>, RCCfg<TY, BG>::NT, RCCfg<TY, BG>::smem());
-  return slots;
+  static PerDevice<long long> slots;
+  return slots.get(current_device(), []() {
+    using RC = RCCfg<TY, BG>;
+    return (long long)sm_count() *
+           resident_blocks(k_smooth_rc<BG, DIR, TY>, RC::NT, RC::smem());
+  });
 }
 
 template <bool BG, bool DIR>
 static long long fr_slots() {
-  static long long slots = 0;
-  if (!slots)
-    slots = (long long)sm_count() *
-            resident_blocks(k_fas_rhs_tiled<BG, DIR>, 256, fas_rhs_tiled_smem(BG));
-  return slots;
+  static PerDevice<long long> slots;
+  return slots.get(current_device(), []() {
+    return (long long)sm_count() *
+           resident_blocks(k_fas_rhs_tiled<BG, DIR>, 256, fas_rhs_tiled_smem(BG));
+  });
 }
 
 template <bool DIR>
 static long long pl_slots() {
-  static long long slots = 0;
-  if (!slots) slots = (long long)sm_count() * resident_blocks(k_prolong_tiled<DIR, false>, 256, 0);
-  return slots;
+  static PerDevice<long long> slots;
+  return slots.get(current_device(), []() {
+    return (long long)sm_count() * resident_blocks(k_prolong_tiled<DIR, false>, 256, 0);
+  });
 }
 
 template <bool DIR>
 static long long rr_slots() {
-  static long long slots = 0;
-  if (!slots) {
+  static PerDevice<long long> slots;
+  return slots.get(current_device(), []() {
     using RC = RRCfg<false>;
-    slots = (long long)sm_count() *
-            resident_blocks(k_resid_restrict_tiled<false, DIR>, RC::NT, RC::smem);
-  }
-  return slots;
+    return (long long)sm_count() *
+           resident_blocks(k_resid_restrict_tiled<false, DIR>, RC::NT, RC::smem);
+  });
 }
 
 template <bool BG, int S>
@@ -1373,12 +1369,7 @@ template <typename T, bool BG, bool DIR>
 static void launch_tail_k(frmg_ctx *ctx, TailSet<T> &t, int skip, int pin, int pout, bool fas,
                         bool finest, const CycleOpts &o, const int *active, cudaStream_t st) {
   auto *k = k_tail<T, BG, DIR>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    CK(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem));
-    attr_set = true;
-  }
+  tail_cluster<T, BG, DIR>(kTailSmem);  // the kernel's attributes on this device
   cudaLaunchConfig_t c = {};
   c.gridDim = dim3((unsigned)(t.size() * t.cs));
   c.blockDim = dim3(tail_threads<T>());
