@@ -14,9 +14,15 @@
 
 namespace frmg {
 
+// v is normal and at least 2^20 away from the ends of the exponent's range (an
+// integer test of the high word: zeros, infinities and NaN fail it too).
+__device__ __forceinline__ bool f64_tame(double v) {
+  return ((__double2hiint(v) >> 20) & 0x7ff) - 21u < 2005u;
+}
+
 // 1/v: the hardware's approximation (about 20 bits) and one step of the
 // third-order iteration r (1 + e + e^2), e = 1 - v r (the geometric series cut
-// after e^2; its remainder e^3 is below 2^-57).  |v| in the normal range.
+// after e^2; its remainder e^3 is below 2^-57).  v tame.
 __device__ __forceinline__ double f64_rcp(double v) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
@@ -26,7 +32,7 @@ __device__ __forceinline__ double f64_rcp(double v) {
 
 // 1/sqrt(v): the hardware's approximation and one step of Halley's third-order
 // iteration, r (1 + e/2 + 3 e^2/8), e = 1 - v r^2 (the binomial series of
-// (1 - e)^(-1/2)).  v > 0 in the normal range.
+// (1 - e)^(-1/2)).  v > 0 and tame.
 __device__ __forceinline__ double f64_rsqrt(double v) {
   double r;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));

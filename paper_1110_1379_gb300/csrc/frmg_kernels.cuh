@@ -324,20 +324,31 @@ struct OpAcc<float, true> {
   }
 };
 
+// 1 / sqrt(B) and e^{-d/2} - 1 = -x / (B + sqrt B), B = 1 + x, for any B
+// (0, infinite and NaN ones too).
+__device__ __noinline__ double2 mass_wide(double xi) {
+  const double B1 = 1.0 + xi, s = sqrt(B1);
+  return make_double2(1.0 / s, -xi / (B1 + s));
+}
+
 // Mass term and final assembly:  N = (alpha/2) acc + beta F (e^{-d/2} - 1),
 // dN = (alpha/2) dacc - (beta/2) F e^{-d/2},  F = e^{-ub/2}.
-// FP32 uses the SFU reciprocal square root
-// and reciprocal (the same expression in every FP32 kernel, so all of them
-// see one and the same discrete operator).
+// FP32 uses the SFU reciprocal square root and reciprocal (the same expression
+// in every FP32 kernel, so all of them see one and the same discrete operator).
 __device__ __forceinline__ void finish_op(double xi, double Ei, double acc, double dacc,
                                           double ah, double beta, bool bg, double &N,
                                           double &dN) {
   const double B1 = 1.0 + xi;
-  const double rs = f64_rsqrt(B1);
-  const double y = -xi * f64_rcp(fma(B1, rs, B1));  // -x / (B + sqrt B)
   const double bF = bg ? beta * rsqrt(Ei) : beta;
-  N = fma(ah, acc, bF * y);
-  dN = fma(ah, dacc, -0.5 * bF * rs);
+  double2 m;
+  if (f64_tame(B1)) {
+    m.x = f64_rsqrt(B1);
+    m.y = -xi * f64_rcp(fma(B1, m.x, B1));
+  } else {
+    m = mass_wide(xi);
+  }
+  N = fma(ah, acc, bF * m.y);
+  dN = fma(ah, dacc, -0.5 * bF * m.x);
 }
 
 // SFU reciprocal and reciprocal square root (PTX rcp.approx / rsqrt.approx,
@@ -372,6 +383,17 @@ __device__ __forceinline__ float newton_du(float N, float f, float dN, float w) 
   return __fmul_rn(w, newton_step(__fsub_rn(N, f), dN));
 }
 
+// The FP64 Newton step with the library's division and root: where the
+// products below leave the range of FP64 (u above about 350, B = 0, non-finite
+// values).
+__device__ __noinline__ double newton_wide(double xi, double acc, double dacc, double f, double ah,
+                                           double beta, double relax) {
+  const double B1 = 1.0 + xi, s = sqrt(B1);
+  const double N = ah * acc + beta * (-xi / (B1 + s));
+  const double dN = ah * dacc - 0.5 * beta / s;
+  return relax * (-(N - f) / dN);
+}
+
 // The clamped, relaxed Newton step of a cell from its face sums.  FP64, plain
 // form: with q = B + sqrt(B) both N - f and dN are multiplied by q, so that one
 // reciprocal serves the mass term and the step.
@@ -382,7 +404,13 @@ __device__ __forceinline__ T newton_from_sums(T xi, T Ei, T acc, T dacc, T f, T 
     const T B1 = T(1) + xi, rs = f64_rsqrt(B1), q = fma(B1, rs, B1);
     const T num = fma(-beta, xi, fma(ah, acc, -f) * q);
     const T den = fma(ah, dacc, T(-0.5) * beta * rs) * q;
-    const T du = -relax * num * f64_rcp(den);
+    T du;
+    // (num below 2^1004, so that relax num is finite; a NaN of num or of rs at
+    // B = 0 fails the tests too)
+    if (f64_tame(den) && ((__double2hiint(num) >> 20) & 0x7ff) < 2027)
+      du = -relax * num * f64_rcp(den);
+    else
+      du = newton_wide(xi, acc, dacc, f, ah, beta, relax);
     // the comparison by the high words first (an FP64 comparison takes the FP64 pipe)
     if ((__double2hiint(du) & 0x7fffffff) < __double2hiint(cap)) return du;
     return du > cap ? cap : (du < -cap ? -cap : du);

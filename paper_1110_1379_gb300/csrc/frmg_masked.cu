@@ -207,7 +207,7 @@ __device__ __forceinline__ void m_cell(const MLevelT<T, BG> &L, long long c, T &
   dacc += bi * (S1 - T(__popc(nb)));
   T s, sm1;
   if constexpr (sizeof(T) == 8) {
-    s = f64_rsqrt(bi);  // e^{-u/2}
+    s = f64_tame(bi) ? f64_rsqrt(bi) : exp(-0.5 * ui);  // e^{-u/2}
     sm1 = s - 1.0;
   } else {
     sm1 = expm1f(-0.5f * ui);
@@ -298,7 +298,7 @@ __device__ __forceinline__ void m_update(const MLevelT<T, BG> &L, long long c, T
   m_cell(L, c, N, dN);
   T du;
   if constexpr (sizeof(T) == 8)
-    du = -relax * (N - L.f[c]) * f64_rcp(dN);
+    du = f64_tame(dN) ? -relax * (N - L.f[c]) * f64_rcp(dN) : -relax * (N - L.f[c]) / dN;
   else
     du = -relax * (N - L.f[c]) / dN;
   du = du > cap ? cap : (du < -cap ? -cap : du);
