@@ -22,7 +22,7 @@ __device__ __forceinline__ bool f64_tame(double v) {
 
 // 1/v: the hardware's approximation (about 20 bits) and one step of the
 // third-order iteration r (1 + e + e^2), e = 1 - v r (the geometric series cut
-// after e^2; its remainder e^3 is below 2^-57).  v tame.
+// after e^2; its remainder e^3 is below 2^-57): error below 0.55 ulp.  v tame.
 __device__ __forceinline__ double f64_rcp(double v) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
@@ -32,7 +32,8 @@ __device__ __forceinline__ double f64_rcp(double v) {
 
 // 1/sqrt(v): the hardware's approximation and one step of Halley's third-order
 // iteration, r (1 + e/2 + 3 e^2/8), e = 1 - v r^2 (the binomial series of
-// (1 - e)^(-1/2)).  v > 0 and tame.
+// (1 - e)^(-1/2)): error below 1.05 ulp (half an ulp from v r, half from the last
+// step).  v > 0 and tame.
 __device__ __forceinline__ double f64_rsqrt(double v) {
   double r;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
@@ -77,8 +78,10 @@ __device__ __forceinline__ void f64_exp_parts(double u, double &t, double &p) {
 }
 
 // e^u - 1 = (t - 1) + t p, the first bracket exact; for |u| < ln2/32 the series
-// itself.  Error at most 2 ulp (near |u| = 0.022; 0.8 ulp beyond 0.4), below
-// 0.07 ulp of e^u where it is largest; 14 FP64 instructions.
+// itself.  Largest errors found (2e7 arguments per range): 0.85 ulp for |u| <
+// ln2/32, 2.24 ulp from there to 0.035 (r, r + dt and p, each as large as the
+// result, are rounded), 1.24 ulp to 0.1, 1.03 ulp beyond; below 0.3 ulp of e^u for
+// |u| < 0.4.  14 FP64 instructions.
 __device__ __forceinline__ double f64_expm1(double u) {
   if (!(fabs(u) < 700.0)) return expm1(u);  // overflow, -1, NaN
   double t, p;
@@ -86,7 +89,7 @@ __device__ __forceinline__ double f64_expm1(double u) {
   return fma(t, p, t - 1.0);
 }
 
-// e^u, error below 1 ulp.
+// e^u, error below 0.55 ulp.
 __device__ __forceinline__ double f64_exp(double u) {
   if (!(fabs(u) < 700.0)) return exp(u);
   double t, p;
