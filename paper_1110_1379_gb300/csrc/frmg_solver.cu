@@ -3298,24 +3298,37 @@ int fr_solve_levels(frmg_ctx *ctx, const double *density, const int dims[3], dou
     for (int lv = 1; lv <= maxlev; lv++) {
       std::vector<Problem> P;
       std::vector<int> ids;
-      // the checks of all patches of the level are read back together: per
-      // patch the density's and the interpolation stencil's flag
-      int *bad = S.get<int>(2 * (size_t)npatch);
-      CK(cudaMemsetAsync(bad, 0, 2 * (size_t)npatch * sizeof(int), st));
+      // the densities of the level's patches are checked, with one read-back,
+      // before any patch's u is written
+      std::vector<const double *> prho(npatch, nullptr);
+      int *bad = S.get<int>((size_t)npatch + 1);
+      CK(cudaMemsetAsync(bad, 0, ((size_t)npatch + 1) * sizeof(int), st));
       for (int i = 0; i < npatch; i++) {
         if (level[i] != lv) continue;
-        fr_patch &pp = patches[i];
-        long long pn = (long long)pp.n[0] * pp.n[1] * pp.n[2];
-        const double *prho = stage(S, back, pp.density, pn, true, false, st);
-        pu[i] = stage(S, back, pp.u, pn, false, true, st);
-        k_check_density<<<nblocks(pn), 256, 0, st>>>(prho, pn, o.allow_negative_density,
-                                                     bad + 2 * i);
+        const fr_patch &pp = patches[i];
+        const long long pn = (long long)pp.n[0] * pp.n[1] * pp.n[2];
+        prho[i] = stage(S, back, pp.density, pn, true, false, st);
+        k_check_density<<<nblocks(pn), 256, 0, st>>>(prho[i], pn, o.allow_negative_density,
+                                                     bad + i);
         CK_LAUNCH(ctx);
+        ids.push_back(i);
+      }
+      std::vector<int> hb(npatch);
+      CK(cudaMemcpyAsync(hb.data(), bad, hb.size() * sizeof(int), cudaMemcpyDeviceToHost, st));
+      CK(cudaStreamSynchronize(st));
+      for (int i : ids)
+        if (hb[i]) einval(kBadDensity);
+      for (int i : ids) {
+        fr_patch &pp = patches[i];
+        const long long pn = (long long)pp.n[0] * pp.n[1] * pp.n[2];
+        pu[i] = stage(S, back, pp.u, pn, false, true, st);
         double *ub = S.get<double>(face_total(pp.n));
         const double *up = pp.parent < 0 ? du : pu[pp.parent];
         const int *pdim = pp.parent < 0 ? dims : pdims[pp.parent].data();
         double hpar = pp.parent < 0 ? 1.0 / dims[0] : ph[pp.parent];
-        patch_bc_launch(ctx, up, pdim, pp.parent < 0, pp.origin, pp.n, pu[i], ub, bad + 2 * i + 1,
+        // (the nesting checked above keeps the stencil inside the parent: the
+        // flag bad[npatch] stays 0)
+        patch_bc_launch(ctx, up, pdim, pp.parent < 0, pp.origin, pp.n, pu[i], ub, bad + npatch,
                         st);
         ph[i] = 0.5 * hpar;
         Problem p;
@@ -3326,18 +3339,10 @@ int fr_solve_levels(frmg_ctx *ctx, const double *density, const int dims[3], dou
         p.a = a;
         p.om = om;
         p.fr0 = fr0;
-        p.rho = prho;
+        p.rho = prho[i];
         p.u = pu[i];
         p.bnd = ub;
         P.push_back(p);
-        ids.push_back(i);
-      }
-      std::vector<int> hb(2 * (size_t)npatch);
-      CK(cudaMemcpyAsync(hb.data(), bad, hb.size() * sizeof(int), cudaMemcpyDeviceToHost, st));
-      CK(cudaStreamSynchronize(st));
-      for (int i : ids) {
-        if (hb[2 * i]) einval(kBadDensity);
-        if (hb[2 * i + 1]) einval(kBadStencil);
       }
       std::vector<fr_stats> sv(P.size());
       memset(sv.data(), 0, sv.size() * sizeof(fr_stats));
