@@ -454,12 +454,17 @@ __global__ void __launch_bounds__(m_threads<T>()) k_mprolong(MLevelT<T, BG> F, M
 //
 // Coarsest level: red-black sweeps until the rms over the active cells falls
 // to max(1e-3 of its value before the first sweep, 0.1 tol), at most 500
-// sweeps.  In FP32 the solve also ends when four sweeps in a row have not
-// brought the rms 1 % below its best: near the FP32 floor of the
-// full-variable form the first rule is never met (500 sweeps, 2.2 ms per
-// cycle).
+// sweeps.  In FP32 the solve also ends at the floor of its arithmetic, which in
+// the full-variable form lies above the first rule's value (500 sweeps, 2.2 ms
+// per cycle, were spent there): when four sweeps in a row have not brought the
+// rms 1 % below its best and it is within kFloor of the residual that
+// neighbouring FP32 values of u differ by, 2^-24 rms(u dN/du).  Emulated in FP32
+// (regions of 14 and 28 cells across, weak and strong diffusion) the rms stalls
+// at 0.37 to 0.50 of that; a large region whose slow mode falls by less than
+// 0.25 % a sweep is far above it and goes on.
 constexpr int kTailNT = 1024;
 constexpr int kTailLevels = 16;
+constexpr float kFloor = 1.0f;
 
 // FP32: up to 4096 active cells (masked 256^3 region, whole solve: 512 cells 7.33
 // ms, 4096 7.06 ms, 12000 8.57 ms), FP64: 256 (the FP64 pipe of one SM).
@@ -493,41 +498,47 @@ __device__ __noinline__ void mt_resid(const MLevelT<T, BG> &L, bool fas) {
   __syncthreads();
 }
 
+// rms over the active cells of the residual d = L(u) - f, or (scale) of u dN/du
+template <typename T, bool BG>
+__device__ __noinline__ T mt_rms(const MLevelT<T, BG> &L, bool scale) {
+  // in the level's precision (FP64 arithmetic runs at 1/64 rate)
+  __shared__ T red[kTailNT / 32];
+  T s = T(0);
+  for (long long t = threadIdx.x; t < L.na; t += kTailNT) {
+    const long long c = L.act[t];
+    T N, dN;
+    m_cell(L, c, N, dN);
+    const T d = scale ? L.u[c] * dN : N - L.f[c];
+    s += d * d;
+  }
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  s = red[threadIdx.x & 31];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  __syncthreads();  // red has been read
+  return sqrt(s / (T)(L.na > 0 ? L.na : 1));
+}
+
 template <typename T, bool BG>
 __device__ __noinline__ void mt_coarsest(const MLevelT<T, BG> &L, double tol, T cap, T relax) {
-  // the rms in the level's precision (FP64 arithmetic runs at 1/64 rate)
-  __shared__ T red[kTailNT / 32];
-  T thr = T(0), best = T(0);
+  T r = mt_rms(L, false), best = r;
+  const T thr = fmax(T(1e-3) * r, (T)(0.1 * tol));
   int flat = 0;
-  for (int it = -1; it < 500; it++) {
-    if (it >= 0) mt_smooth(L, 1, cap, relax);
-    T s = T(0);
-    for (long long t = threadIdx.x; t < L.na; t += kTailNT) {
-      const long long c = L.act[t];
-      T N, dN;
-      m_cell(L, c, N, dN);
-      const T d = N - L.f[c];
-      s += d * d;
-    }
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    s = red[threadIdx.x & 31];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    const T r = sqrt(s / (T)(L.na > 0 ? L.na : 1));
-    __syncthreads();  // red has been read
-    if (it < 0) {
-      thr = fmax(T(1e-3) * r, (T)(0.1 * tol));
-      best = r;
-      continue;
-    }
+  for (int it = 0; it < 500; it++) {
+    mt_smooth(L, 1, cap, relax);
+    r = mt_rms(L, false);
     if (r < T(0.99) * best) {
       best = r;
       flat = 0;
     } else {
       flat++;
     }
-    if (r <= thr || (sizeof(T) == 4 && flat >= 4)) return;
+    if (r <= thr) return;
+    if (sizeof(T) == 4 && flat >= 4) {
+      if (!(r > T(kFloor) * T(0x1p-24) * mt_rms(L, true))) return;  // (or NaN)
+      flat = 0;
+    }
   }
 }
 
