@@ -1123,36 +1123,39 @@ struct PFine {
   float ih2h, ih2l;    // 1/h^2 as a double-float pair
 };
 
-// Sum of double-float values across a warp, on every lane.
-__device__ __forceinline__ df warp_df_sum(df v) {
-  for (int o = 16; o > 0; o >>= 1) {
-    df w = {__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)};
-    v = df_add(v, w);
-  }
-  return v;
+// Sum of v over NV values of a block's shared array, one per lane of its first
+// warp, in FP64; on lane 0.
+template <int NV>
+__device__ __forceinline__ double warp_sum64(const double *v) {
+  const int lane = threadIdx.x & 31;
+  double s = lane < NV ? v[lane] : 0.0;
+  for (int o = NV / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
 }
 
-// Block (sum, max) of a double-float per-thread value: partial[2 b] = sum
-// (as FP64), partial[2 b + 1] = max |value| (the max is taken on the high
-// parts).  No FP64 arithmetic: the warp sums are added as pairs too.
+// Block (sum, max) of a double-float per-thread value (of four cells): partial[2
+// b] = sum (as FP64), partial[2 b + 1] = max |value| (the max is taken on the
+// high parts).  Eight threads' values are added as pairs, the 32 sums of such
+// groups in FP64 (five FP64 warp instructions per 1024 cells).
 __device__ __forceinline__ void block_df_partial(df v, float amax, double *partial) {
-  __shared__ float2 ws[kNT / 32];
+  __shared__ double ws[kNT / 8];
   __shared__ float wm[kNT / 32];
-  v = warp_df_sum(v);
+  static_assert(kNT / 8 == 32, "one group per lane");
+  for (int o = 4; o > 0; o >>= 1) {
+    const df w = {__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)};
+    v = df_add(v, w);
+  }
   for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
   const int lane = threadIdx.x & 31;
-  if (lane == 0) {
-    ws[threadIdx.x >> 5] = make_float2(v.h, v.l);
-    wm[threadIdx.x >> 5] = amax;
-  }
+  if ((lane & 7) == 0) ws[threadIdx.x >> 3] = join_bits(v.h, v.l);
+  if (lane == 0) wm[threadIdx.x >> 5] = amax;
   __syncthreads();
   if (threadIdx.x < 32) {
-    const float2 w = lane < kNT / 32 ? ws[lane] : make_float2(0.f, 0.f);
-    v = warp_df_sum(df{w.x, w.y});
+    const double s = warp_sum64<32>(ws);
     amax = lane < kNT / 32 ? wm[lane] : 0.0f;
-    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+    for (int o = 4; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
     if (lane == 0) {
-      partial[2 * blockIdx.x] = join_bits(v.h, v.l);
+      partial[2 * blockIdx.x] = s;
       partial[2 * blockIdx.x + 1] = (double)amax;
     }
   }
@@ -1282,24 +1285,23 @@ __global__ void __launch_bounds__(kNT)
     ss = fmaf(dv.y, dv.y, dv.x * dv.x);
     mx = fmaxf(fabsf(dv.x), fabsf(dv.y));
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    ss += __shfl_down_sync(0xffffffffu, ss, o);
-    mx = fmaxf(mx, __shfl_down_sync(0xffffffffu, mx, o));
-  }
-  __shared__ float a[kNT / 32], b[kNT / 32];
-  if ((threadIdx.x & 31) == 0) {
-    a[threadIdx.x >> 5] = ss;
-    b[threadIdx.x >> 5] = mx;
-  }
+  // sixteen threads' squares are added in FP32, the block's 16 sums in FP64
+  for (int o = 8; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  __shared__ double a[kNT / 16];
+  __shared__ float b[kNT / 32];
+  const int lane = threadIdx.x & 31;
+  if ((lane & 15) == 0) a[threadIdx.x >> 4] = (double)ss;
+  if (lane == 0) b[threadIdx.x >> 5] = mx;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    float s2 = 0.0f, m2 = 0.0f;
-    for (int w = 0; w < kNT / 32; w++) {
-      s2 += a[w];
-      m2 = fmaxf(m2, b[w]);
+  if (threadIdx.x < 32) {
+    const double s2 = warp_sum64<kNT / 16>(a);
+    mx = lane < kNT / 32 ? b[lane] : 0.0f;
+    for (int o = 4; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) {
+      partial[2 * blockIdx.x] = s2;
+      partial[2 * blockIdx.x + 1] = (double)mx;
     }
-    partial[2 * blockIdx.x] = (double)s2;
-    partial[2 * blockIdx.x + 1] = (double)m2;
   }
 }
 
