@@ -1218,8 +1218,9 @@ __global__ void __launch_bounds__(kNT)
 
 // Fine defect d = L(phi) - (s - smean) in double-float; the FP32 correction
 // problem gets f = -d and e = 0.  Per-block partials of (d^2, max |d|).  One
-// x-pair per thread.  The sum of the neighbours carries its rounding errors and
-// the low parts in one FP32 sum (TwoSum per neighbour) and is normalised once.
+// x-pair per thread.  The neighbours are added pair by pair, each sum
+// normalised: with the low parts left to one FP32 sum the defect's rounding
+// error was 1.35 times as large (rms 4.8 against 3.5 units of 2^-48 |phi| / h^2).
 __global__ void __launch_bounds__(kNT)
     k_pdefect(PFine P, float smh, float sml, float *f32, float *e32, double *partial) {
   const long long t = (long long)blockIdx.x * kNT + threadIdx.x;
@@ -1252,12 +1253,9 @@ __global__ void __launch_bounds__(kNT)
       nb.y -= 1.0f;
     }
     // cell 0: xl + cell 1; cell 1: cell 0 + xr
-    df2 a = two_sum2(make_float2(xl.x, pi.h.x), make_float2(pi.h.y, xr.x));
-    float2 lo = add2(a.l, add2(make_float2(xl.y, pi.l.x), make_float2(pi.l.y, xr.y)));
-    auto add = [&](const df2 &v) {
-      a = two_sum2(a.h, v.h);
-      lo = add2(lo, add2(a.l, v.l));
-    };
+    df2 acc = df_add2(df2{make_float2(xl.x, pi.h.x), make_float2(xl.y, pi.l.x)},
+                      df2{make_float2(pi.h.y, xr.x), make_float2(pi.l.y, xr.y)});
+    auto add = [&](const df2 &v) { acc = df_add2(acc, v); };
     auto pair_face = [&](bool inside, long long in, long long wrap, int f, long long o) {
       if (inside || !pat) {
         add(ld_df2(P.phi, (inside ? in : wrap) >> 1));
@@ -1275,8 +1273,7 @@ __global__ void __launch_bounds__(kNT)
     // diagonal: -(6 + missing) phi_i = -(12 - nb) phi_i
     const float2 dg = sub2(nb, splat2(12.0f));
     const df2 m = two_prod2(pi.h, dg);
-    add(df2{m.h, fma2(pi.l, dg, m.l)});
-    const df2 acc = fast_two_sum2(a.h, lo);
+    add(fast_two_sum2(m.h, fma2(pi.l, dg, m.l)));
     df2 d = df_mul2(acc, df2{splat2(P.ih2h), splat2(P.ih2l)});
     d = df_sub2(d, df_sub2(ld_df2(P.s, t), df2{splat2(smh), splat2(sml)}));
     const float2 dv = add2(d.h, d.l);
