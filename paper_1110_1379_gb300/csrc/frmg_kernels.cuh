@@ -2538,10 +2538,6 @@ __global__ void __launch_bounds__(256)
 // ---------------------------------------------------------------------------
 // Asynchronous global-to-shared copy of 8 bytes (PTX cp.async; both
 // addresses 8-byte aligned); commit_group / wait_group track completion.
-__device__ __forceinline__ void cp_async8(void *smem, const void *gmem) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sa), "l"(gmem) : "memory");
-}
 __device__ __forceinline__ void cp_async4(void *smem, const void *gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sa), "l"(gmem) : "memory");
@@ -2574,7 +2570,8 @@ __device__ __forceinline__ void cp_async_wait() {
 // 512^3: 0.379 ms plain, 0.715 ms in the correction form (3 and 5 arrays read,
 // 0.28 and 0.44 ms of memory time); with every neighbour of a cell read from
 // shared memory, which left one or two blocks per SM, 0.477 and 0.824 ms.
-// Bound by instruction issue (packed FP32, shuffles) at 16 and 24 warps per SM.
+// Bound by instruction issue (packed FP32, shuffles) at 24 warps per SM in the
+// plain form, 16 in the correction form.
 template <bool BG>
 struct RRCfg {
   static constexpr int TX = 64, TY = 16, NT = 256, NW = NT / 32;
@@ -2623,19 +2620,19 @@ __global__ void __launch_bounds__(RRCfg<BG>::NT, RRCfg<BG>::MINB)
     const int gx = X0 + 2 * lane, gy = Y0 + 2 * w;
     const bool valid = gx < n0 && gy < n1;
     const long long fplane = (long long)n0 * n1;
-    // What a lane copies of a plane (offsets, -1: none).  Rows of whole quads:
-    // 16 bytes of row 2 w (lanes 0 - 15) or 2 w + 1, and of the row beyond the
-    // tile (first and last warp); else pairs of both rows.  The first and last
-    // lane also copy the cells left and right of the tile.
+    // What a lane copies of a plane (offsets, -1: none): 16 bytes of row 2 w
+    // (lanes 0 - 15) or 2 w + 1, and of the row beyond the tile (first and last
+    // warp).  The first and last lane also copy the cells left and right of the
+    // tile.  (Rows are whole quads: a level that has a coarser one has n0 a
+    // multiple of 4, see count_levels.)
     auto at = [&](int x, int y) -> int {
       if (DIR) return x >= 0 && x < n0 && y >= 0 && y < n1 ? y * n0 + x : -1;
       return wrapmod(y, n1) * n0 + wrapmod(x, n0);
     };
-    const bool quad = !(n0 & 3);
-    const int lx = quad ? 4 * (lane & 15) : 2 * lane, ly = quad ? lane >> 4 : 0;
+    const int lx = 4 * (lane & 15), ly = lane >> 4;
     const int o0 = at(X0 + lx, gy + ly);
-    const int oh = w == 0 && !(quad && ly) ? at(X0 + lx, gy - 1)
-                   : (w == C::NW - 1 && !(quad && ly) ? at(X0 + lx, gy + 2) : -1);
+    const int oh = w == 0 && !ly ? at(X0 + lx, gy - 1)
+                                 : (w == C::NW - 1 && !ly ? at(X0 + lx, gy + 2) : -1);
     const int ex = lane == 0 ? X0 - 1 : X0 + TX;
     const bool edge = lane == 0 || lane == 31;
     const int oe = edge ? at(ex, gy) : -1;  // (and the row above: n1 is even)
@@ -2664,30 +2661,15 @@ __global__ void __launch_bounds__(RRCfg<BG>::NT, RRCfg<BG>::MINB)
         for (int a = 0; a < NA; a++) {
           const float *v = in[a] + zo;
           float *ha = h + a * C::AN;
-          if (quad) {
-            if (o0 >= 0) cp_async16(ha + qc, v + o0);
-            if (own && oh >= 0) cp_async16(ha + qh, v + oh);
-          } else {
-            if (o0 >= 0) {
-              cp_async8(ha + qc, v + o0);
-              cp_async8(ha + qc + TX, v + o0 + n0);
-            }
-            if (own && oh >= 0) cp_async8(ha + qh, v + oh);
-          }
+          if (o0 >= 0) cp_async16(ha + qc, v + o0);
+          if (own && oh >= 0) cp_async16(ha + qh, v + oh);
           if (own && oe >= 0) {
             cp_async4(ha + qe, v + oe);
             cp_async4(ha + qe + 1, v + oe + n0);
           }
         }
-        if (fin && own && o0 >= 0) {
-          float *hf = h + NA * C::AN + qc - TX;
-          if (quad) {
-            cp_async16(hf, fin + zo + o0);
-          } else {
-            cp_async8(hf, fin + zo + o0);
-            cp_async8(hf + TX, fin + zo + o0 + n0);
-          }
-        }
+        if (fin && own && o0 >= 0)
+          cp_async16(h + NA * C::AN + qc - TX, fin + zo + o0);
       }
       cp_async_commit();
     };
