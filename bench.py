@@ -58,7 +58,9 @@ ALG_BYTES = {
     # bytes plus the coarse correction (u^H, R u^h: 8 B per 8 fine cells)
     "smooth_prolong_f32@fine": 13.0,
     "smooth_prolong_bg_f32@fine": 21.0,
-    "resid_restrict_f32@fine": 10.0,  # read u, rhs (8 B) + 4 coarse words / 8 cells
+    # read u, rhs (8 B) + 4 coarse words / 8 cells: the plain form, also where the
+    # family's launches include the correction form's (18 B)
+    "resid_restrict_f32@fine": 10.0,
     "resid_restrict_f64@fine": 20.0,
     "prolong_f32@fine": 9.0,         # read/write u (8 B) + 2 coarse words / 8 cells
     "prolong_f64@fine": 18.0,
@@ -71,21 +73,21 @@ ALG_BYTES = {
 # DRAM bytes per cell of one launch (dram__bytes_read.sum + dram__bytes_write.sum
 # over the cells of the launch) from one ncu capture of each kernel on a 384^3
 # fine grid of the same workload recipe (traffic grows in proportion to the
-# cells, so it is scaled to the workload's grid).  Valid for the kernels as
-# captured; the second entry names the captured launch.
+# cells, so it is scaled to the workload's grid).  The second entry names the
+# captured launch (profiles/ has its counters).  Not here: the residual +
+# restriction, whose family's time averages launches of the plain form (14.2 B per
+# cell) and of the correction form (22.4 B).
 TRAFFIC_PER_CELL = {
-    "smooth_f32@fine": ((702.4e6 + 418.0e6) / 384 ** 3,
+    "smooth_f32@fine": ((705.5e6 + 419.8e6) / 384 ** 3,
                         "k_smooth_rc plain form, 64x16 tiles, one 384^3 launch"),
-    "smooth_prolong_f32@fine": ((536.8e6 + 412.4e6) / 384 ** 3,
+    "smooth_prolong_f32@fine": ((543.4e6 + 413.6e6) / 384 ** 3,
                                 "k_smooth_rc plain form with the prolongation fused, 64x16 "
                                 "tiles, one 384^3 launch"),
-    "smooth_bg_f32@fine": ((1176.2e6 + 430.6e6) / 384 ** 3,
+    "smooth_bg_f32@fine": ((1171.3e6 + 431.0e6) / 384 ** 3,
                            "k_smooth_rc correction form, 64x8 tiles, one 384^3 launch"),
-    "resid_restrict_f32@fine": ((715.0e6 + 102.6e6) / 384 ** 3,
-                                "k_resid_restrict_tiled plain form, one 384^3 launch"),
-    "prolong_f32@fine": ((286.715e6 + 392.129e6) / 384 ** 3,
+    "prolong_f32@fine": ((286.8e6 + 392.5e6) / 384 ** 3,
                          "k_prolong_tiled, one 384^3 launch (the fine level)"),
-    "df_defect": ((1363.777e6 + 1101.749e6) / 384 ** 3,
+    "df_defect": ((1363.9e6 + 1103.2e6) / 384 ** 3,
                   "k_df_defect, two cells per thread, one 384^3 launch"),
 }
 

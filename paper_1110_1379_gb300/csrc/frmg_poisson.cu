@@ -1164,8 +1164,8 @@ __device__ __forceinline__ void block_df_partial(df v, float amax, double *parti
 // The double-float passes over the fine grid work on x-pairs (every n0 is
 // even), the pair arithmetic on packed FP32 pairs; the sums take kPP pairs per
 // thread, 256 apart, so that their block reduction (about 150 instructions) is
-// shared by 2 kPP cells.  At 512^3: source 3.20 -> 1.98 ms, sum of phi 0.80 ->
-// 0.18 ms, defect 1.47 -> 1.13 ms (one cell per thread before).
+// shared by 2 kPP cells.  At 512^3: source 3.20 -> 2.04 ms, sum of phi 0.80 ->
+// 0.20 ms, defect 1.47 -> 1.18 ms (one cell per thread before).
 constexpr int kPP = 2;
 
 __device__ __forceinline__ df2 ld_df2(const float2 *p, long long pair) {
