@@ -706,10 +706,9 @@ __device__ __noinline__ void tail_coarsest_warp(TailBlock<T> &B, int l, const Ta
 //
 // Bound: latency of the dependent steps (at 2 GHz, plain form, 32^3 on 16
 // blocks: 4600 cycles a colour at 32^3, 1850 at 16^3, 950 at 8^3; 15,000 for
-// the coarsest solve at 4^3): warps wait at barriers three times as long as
-// for everything else.  The 32^3 tail takes 53 to 56 us (plain) and 67 us
-// (correction form) with V(2,2), 40 to 43 and 52 to 60 us with V(1,1); its 35
-// launches took 240 us.  16 blocks per cluster are
+// the coarsest solve at 4^3); barriers take 58 % of a warp's time.  The 32^3 tail
+// takes 53 to 56 us (plain) and 67 us (correction form) with V(2,2), 40 to 43 and
+// 52 to 60 us with V(1,1); its 35 launches took 240 us.  16 blocks per cluster are
 // the fastest for up to 8 grids (8 blocks: 64 and 85 us); with more grids
 // clusters of 8 let more of them run at once (28 patches of 32 to 64 cells:
 // 120 against 133 us).
